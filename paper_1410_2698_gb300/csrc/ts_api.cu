@@ -1,6 +1,7 @@
 // ts_api.cu -- the extern "C" boundary declared in include/ts.h.
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -210,6 +211,19 @@ ts_status ts_index_export(const ts_index *h, int32_t field, int32_t dim, void *d
         return TS_ERR_CAPACITY;
     }
     TS_CUDA(cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost));
+    if (field == TS_FIELD_ST_IDS) {
+        // the array is swept in (subbin, bin, Morton) order; bins follow the start-time order,
+        // so sorting a subbin's ids gives its ranges in start-time order
+        return guarded([&]() -> ts_status {
+            const uint64_t cells = (uint64_t)ix->v[dim] * ix->m;
+            std::vector<uint32_t> off(cells + 1);
+            TS_CUDA(cudaMemcpy(off.data(), ix->st_off[dim], 4 * (cells + 1),
+                               cudaMemcpyDeviceToHost));
+            uint32_t *ids = static_cast<uint32_t *>(dst);
+            for (uint64_t j = 0; j < cells; j += ix->m) std::sort(ids + off[j], ids + off[j + ix->m]);
+            return clear_error(TS_OK);
+        });
+    }
     return clear_error(TS_OK);
 }
 

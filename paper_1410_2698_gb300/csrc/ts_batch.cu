@@ -43,6 +43,7 @@ __global__ void k_run_start(const ReqDesc *h_reqs, const uint32_t *h_run, ReqDes
         b.status[0] = 0;
         b.counters[0] = 0;
         b.counters[1] = 0;
+        b.counters[2] = 0;
     }
 }
 
@@ -109,7 +110,7 @@ static void layout(BatchPlan *p, Carver &c)
     b.g_count = c.take<uint32_t>(k.groups);
     b.g_nseg = c.take<uint32_t>(k.groups);
     b.gmem = c.take<MemberRec>(GROUP * k.groups);
-    b.ghdr = c.take<float4>(k.groups);
+    b.ghdr = c.take<float4>(3 * k.groups);
     b.seg_lo = c.take<uint32_t>(GROUP * k.groups);
     b.seg_hi = c.take<uint32_t>(GROUP * k.groups);
     b.seg_sel = c.take<uint32_t>(GROUP * k.groups);

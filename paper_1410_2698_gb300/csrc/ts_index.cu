@@ -136,18 +136,19 @@ __global__ void k_gather(SegIn in, uint64_t n, const uint32_t *perm, SegD *seg, 
     orig[s] = i;
 }
 
-// Key of an entry inside its bin: (bin, x of its FP32 box centre as an order-preserving integer).
-// Any order inside a bin leaves every bin's range unchanged; x order makes aligned chunks of 64
-// entries narrow in x, so a chunk's bounding record rejects most queries.
-__global__ void k_tx_key(const RecF *rec, const uint32_t *bin_of, uint64_t n, uint64_t *keys,
-                         uint32_t *vals)
+// Key of an entry inside its bin: (bin, Morton code of its FP32 box centre, `bits` per axis). Any
+// order inside a bin leaves every bin's range unchanged; along the Morton curve 64 consecutive
+// entries are near each other in all three axes, so a chunk's bounding record rejects most
+// queries (ordered by x alone, a chunk was a slab of the whole y-z extent).
+__global__ void k_tm_key(const RecF *rec, const uint32_t *bin_of, uint64_t n, MortonMap mm,
+                         uint64_t *keys, uint32_t *vals)
 {
     const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const RecF r = rec[s];
-    uint32_t u = __float_as_uint(0.5f * r.xmin + 0.5f * r.xmax + 0.0f);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    keys[s] = ((uint64_t)bin_of[s] << 32) | u;
+    keys[s] = ((uint64_t)bin_of[s] << (3 * mm.bits)) |
+              mm.code(0.5f * r.xmin + 0.5f * r.xmax, 0.5f * r.ymin + 0.5f * r.ymax,
+                      0.5f * r.zmin + 0.5f * r.zmax);
     vals[s] = (uint32_t)s;
 }
 
@@ -269,29 +270,33 @@ __global__ void k_mbb(SegIn in, const uint32_t *orig, uint64_t n, int dim, doubl
     hi[s] = a < b ? b : a;
 }
 
-__global__ void k_part_count(const double *lo, const double *hi, uint64_t n, double plo, double pw,
-                             int v, uint32_t *cnt)
+// (in the sweep order `tid` of the bins' entries)
+__global__ void k_part_count(const double *lo, const double *hi, const uint32_t *tid, uint64_t n,
+                             double plo, double pw, int v, uint32_t *cnt)
 {
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
+    uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t s = tid[p];
     int a = part_of(lo[s], plo, pw, v);
     int b = part_of(hi[s], plo, pw, v);
     if (a < 0) a = 0;
-    cnt[s] = b >= a ? (uint32_t)(b - a + 1) : 0u;
+    cnt[p] = b >= a ? (uint32_t)(b - a + 1) : 0u;
 }
 
-__global__ void k_part_emit(const double *lo, const double *hi, uint64_t n, double plo, double pw,
-                            int v, const uint32_t *pos, uint32_t *keys, uint32_t *vals)
+__global__ void k_part_emit(const double *lo, const double *hi, const uint32_t *tid, uint64_t n,
+                            double plo, double pw, int v, const uint32_t *pos, uint32_t *keys,
+                            uint32_t *vals)
 {
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
+    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t s = tid[i];
     int a = part_of(lo[s], plo, pw, v);
     int b = part_of(hi[s], plo, pw, v);
     if (a < 0) a = 0;
-    uint32_t p = pos[s];
+    uint32_t p = pos[i];
     for (int j = a; j <= b; j++, p++) {
         keys[p] = (uint32_t)j;
-        vals[p] = (uint32_t)s;
+        vals[p] = s;
     }
 }
 
@@ -374,7 +379,22 @@ ts_status counts_to_pos(Ctx &c, const uint32_t *cnt, uint64_t n, DevBuf &pos, ui
     return TS_OK;
 }
 
-// One dimension of the spatiotemporal index.
+// Bounding records of an array's chunks.
+ts_status build_boxes(Ctx &c, Index *ix, const RecF *rec, uint64_t n, RecF **box)
+{
+    const uint64_t nchunks = (n + 63) / 64;
+    TS_CHECK(ix->alloc(box, nchunks));
+    const unsigned cb = (unsigned)std::min<uint64_t>((nchunks * 32 + TPB - 1) / TPB, 152 * 32);
+    if (nchunks) {
+        k_chunk_box<<<cb, TPB, 0, c.s>>>(rec, n, nchunks, *box);
+        TS_LAUNCHED();
+    }
+    return TS_OK;
+}
+
+// One dimension of the spatiotemporal index. The ids are emitted in the bins' sweep order and
+// sorted stably by subbin, so a (subbin, bin) range keeps the Morton order inside and its chunks
+// are small boxes too.
 ts_status build_st_dim(Ctx &c, Index *ix, int dim, const double *lo, const double *hi,
                        const uint32_t *bin_of)
 {
@@ -382,15 +402,15 @@ ts_status build_st_dim(Ctx &c, Index *ix, int dim, const double *lo, const doubl
     const int v = (int)ix->v[dim];
     DevBuf cnt, pos;
     TS_CHECK(cnt.alloc(sizeof(uint32_t) * n, c.s));
-    k_part_count<<<nblocks(n), TPB, 0, c.s>>>(lo, hi, n, ix->sub_lo[dim], ix->sub_w[dim], v,
-                                              cnt.as<uint32_t>());
+    k_part_count<<<nblocks(n), TPB, 0, c.s>>>(lo, hi, ix->tid, n, ix->sub_lo[dim], ix->sub_w[dim],
+                                              v, cnt.as<uint32_t>());
     TS_LAUNCHED();
     uint64_t len = 0;
     TS_CHECK(counts_to_pos(c, cnt.as<uint32_t>(), n, pos, &len));
     DevBuf keys;
     TS_CHECK(keys.alloc(sizeof(uint32_t) * len, c.s));
     TS_CHECK(ix->alloc(&ix->st_ids[dim], len));
-    k_part_emit<<<nblocks(n), TPB, 0, c.s>>>(lo, hi, n, ix->sub_lo[dim], ix->sub_w[dim], v,
+    k_part_emit<<<nblocks(n), TPB, 0, c.s>>>(lo, hi, ix->tid, n, ix->sub_lo[dim], ix->sub_w[dim], v,
                                              pos.as<uint32_t>(), keys.as<uint32_t>(),
                                              ix->st_ids[dim]);
     TS_LAUNCHED();
@@ -408,6 +428,7 @@ ts_status build_st_dim(Ctx &c, Index *ix, int dim, const double *lo, const doubl
     TS_CHECK(ix->alloc(&ix->st_rec[dim], len));
     k_gather_rec<<<nblocks(len), TPB, 0, c.s>>>(ix->st_ids[dim], len, ix->rec, ix->st_rec[dim]);
     TS_LAUNCHED();
+    TS_CHECK(build_boxes(c, ix, ix->st_rec[dim], len, &ix->st_box[dim]));
     ix->st_len[dim] = len;
     return c.read_status();
 }
@@ -438,11 +459,7 @@ ts_status build_grid(Ctx &c, Index *ix, const double *lo3, const double *hi3)
     TS_LAUNCHED();
     // chunk bounding records: the cell sort is stable over the start-time order, so a chunk of
     // a cell spans a short stretch of time and a query's window skips most of a cell's chunks
-    const uint64_t nchunks = (n + 63) / 64;
-    TS_CHECK(ix->alloc(&ix->gbox, nchunks));
-    const unsigned cb = (unsigned)std::min<uint64_t>((nchunks * 32 + TPB - 1) / TPB, 152 * 32);
-    k_chunk_box<<<cb, TPB, 0, c.s>>>(ix->ga_rec, n, nchunks, ix->gbox);
-    TS_LAUNCHED();
+    TS_CHECK(build_boxes(c, ix, ix->ga_rec, n, &ix->gbox));
     ix->g_len = n;
     return c.read_status();
 }
@@ -599,26 +616,26 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     TS_LAUNCHED();
 
     if (p->kind != TS_INDEX_SPATIAL) {
-        // bins ordered by x inside (ranges over the start-time order cover whole bins)
+        // bins ordered along the Morton curve inside (ranges over the start-time order cover
+        // whole bins): 4 bits an axis more than it takes to tell the entries of a mean bin apart
+        const int per_bin = bits_for(n / ix->m);
+        const MortonMap mm =
+            morton_map(ix, std::min(10, std::max(4, (per_bin + 2) / 3 + 4)));
         DevBuf tkeys, tvals;
         TS_CHECK(tkeys.alloc(sizeof(uint64_t) * n, s));
         TS_CHECK(tvals.alloc(sizeof(uint32_t) * n, s));
-        k_tx_key<<<nblocks(n), TPB, 0, s>>>(ix->rec, bin_of.as<uint32_t>(), n,
+        k_tm_key<<<nblocks(n), TPB, 0, s>>>(ix->rec, bin_of.as<uint32_t>(), n, mm,
                                             tkeys.as<uint64_t>(), tvals.as<uint32_t>());
         TS_LAUNCHED();
         TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), tvals.as<uint32_t>(), n,
-                                32 + bits_for((uint64_t)ix->m - 1), s));
-        const uint64_t nchunks = (n + 63) / 64;
+                                3 * mm.bits + bits_for((uint64_t)ix->m - 1), s));
         TS_CHECK(ix->alloc(&ix->trec, n));
         TS_CHECK(ix->alloc(&ix->tid, n));
-        TS_CHECK(ix->alloc(&ix->tbox, nchunks));
         TS_CUDA(cudaMemcpyAsync(ix->tid, tvals.p, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice,
                                 s));
         k_gather_rec<<<nblocks(n), TPB, 0, s>>>(ix->tid, n, ix->rec, ix->trec);
         TS_LAUNCHED();
-        const unsigned cb = (unsigned)std::min<uint64_t>((nchunks * 32 + TPB - 1) / TPB, 152 * 32);
-        k_chunk_box<<<cb, TPB, 0, s>>>(ix->trec, n, nchunks, ix->tbox);
-        TS_LAUNCHED();
+        TS_CHECK(build_boxes(c, ix, ix->trec, n, &ix->tbox));
     }
 
     if (p->kind == TS_INDEX_SPATIOTEMPORAL || p->kind == TS_INDEX_SPATIAL) {

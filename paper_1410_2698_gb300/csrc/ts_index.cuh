@@ -25,7 +25,7 @@ struct Index {
     double tmin = 0, tmax = 0, max_dur = 0;
     double emin[3] = {0, 0, 0}, emax[3] = {0, 0, 0}, longest[3] = {0, 0, 0};
 
-    // the entries of every temporal bin once more, ordered by x inside the bin (the bins keep
+    // the entries of every temporal bin once more, in Morton order inside the bin (the bins keep
     // their ranges [B^first, B^last]): records, their start-time positions, and the bounding
     // record of every aligned chunk of 64 (built for every kind whose ranges cover bins)
     RecF *trec = nullptr;
@@ -38,12 +38,14 @@ struct Index {
     double *bin_start = nullptr, *bin_end = nullptr, *bin_pmax = nullptr;  // m each
     uint32_t *bin_off = nullptr;  // m + 1
 
-    // spatiotemporal subbins (Sec. 4.3): per dimension an id array in (subbin, bin, time) order,
-    // a duplicated prefilter record per id, and offsets off[j*m + i]
+    // spatiotemporal subbins (Sec. 4.3): per dimension an id array in (subbin, bin, Morton) order
+    // (the export gives it in start-time order), a duplicated prefilter record per id, the
+    // chunks' bounding records, and offsets off[j*m + i]
     uint32_t v[3] = {0, 0, 0};
     double sub_lo[3] = {0, 0, 0}, sub_w[3] = {0, 0, 0};
     uint32_t *st_ids[3] = {nullptr, nullptr, nullptr};
     RecF *st_rec[3] = {nullptr, nullptr, nullptr};
+    RecF *st_box[3] = {nullptr, nullptr, nullptr};
     uint32_t *st_off[3] = {nullptr, nullptr, nullptr};
     double *sub_bound[3] = {nullptr, nullptr, nullptr};  // lo + j*w for j = 0..v
     uint64_t st_len[3] = {0, 0, 0};
@@ -78,5 +80,42 @@ struct Index {
         return TS_OK;
     }
 };
+
+// Morton code of a point of the database's extents: `bits` per axis, interleaved. Points outside
+// (queries) take the nearest cell; the code only orders, so its FP32 rounding never matters.
+struct MortonMap {
+    float lo[3], inv[3];
+    int bits;
+
+    __device__ static __forceinline__ uint32_t spread(uint32_t v)  // bit k -> bit 3k, 10 bits
+    {
+        v = (v | (v << 16)) & 0x030000ffu;
+        v = (v | (v << 8)) & 0x0300f00fu;
+        v = (v | (v << 4)) & 0x030c30c3u;
+        return (v | (v << 2)) & 0x09249249u;
+    }
+    __device__ __forceinline__ uint32_t cell(float x, int d) const
+    {
+        const float top = (float)((1 << bits) - 1);
+        return (uint32_t)fminf(fmaxf((x - lo[d]) * inv[d], 0.0f), top);  // (NaN: 0)
+    }
+    __device__ __forceinline__ uint32_t code(float x, float y, float z) const
+    {
+        return spread(cell(x, 0)) | (spread(cell(y, 1)) << 1) | (spread(cell(z, 2)) << 2);
+    }
+};
+
+inline MortonMap morton_map(const Index *ix, int bits)
+{
+    MortonMap m;
+    m.bits = bits;
+    for (int d = 0; d < 3; d++) {
+        const double ext = ix->emax[d] - ix->emin[d];
+        m.lo[d] = (float)ix->emin[d];
+        const float inv = ext > 0.0 ? (float)((double)(1 << bits) / ext) : 0.0f;
+        m.inv[d] = inv < 3.0e38f ? inv : 0.0f;
+    }
+    return m;
+}
 
 }  // namespace ts

@@ -225,9 +225,9 @@ struct DevBuf {
 // ---------------------------------------------------------------------------------------------
 // The primitives take a capacity n and optionally n_dev, a device word holding the actual count
 // (<= n) of a run whose size only the device knows; the work then follows the actual count.
-// exclusive scan of n u32 values into n+1 u64 offsets (out[n] = total)
+// exclusive scan of n u32 values (their bits in `mask`) into n+1 u64 offsets (out[n] = total)
 ts_status scan_u32_to_u64(const uint32_t *in, uint64_t *out, uint64_t n, cudaStream_t s,
-                          const uint32_t *n_dev = nullptr);
+                          const uint32_t *n_dev = nullptr, uint32_t mask = ~0u);
 // exclusive scan of n u32 values into n+1 u32 offsets; sets DEV_ERR_OVERFLOW in *status when the
 // total does not fit in 32 bits
 ts_status scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *status,

@@ -159,7 +159,8 @@ __device__ __forceinline__ uint64_t dev_count(uint64_t cap, const uint32_t *n_de
 }
 
 template <class Tin, class Tout>
-__global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tout *sums)
+__global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
+                            Tout *sums)
 {
     pdl_enter();
     const uint64_t n = dev_count(ncap, n_dev);
@@ -171,7 +172,7 @@ __global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
     Tout acc = 0;
     for (int k = 0; k < SCAN_ITEMS; k++) {
         uint64_t i = base + (uint64_t)k * SCAN_THREADS + threadIdx.x;
-        if (i < n) acc += (Tout)in[i];
+        if (i < n) acc += (Tout)(in[i] & mask);
     }
     Tout total;
     block_excl_scan<Tout>(acc, &total);
@@ -181,7 +182,7 @@ __global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
 // Scan one tile per block with the tile's starting offset taken from `tile_off` (or 0), writing
 // out[i] = exclusive prefix; the block whose tile holds index n writes out[n] = total.
 template <class Tin, class Tout>
-__global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
+__global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
                             const Tout *tile_off, Tout *out)
 {
     pdl_enter();
@@ -195,7 +196,7 @@ __global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         uint64_t i = tbase + k;
-        v[k] = i < n ? (Tout)in[i] : Tout(0);
+        v[k] = i < n ? (Tout)(in[i] & mask) : Tout(0);
         acc += v[k];
     }
     Tout total;
@@ -216,7 +217,7 @@ __global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
 constexpr uint64_t SCAN_LOOKBACK = 4096;
 
 template <class Tin, class Tout>
-__global__ void k_tile_scan_lb(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
+__global__ void k_tile_scan_lb(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
                                const Tout *sums, Tout *out)
 {
     pdl_enter();
@@ -233,7 +234,7 @@ __global__ void k_tile_scan_lb(const Tin *in, uint64_t ncap, const uint32_t *n_d
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         const uint64_t i = tbase + k;
-        v[k] = i < n ? (Tout)in[i] : Tout(0);
+        v[k] = i < n ? (Tout)(in[i] & mask) : Tout(0);
         acc += v[k];
     }
     Tout total;
@@ -251,7 +252,7 @@ __global__ void k_tile_scan_lb(const Tin *in, uint64_t ncap, const uint32_t *n_d
 // of SCAN_TILE values plus one, so that the tile holding index n always exists.
 template <class Tin, class Tout>
 static ts_status scan_impl(const Tin *in, Tout *out, uint64_t n, const uint32_t *n_dev,
-                           cudaStream_t s)
+                           cudaStream_t s, Tin mask = ~Tin(0))
 {
     if (n == 0) {
         TS_CUDA(cudaMemsetAsync(out, 0, sizeof(Tout), s));
@@ -260,30 +261,30 @@ static ts_status scan_impl(const Tin *in, Tout *out, uint64_t n, const uint32_t 
     const uint64_t nt = n / SCAN_TILE + 1;
     if (nt == 1) {
         TS_LAUNCH_PDL(k_tile_scan<Tin, Tout>, dim3(1), dim3(SCAN_THREADS), 0, s,
-                      in, n, n_dev, nullptr, out);
+                      in, n, n_dev, mask, nullptr, out);
         return TS_OK;
     }
     DevBuf sums;
     TS_CHECK(sums.alloc(sizeof(Tout) * nt, s));
     TS_LAUNCH_PDL(k_tile_sums<Tin, Tout>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                  in, n, n_dev, sums.as<Tout>());
+                  in, n, n_dev, mask, sums.as<Tout>());
     if (nt <= SCAN_LOOKBACK) {
         TS_LAUNCH_PDL(k_tile_scan_lb<Tin, Tout>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                      in, n, n_dev, sums.as<Tout>(), out);
+                      in, n, n_dev, mask, sums.as<Tout>(), out);
         return TS_OK;
     }
     DevBuf offs;
     TS_CHECK(offs.alloc(sizeof(Tout) * (nt + 1), s));
     TS_CHECK((scan_impl<Tout, Tout>(sums.as<Tout>(), offs.as<Tout>(), nt, nullptr, s)));
     TS_LAUNCH_PDL(k_tile_scan<Tin, Tout>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                  in, n, n_dev, offs.as<Tout>(), out);
+                  in, n, n_dev, mask, offs.as<Tout>(), out);
     return TS_OK;
 }
 
 ts_status scan_u32_to_u64(const uint32_t *in, uint64_t *out, uint64_t n, cudaStream_t s,
-                          const uint32_t *n_dev)
+                          const uint32_t *n_dev, uint32_t mask)
 {
-    return scan_impl<uint32_t, uint64_t>(in, out, n, n_dev, s);
+    return scan_impl<uint32_t, uint64_t>(in, out, n, n_dev, s, mask);
 }
 
 __global__ void k_narrow_u64(const uint64_t *in, uint32_t *out, uint64_t ncap,

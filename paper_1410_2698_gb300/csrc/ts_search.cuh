@@ -67,13 +67,15 @@ struct PipeBufs {
     // groups
     uint32_t *g_first, *g_count, *g_nseg;
     MemberRec *gmem;      // GROUP per group, in the group's (array, start) order
-    float4 *ghdr;         // per group: its request's d_dn, d2u, q_first (bits), 0
+    // per group, three: its request's d_dn, d2u, q_first (bits), members (bits); the lower and
+    // the upper bounds of its members' expanded boxes (the windows' in .w)
+    float4 *ghdr;
     uint32_t *seg_lo, *seg_hi, *seg_sel, *seg_t0;  // GROUP per group
     uint32_t *ntiles;
     uint64_t *tile_base;  // groups + 1
     // tiles and rows
-    uint4 *tdesc;         // per tile: {group, s0, s1, sel | (members - 1) << 3 | request << 8}
-    uint32_t *tile_hits;
+    uint4 *tdesc;         // per listed tile: {tile | sel << 29, chunk mask, group, first record}
+    uint32_t *tile_hits;  // per tile: hits, and TILE_REDO
     uint64_t *tile_off;   // tiles + 1
     uint32_t *out_q, *out_e;
     double *out_tin, *out_tout;
@@ -84,7 +86,7 @@ struct PipeBufs {
     uint32_t *hdr;
     unsigned long long *stats;
     uint32_t *status;
-    uint32_t *counters;   // 2 tile counters (count pass, write pass)
+    uint32_t *counters;   // 2 tile counters (count pass, write pass), listed tiles
     const uint32_t *run;  // optional device run header {nq, nreq}: sizes read at run time (graphs)
 };
 
@@ -138,9 +140,15 @@ ts_status pipe_scan_rows(const PipeBufs &b, const PipeCaps &c, cudaStream_t s);
 void inject_stall(uint64_t ns);
 ts_status pipe_write(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, const PipeCaps &c,
                      cudaStream_t s);
-// Layout of a unit's sort key: request | array (sel_bits) | top lo_bits bits of the range start.
+// Layout of a unit's sort key: request | array (sel_bits) | top lo_bits bits of the range start |
+// Morton code of the query (morton bits per axis).
 struct KeyFmt {
-    int lo_bits = 0, lo_shift = 0, sel_bits = 0;
+    int lo_bits = 0, lo_shift = 0, sel_bits = 0, morton = 0;
+};
+// One pointer per candidate array (SEL_X .. SEL_GRID).
+template <class T>
+struct ArrayPtrs {
+    T *p[5];
 };
 constexpr int KEY_LO_BITS = 13;
 constexpr int KEY_LO_MIN = 11;
