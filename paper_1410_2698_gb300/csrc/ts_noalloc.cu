@@ -285,9 +285,7 @@ __global__ void __launch_bounds__(NA_WARPS * 32) k_na_tiles(NaParams P)
                 uint32_t pr = 0;
                 if (b + lane < np) {
                     pr = W.pair[b + lane];
-                    Quad qd;
-                    h = pair_quad(W.q[pr >> 5], W.e[pr & 31u], qd) &&
-                        quad_solve(qd, PASS == 1, &tin, &tout);
+                    h = pair_test(W.q[pr >> 5], W.e[pr & 31u], PASS == 1, &tin, &tout);
                 }
                 const unsigned hm = __ballot_sync(FULL, h);
                 if (PASS == 1 && h) {

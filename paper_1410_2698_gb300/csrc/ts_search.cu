@@ -759,7 +759,7 @@ struct PairParams {
     uint64_t stall_ns;
 };
 
-// Exact FP64 test of one (query, entry) pair and, when `interval`, its hit interval. Not inlined:
+// Exact test of one (query, entry) pair and, when `interval`, its hit interval. Not inlined:
 // the pair kernel calls it only for the candidates that passed both FP32 filters, so the registers
 // it needs are saved around the call instead of being reserved across the whole sweep.
 __device__ __noinline__ bool exact_test(const QueryD *qp, const SegD *ep, bool interval,
@@ -767,8 +767,7 @@ __device__ __noinline__ bool exact_test(const QueryD *qp, const SegD *ep, bool i
 {
     const SegD e = *ep;
     const QueryD q = *qp;
-    Quad qd;
-    return pair_quad(q, e, qd) && quad_solve(qd, interval, tin, tout);
+    return pair_test(q, e, interval, tin, tout);
 }
 
 // Persistent pair kernel. Warps take tiles (a group of up to 32 query units and up to `tile`
