@@ -190,8 +190,9 @@ ts_status create_plan(const Index *ix, const ts_batch_params *prm, cudaStream_t 
     // hits the count pass keeps for placement after the scan; more hits than this make the
     // write pass sweep the tiles again
     k.scratch = prm->scratch_rows ? prm->scratch_rows
-                : own_rows       ? prm->max_rows
-                                 : std::min<uint64_t>(4 * k.nq + (1ull << 20), SCRATCH_MAX);
+                : scratch_slots(own_rows ? prm->max_rows
+                                         : std::min<uint64_t>(4 * k.nq + (1ull << 20), SCRATCH_MAX));
+    if (k.scratch > 0xffffffffull) k.scratch = 0xffffffffull;  // (slots are numbered in 32 bits)
     Carver sz;
     layout(p.get(), sz);
     p->dbytes = sz.off;

@@ -153,7 +153,7 @@ __global__ void k_tm_key(const RecF *rec, const uint32_t *bin_of, uint64_t n, Mo
 }
 
 // Bounding record of every aligned chunk of 64 records, a warp per chunk.
-__global__ void k_chunk_box(const RecF *rec, uint64_t n, uint64_t nchunks, RecF *box)
+__global__ void k_chunk_box(const Chunk *rec, uint64_t n, uint64_t nchunks, RecF *box)
 {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
@@ -164,7 +164,7 @@ __global__ void k_chunk_box(const RecF *rec, uint64_t n, uint64_t nchunks, RecF 
         for (int h = 0; h < 2; h++) {
             const uint64_t i = c * 64 + h * 32 + lane;
             if (i < n) {
-                const RecF r = rec[i];
+                const RecF r = rec[c].r[h * 32 + lane];
                 lo[0] = fminf(lo[0], r.xmin); hi[0] = fmaxf(hi[0], r.xmax);
                 lo[1] = fminf(lo[1], r.ymin); hi[1] = fmaxf(hi[1], r.ymax);
                 lo[2] = fminf(lo[2], r.zmin); hi[2] = fmaxf(hi[2], r.zmax);
@@ -308,10 +308,13 @@ __global__ void k_st_hist(const uint32_t *keys, const uint32_t *ids, uint64_t le
     atomicAdd(&cnt[(uint64_t)keys[p] * m + bin_of[ids[p]]], 1u);
 }
 
-__global__ void k_gather_rec(const uint32_t *ids, uint64_t len, const RecF *rec, RecF *out)
+__global__ void k_gather_rec(const uint32_t *ids, uint64_t len, const RecF *rec, Chunk *out)
 {
     uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < len) out[p] = rec[ids[p]];
+    if (p >= len) return;
+    const uint32_t s = ids[p];
+    out[p / CHUNK].r[p % CHUNK] = rec[s];
+    out[p / CHUNK].id[p % CHUNK] = s;
 }
 
 // grid: every sorted entry is keyed by the cell of its MBB's minimum corner (single assignment)
@@ -380,7 +383,7 @@ ts_status counts_to_pos(Ctx &c, const uint32_t *cnt, uint64_t n, DevBuf &pos, ui
 }
 
 // Bounding records of an array's chunks.
-ts_status build_boxes(Ctx &c, Index *ix, const RecF *rec, uint64_t n, RecF **box)
+ts_status build_boxes(Ctx &c, Index *ix, const Chunk *rec, uint64_t n, RecF **box)
 {
     const uint64_t nchunks = (n + 63) / 64;
     TS_CHECK(ix->alloc(box, nchunks));
@@ -425,7 +428,7 @@ ts_status build_st_dim(Ctx &c, Index *ix, int dim, const double *lo, const doubl
     TS_LAUNCHED();
     TS_CHECK(ix->alloc(&ix->st_off[dim], nbins + 1));
     TS_CHECK(scan_u32(h.as<uint32_t>(), ix->st_off[dim], nbins, c.status.as<uint32_t>(), c.s));
-    TS_CHECK(ix->alloc(&ix->st_rec[dim], len));
+    TS_CHECK(ix->alloc(&ix->st_rec[dim], (len + CHUNK - 1) / CHUNK));
     k_gather_rec<<<nblocks(len), TPB, 0, c.s>>>(ix->st_ids[dim], len, ix->rec, ix->st_rec[dim]);
     TS_LAUNCHED();
     TS_CHECK(build_boxes(c, ix, ix->st_rec[dim], len, &ix->st_box[dim]));
@@ -454,7 +457,7 @@ ts_status build_grid(Ctx &c, Index *ix, const double *lo3, const double *hi3)
     TS_LAUNCHED();
     TS_CHECK(ix->alloc(&ix->g_off, ncell + 1));
     TS_CHECK(scan_u32(h.as<uint32_t>(), ix->g_off, ncell, c.status.as<uint32_t>(), c.s));
-    TS_CHECK(ix->alloc(&ix->ga_rec, n));
+    TS_CHECK(ix->alloc(&ix->ga_rec, (n + CHUNK - 1) / CHUNK));
     k_gather_rec<<<nblocks(n), TPB, 0, c.s>>>(ix->ga, n, ix->rec, ix->ga_rec);
     TS_LAUNCHED();
     // chunk bounding records: the cell sort is stable over the start-time order, so a chunk of
@@ -629,7 +632,7 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         TS_LAUNCHED();
         TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), tvals.as<uint32_t>(), n,
                                 3 * mm.bits + bits_for((uint64_t)ix->m - 1), s));
-        TS_CHECK(ix->alloc(&ix->trec, n));
+        TS_CHECK(ix->alloc(&ix->trec, (n + CHUNK - 1) / CHUNK));
         TS_CHECK(ix->alloc(&ix->tid, n));
         TS_CUDA(cudaMemcpyAsync(ix->tid, tvals.p, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice,
                                 s));

@@ -28,7 +28,7 @@ struct Index {
     // the entries of every temporal bin once more, in Morton order inside the bin (the bins keep
     // their ranges [B^first, B^last]): records, their start-time positions, and the bounding
     // record of every aligned chunk of 64 (built for every kind whose ranges cover bins)
-    RecF *trec = nullptr;
+    Chunk *trec = nullptr;
     uint32_t *tid = nullptr;
     RecF *tbox = nullptr;
 
@@ -44,7 +44,7 @@ struct Index {
     uint32_t v[3] = {0, 0, 0};
     double sub_lo[3] = {0, 0, 0}, sub_w[3] = {0, 0, 0};
     uint32_t *st_ids[3] = {nullptr, nullptr, nullptr};
-    RecF *st_rec[3] = {nullptr, nullptr, nullptr};
+    Chunk *st_rec[3] = {nullptr, nullptr, nullptr};
     RecF *st_box[3] = {nullptr, nullptr, nullptr};
     uint32_t *st_off[3] = {nullptr, nullptr, nullptr};
     double *sub_bound[3] = {nullptr, nullptr, nullptr};  // lo + j*w for j = 0..v
@@ -57,7 +57,7 @@ struct Index {
     uint32_t g = 0;
     double g_lo[3] = {0, 0, 0}, g_w[3] = {0, 0, 0};
     uint32_t *ga = nullptr;
-    RecF *ga_rec = nullptr;
+    Chunk *ga_rec = nullptr;
     RecF *gbox = nullptr;  // bounding record of every aligned chunk of 64 of ga_rec
     uint32_t *g_off = nullptr;  // g^3 + 1
     double *g_bound[3] = {nullptr, nullptr, nullptr};  // lo + j*w for j = 0..g

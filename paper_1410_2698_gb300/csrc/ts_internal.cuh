@@ -4,9 +4,9 @@
 //   SegD  : 64 B per entry, FP64 start point, start time, velocity, end time (exact test)
 //   RecF  : 32 B per entry, FP32 MBB rounded outward + start/end time rounded outward
 //           (conservative prefilter)
-//   Entries are stored in start-time order (Sec. 4.2); the spatiotemporal id arrays (Sec. 4.3)
-//   and the grid lookup array (Sec. 4.1) keep a duplicated RecF next to every id so candidate
-//   ranges stream contiguously.
+//   Entries are stored in start-time order (Sec. 4.2); the temporal bins' sweep order, the
+//   spatiotemporal id arrays (Sec. 4.3) and the grid lookup array (Sec. 4.1) keep a duplicated
+//   RecF next to every id, in chunks of 64, so candidate ranges stream contiguously.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -31,7 +31,16 @@ struct __align__(16) RecF {
 };
 static_assert(sizeof(RecF) == 32, "RecF is 32 bytes");
 
-struct __align__(16) SegD {
+// 64 consecutive records of a swept array with their entries' positions in the start-time order:
+// one bulk copy of the pair kernel. (The slots past an array's end hold nothing.)
+constexpr int CHUNK = 64;
+struct __align__(16) Chunk {
+    RecF r[CHUNK];
+    uint32_t id[CHUNK];
+};
+static_assert(sizeof(Chunk) == 2304, "Chunk is 2304 bytes");
+
+struct __align__(32) SegD {
     double x0, y0, z0, t0;
     double vx, vy, vz, t1;
 };
@@ -40,12 +49,12 @@ static_assert(sizeof(SegD) == 64, "SegD is 64 bytes");
 // Exact data of one query segment: its position at the start w0 of its clipped window [w0, w1],
 // its velocity, and minus the request's d^2 (the addend of c, stored negated so that no FP64
 // instruction negates it).
-struct __align__(16) QueryD {
+struct __align__(32) QueryD {
     double xw, yw, zw, w0;
     double vx, vy, vz, w1;
-    double ndd, pad;
+    double ndd, pad[3];
 };
-static_assert(sizeof(QueryD) == 80, "QueryD is 80 bytes");
+static_assert(sizeof(QueryD) == 96, "QueryD is 96 bytes");
 
 // Query group: up to 32 consecutive (sorted) queries sharing one candidate array and range.
 struct Group {
@@ -69,10 +78,12 @@ enum : uint32_t {
 // Stats slots (u64 array in device memory).
 enum : int {
     ST_QSEGS = 0, ST_TESTS = 1, ST_EXACT = 2, ST_HITS = 3, ST_TILES = 4, ST_GROUPS = 5,
-    ST_SUBBIN = 6, ST_SCRATCH = 7,  // ST_SCRATCH: hits offered to the scratch
+    ST_SUBBIN = 6, ST_SCRATCH = 7,  // ST_SCRATCH: slots of the scratch taken
     // pair kernel sweep (count pass): chunks swept, chunks swept by the two-axis bitmask, member
     // visits of the sparse path, survivors of the bitmask given the full FP32 filters
-    ST_CHUNKS = 8, ST_DENSE = 9, ST_SPARSE = 10, ST_STAGE2 = 11, ST_NSLOTS = 12
+    ST_CHUNKS = 8, ST_DENSE = 9, ST_SPARSE = 10, ST_STAGE2 = 11,
+    ST_LOST = 12,  // some hit found no slot of the scratch
+    ST_NSLOTS = 13
 };
 
 // ---------------------------------------------------------------------------------------------

@@ -274,7 +274,6 @@ __global__ void __launch_bounds__(NA_WARPS * 32) k_na_tiles(NaParams P)
                     q.yw = fma(q.vy, dw, v[1]);
                     q.zw = fma(q.vz, dw, v[2]);
                     q.ndd = -P.dd;
-                    q.pad = 0.0;
                     W.q[lane] = q;
                 }
             }

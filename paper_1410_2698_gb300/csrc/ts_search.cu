@@ -231,7 +231,7 @@ __global__ void k_qprep(PrepParams P)
         q.yw = fma(q.vy, dw, v[1]);
         q.zw = fma(q.vz, dw, v[2]);
         q.ndd = -R.dd;
-        q.pad = 0.0;
+        q.pad[0] = q.pad[1] = q.pad[2] = 0.0;
         const bool valid = fin && (v[7] > v[3]) && (q.w0 < q.w1);
         P.b.qd[i] = q;
         P.b.qreq[i] = r;
@@ -717,21 +717,26 @@ __global__ void k_tile_desc(uint64_t gcap, uint64_t tcap, uint32_t tile, ArrayPt
 // pair kernel
 // ---------------------------------------------------------------------------------------------
 struct __align__(16) WarpSmem {
-    RecF stage[PK_STAGES][PK_CH];
+    Chunk stage[PK_STAGES];
     MemberRec mem[GROUP];  // the tile's group members
-    float4 ghdr;           // their request's d_dn, d2u, q_first (and the request)
-    uint4 dnext;           // the next tile's descriptor (asynchronous copy during the sweep)
-    RecF cbox[32];         // bounding records of the tile's chunks (arrays that have them)
+    float4 ghdr;           // their request's d_dn, d2u, q_first, and their number
+    uint4 dnext;           // the next listed tile (asynchronous copy during the sweep)
+    RecF cbox[32];         // bounding records of the tile's chunks
     // exact-test queue, first in first out, carried from tile to tile: query index in the batch,
-    // entry position in its sorted array, tile | sel << 29, query index within its request
-    uint32_t q_qi[PK_QUEUE], q_pos[PK_QUEUE], q_tile[PK_QUEUE], q_ql[PK_QUEUE];
+    // entry, tile, query index within its request
+    uint32_t q_qi[PK_QUEUE], q_e[PK_QUEUE], q_tile[PK_QUEUE], q_ql[PK_QUEUE];
     uint32_t plist[PK_PLIST];  // (member << 8 | slot) pairs of a chunk that passed the box test
     unsigned long long bar[PK_STAGES];
     unsigned long long mbar;  // members + chunk boxes
     unsigned long long xbar;  // injected stall (tests): a barrier nothing ever arrives on
-    // counts of the count pass: chunks, bitmask chunks, sparse member visits, survivors (then,
-    // at the end, the warp's FP64 tests and hits; the last slots pad to 64 bytes)
-    unsigned long long sweep[8];
+    // counts: chunks, bitmask chunks, sparse member visits, survivors, exact tests, hits
+    unsigned long long count[6];
+    uint32_t wt_cur, wt_cnt;  // last tile with hits, its hits so far
+    // Count pass: this warp's part [sc_at, sc_end) of the scratch. Parts are taken from a shared
+    // counter, 32 slots first and then half of what the warp has had (sc_had), at most 256: an
+    // atomic for every batch of hits put its round trip to L2 into each batch, and all of them on
+    // one address. `room` until a part did not fit.
+    uint32_t sc_at, sc_end, sc_had, room;
 };
 
 enum { PASS_COUNT = 0, PASS_WRITE = 1 };
@@ -744,9 +749,8 @@ constexpr uint32_t TILE_REDO = 0x80000000u;
 struct PairParams {
     PipeBufs b;
     const ReqDesc *reqs;
-    const RecF *rec[5];
-    const uint32_t *ids[5];
-    const RecF *box[5];  // bounding record per aligned chunk of 64 records
+    const Chunk *rec[5];
+    const RecF *box[5];  // bounding record per chunk
     uint32_t len[5];     // records of the array
     const SegD *seg;
     const uint32_t *orig;
@@ -759,30 +763,184 @@ struct PairParams {
     uint64_t stall_ns;
 };
 
-// Exact test of one (query, entry) pair and, when `interval`, its hit interval. Not inlined:
-// the pair kernel calls it only for the candidates that passed both FP32 filters, so the registers
-// it needs are saved around the call instead of being reserved across the whole sweep.
-__device__ __noinline__ bool exact_test(const QueryD *qp, const SegD *ep, bool interval,
-                                        double *tin, double *tout)
+// Exact test of nflush queued candidates from the queue's place `at` on, one per lane, and what
+// becomes of their hits.
+template <int PASS>
+__device__ __forceinline__ void pair_batch(WarpSmem &W, const PairParams &P, uint32_t at,
+                                           uint32_t nflush)
 {
-    const SegD e = *ep;
-    const QueryD q = *qp;
-    return pair_test(q, e, interval, tin, tout);
+    const int lane = threadIdx.x & 31;
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    const PipeBufs &B = P.b;
+    uint32_t qi = 0, eid = 0, tile = 0xffffffffu, ql = 0, orig = 0;
+    if ((uint32_t)lane < nflush) {
+        qi = W.q_qi[at + lane];
+        eid = W.q_e[at + lane];
+        tile = W.q_tile[at + lane];
+        ql = W.q_ql[at + lane];
+        orig = P.orig[eid];
+    }
+    const bool room = W.room != 0;
+    // the count pass computes hit intervals only while the scratch still has room, as far as this
+    // warp has seen (after an overflow the write pass sweeps and computes them)
+    const bool interval = PASS == PASS_WRITE || room;
+    bool h = false;
+    double tin = 0.0, tout = 0.0;
+    if ((uint32_t)lane < nflush) {
+        SegD e;
+        QueryD q;
+        ld32(P.seg + eid, &e.x0);
+        ld32(&P.seg[eid].vx, &e.vx);
+        ld32(B.qd + qi, &q.xw);
+        ld32(&B.qd[qi].vx, &q.vx);
+        q.ndd = B.qd[qi].ndd;
+        h = pair_test(q, e, interval, &tin, &tout);
+    }
+    const unsigned hm = __ballot_sync(FULL, h);
+    if (lane == 0) {
+        W.count[4] += nflush;
+        W.count[5] += __popc(hm);
+    }
+    if (!hm) return;
+    // hits of the same tile (the queue holds a tile's candidates contiguously, tiles in the order
+    // this warp took them)
+    const unsigned mine = hm & __match_any_sync(FULL, h ? tile : 0xffffffffu);
+    // rank of the hit among its tile's rows (queue order, the same in both passes)
+    const uint32_t wt_cur = W.wt_cur, wt_cnt = W.wt_cnt;
+    const uint32_t rank = (tile == wt_cur ? wt_cnt : 0u) + __popc(mine & lt_mask);
+    if (PASS == PASS_COUNT) {
+        if (h && (mine & lt_mask) == 0) atomicAdd(&B.tile_hits[tile], (uint32_t)__popc(mine));
+        if (P.scap) {
+            const uint32_t sc_at = W.sc_at, sc_end = W.sc_end;
+            const uint32_t nh = __popc(hm), left = sc_end - sc_at;
+            const uint32_t k = __popc(hm & lt_mask);  // rank among the batch's hits
+            uint32_t slot = sc_at + k;
+            bool kept = h && k < left;
+            __syncwarp();
+            if (nh <= left) {
+                if (lane == 0) W.sc_at = sc_at + nh;
+            } else if (room) {
+                const uint32_t had = W.sc_had, want = min(256u, max(32u, had / 2));
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(&B.stats[ST_SCRATCH], (unsigned long long)want);
+                base = __shfl_sync(FULL, base, 0);
+                if (base + want <= P.scap) {
+                    if (k >= left) slot = (uint32_t)base + (k - left);
+                    kept = h;
+                    if (lane == 0) {
+                        W.sc_at = (uint32_t)base + (nh - left);
+                        W.sc_end = (uint32_t)base + want;
+                        W.sc_had = had + want;
+                    }
+                } else {
+                    // (the part's slots inside the scratch hold no hit)
+                    for (unsigned long long j = base + lane; j < P.scap; j += 32)
+                        B.s_tile[j] = 0xffffffffu;
+                    if (lane == 0) {
+                        B.stats[ST_LOST] = 1;
+                        W.sc_at = sc_end;
+                        W.room = 0;
+                    }
+                }
+            }
+            if (kept) {
+                B.s_tile[slot] = tile;
+                B.s_rank[slot] = rank;
+                B.s_q[slot] = ql;
+                B.s_e[slot] = orig;
+                B.s_tin[slot] = tin;
+                B.s_tout[slot] = tout;
+            }
+            // a tile with a hit the scratch could not keep is swept again by the write pass
+            const unsigned lost = __ballot_sync(FULL, h && !kept);
+            if (h && !kept && (mine & lost & lt_mask) == 0)
+                atomicOr(&B.tile_hits[tile], TILE_REDO);
+        }
+    } else if (h) {
+        const uint64_t o = B.tile_off[tile] + rank;
+        if (o < B.tile_off[tile + 1]) {
+            B.out_q[o] = ql;
+            B.out_e[o] = orig;
+            B.out_tin[o] = tin;
+            B.out_tout[o] = tout;
+        } else {
+            atomicOr(B.status, DEV_ERR_INTERNAL);  // the passes disagree
+        }
+    }
+    const int last = 31 - __clz(hm);
+    const uint32_t last_tile = __shfl_sync(FULL, tile, last);
+    const uint32_t last_n = __popc(__shfl_sync(FULL, mine, last));
+    __syncwarp();
+    if (lane == 0) {
+        W.wt_cnt = (last_tile == wt_cur ? wt_cnt : 0u) + last_n;
+        W.wt_cur = last_tile;
+    }
+    __syncwarp();
 }
 
-// Persistent pair kernel. Warps take tiles (a group of up to 32 query units and up to `tile`
-// consecutive entries of one sorted array): the first by their index in the grid, the rest from
-// a device counter. Entry records stream through
-// a ring of PK_STAGES shared-memory buffers filled by 1-D bulk copies. The conservative FP32
-// filters pick the candidates of the exact FP64 test; those wait in a per-warp queue that is
-// carried across tiles and drained 32 at a time, so that the FP64 instructions run on full warps.
-// Count pass: hits per tile. Write pass: the rows of every tile with hits, at its offset from the
-// scan, in queue order (the same order in both passes, so the offsets match).
+// Exact tests of the queued candidates, oldest first, 32 at a time; with `all` the rest too.
+// Returns how many stay queued (moved to the front). Not inlined, and called at one place, where
+// the sweep has little in registers (what lasts is in shared memory), so that those of the exact
+// test do not limit the warps that sweep.
 template <int PASS>
-__global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(PairParams P)
+__device__ __noinline__ uint32_t pair_flush(uint32_t qn, bool all)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    WarpSmem &W = reinterpret_cast<WarpSmem *>(smem_raw)[threadIdx.x >> 5];
+    const PairParams &P = *reinterpret_cast<const PairParams *>(smem_raw + PK_WARPS * sizeof(WarpSmem));
+    const int lane = threadIdx.x & 31;
+    uint32_t at = 0;
+    __syncwarp();
+    for (; qn - at >= 32; at += 32) pair_batch<PASS>(W, P, at, 32);
+    if (all && qn > at) {
+        pair_batch<PASS>(W, P, at, qn - at);
+        at = qn;
+    }
+    uint32_t v[4];
+    const bool keep = at + lane < qn;
+    if (keep) {
+        v[0] = W.q_qi[at + lane];
+        v[1] = W.q_e[at + lane];
+        v[2] = W.q_tile[at + lane];
+        v[3] = W.q_ql[at + lane];
+    }
+    __syncwarp();
+    if (keep) {
+        W.q_qi[lane] = v[0];
+        W.q_e[lane] = v[1];
+        W.q_tile[lane] = v[2];
+        W.q_ql[lane] = v[3];
+    }
+    __syncwarp();
+    return qn - at;
+}
+
+// Persistent pair kernel. Warps take listed tiles (a group of up to 32 query units and up to
+// `tile` consecutive entries of one sorted array): the first by their index in the grid, the rest
+// from a device counter. Entry records stream through a ring of PK_STAGES shared-memory buffers
+// filled by 1-D bulk copies. The conservative FP32 filters pick the candidates of the exact test;
+// those wait in a per-warp queue that is carried across tiles and drained 32 at a time, so that
+// the exact tests run on full warps.
+//
+// Bound: instruction issue (63 % of the slots on 11 M exact tests among 2.3 G candidates; ALU 50 %,
+// shared-memory wavefronts 52 %, FP64 33 %). What it waits for is mostly the fixed latency of its
+// own arithmetic, so the number of resident warps counts: 20 per SM (96 registers) instead of 16
+// took 1.13 G exact tests (merger, 20M segments, d = 1 and 5) from 88 to 76 ms; 24 (80
+// registers, spilled, and little L1 left) take 122. Flushes where the queue fills, rather than
+// in the middle of every batch of survivors, the ids beside the records and the scratch taken in
+// parts: 100 to 88 ms. Count pass: hits per tile. Write pass: the rows of every
+// tile with hits, at its offset from the scan, in queue order (the same order in both passes, so
+// the offsets match).
+template <int PASS>
+__global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairParams P)
 {
     pdl_enter();
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    // (pair_flush's copy of the parameters)
+    if (threadIdx.x == 0)
+        *reinterpret_cast<PairParams *>(smem_raw + PK_WARPS * sizeof(WarpSmem)) = P;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     WarpSmem &W = reinterpret_cast<WarpSmem *>(smem_raw)[wid];
@@ -791,20 +949,21 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(PairParams P
     const PipeBufs &B = P.b;
 
     if (lane == 0) {
-        for (int k = 0; k < 4; k++) W.sweep[k] = 0;
+        for (int k = 0; k < 6; k++) W.count[k] = 0;
+        W.wt_cur = 0xffffffffu;
+        W.wt_cnt = 0;
+        W.sc_at = W.sc_end = W.sc_had = 0;
+        W.room = PASS == PASS_COUNT && P.scap != 0;
         for (int k = 0; k < PK_STAGES; k++) mbar_init(&W.bar[k], 1);
         mbar_init(&W.mbar, 1);
         mbar_init(&W.xbar, 1);
         fence_mbar_init();
     }
     __syncwarp();
-    uint32_t parity[PK_STAGES], mparity = 0u;
-    bool pending[PK_STAGES], mpending = false;
-#pragma unroll
-    for (int k = 0; k < PK_STAGES; k++) {
-        parity[k] = 0u;
-        pending[k] = false;
-    }
+    // bits k: the parity the next wait on bar[k] is for, bit PK_STAGES: on mbar; and the copies in
+    // flight
+    uint32_t parity = 0u, pending = 0u;
+    constexpr uint32_t MEM = 1u << PK_STAGES;
     bool abort = false;
     if (P.stall_ns && blockIdx.x == 0 && wid == 0)
         abort = !mbar_wait_bounded(&W.xbar, 0u, P.stall_ns);  // (never arrived on: times out)
@@ -812,7 +971,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(PairParams P
     const uint64_t all_tiles = (uint64_t)B.hdr[HDR_T_LO] | ((uint64_t)B.hdr[HDR_T_HI] << 32);
     uint32_t ntiles = B.counters[2];  // listed tiles
     if (all_tiles > P.tcap || all_tiles > PK_MAX_TILES) ntiles = 0;  // overflow already flagged
-    if (PASS == PASS_WRITE && P.scap && B.stats[ST_SCRATCH] <= P.scap)
+    if (PASS == PASS_WRITE && P.scap && B.stats[ST_LOST] == 0)
         ntiles = 0;  // the count pass kept every hit: k_place writes the rows
     // (otherwise the write pass sweeps only the tiles whose hits were not all kept)
     if (PASS == PASS_WRITE && ntiles && B.tile_off[all_tiles] > P.rows_cap) {
@@ -820,93 +979,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(PairParams P
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(B.status, DEV_ERR_OVERFLOW);
         ntiles = 0;
     }
-    unsigned long long acc_exact = 0, acc_hits = 0;
-    uint32_t qn = 0;                            // queued candidates (warp-uniform)
-    uint32_t wt_cur = 0xffffffffu, wt_cnt = 0;  // last tile with hits, its hits so far
-    // count pass: the scratch had room after this warp's last reservation (the warp's own view:
-    // reading the shared counter before every batch of exact tests would put a round trip to L2
-    // in front of each)
-    bool room = true;
-
-    // Exact test of the oldest nflush queued candidates, one per lane.
-    auto flush = [&](uint32_t nflush) {
-        uint32_t qi = 0, pos = 0, tw = 0xffffffffu, ql = 0;
-        if ((uint32_t)lane < nflush) {
-            qi = W.q_qi[lane];
-            pos = W.q_pos[lane];
-            tw = W.q_tile[lane];
-            ql = W.q_ql[lane];
-        }
-        __syncwarp();
-        if (qn > nflush && (uint32_t)lane < qn - nflush) {
-            const uint32_t j = nflush + lane;
-            W.q_qi[lane] = W.q_qi[j];
-            W.q_pos[lane] = W.q_pos[j];
-            W.q_tile[lane] = W.q_tile[j];
-            W.q_ql[lane] = W.q_ql[j];
-        }
-        __syncwarp();
-        qn -= nflush;
-        acc_exact += nflush;
-        bool h = false;
-        double tin = 0.0, tout = 0.0;
-        uint32_t eid = 0;
-        const uint32_t tile = tw & PK_MAX_TILES;
-        // the count pass computes hit intervals only while the scratch still has room, as far
-        // as this warp has seen (after an overflow the write pass sweeps and computes them; a
-        // hit is kept only when its slot fits, so a stale view costs at most some intervals)
-        const bool interval = PASS == PASS_WRITE || (P.scap != 0 && room);
-        if ((uint32_t)lane < nflush) {
-            eid = P.ids[tw >> 29][pos];
-            h = exact_test(B.qd + qi, P.seg + eid, interval, &tin, &tout);
-        }
-        const unsigned hm = __ballot_sync(FULL, h);
-        if (!hm) return;
-        acc_hits += __popc(hm);
-        // hits of the same tile (the queue holds a tile's candidates contiguously, tiles in the
-        // order this warp took them)
-        const unsigned mine = hm & __match_any_sync(FULL, h ? tile : 0xffffffffu);
-        // rank of the hit among its tile's rows (queue order, the same in both passes)
-        const uint32_t rank = (tile == wt_cur ? wt_cnt : 0u) + __popc(mine & lt_mask);
-        if (PASS == PASS_COUNT) {
-            if (h && (mine & lt_mask) == 0) atomicAdd(&B.tile_hits[tile], (uint32_t)__popc(mine));
-            if (P.scap) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(&B.stats[ST_SCRATCH], (unsigned long long)__popc(hm));
-                base = __shfl_sync(FULL, base, 0);
-                room = base + (unsigned long long)__popc(hm) < P.scap;
-                const unsigned long long slot = base + __popc(hm & lt_mask);
-                const bool kept = h && slot < P.scap && interval;
-                if (kept) {
-                    B.s_tile[slot] = tile;
-                    B.s_rank[slot] = rank;
-                    B.s_q[slot] = ql;
-                    B.s_e[slot] = P.orig[eid];
-                    B.s_tin[slot] = tin;
-                    B.s_tout[slot] = tout;
-                }
-                // a tile with a hit the scratch could not keep is swept again by the write pass
-                const unsigned lost = __ballot_sync(FULL, h && !kept);
-                if (h && !kept && (mine & lost & lt_mask) == 0)
-                    atomicOr(&B.tile_hits[tile], TILE_REDO);
-            }
-        } else if (h) {
-            const uint64_t o = B.tile_off[tile] + rank;
-            if (o < B.tile_off[tile + 1]) {
-                B.out_q[o] = ql;
-                B.out_e[o] = P.orig[eid];
-                B.out_tin[o] = tin;
-                B.out_tout[o] = tout;
-            } else {
-                atomicOr(B.status, DEV_ERR_INTERNAL);  // the passes disagree
-            }
-        }
-        const int last = 31 - __clz(hm);
-        const uint32_t last_tile = __shfl_sync(FULL, tile, last);
-        const uint32_t last_n = __popc(__shfl_sync(FULL, mine, last));
-        wt_cnt = (last_tile == wt_cur ? wt_cnt : 0u) + last_n;
-        wt_cur = last_tile;
-    };
+    uint32_t qn = 0;  // queued candidates (warp-uniform)
 
     // listed tiles are taken from a device counter; the next entry is fetched while a tile is
     // swept
@@ -927,270 +1000,259 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(PairParams P
                 continue;
             }
         }
-        const uint32_t tw = D.x, sel = D.x >> 29, cand = D.y, g = D.z, s0 = D.w;
-        const RecF *recs = P.rec[sel];
-        const uint32_t n_rec = P.len[sel];
-        // chunks are whole but for the array's last (slots past a member's range are masked by
-        // the range itself)
-        auto copy_chunk = [&](uint32_t c, int st) {
-            const uint32_t cs = s0 + c * PK_CH;
-            const uint32_t nb = min((uint32_t)PK_CH, n_rec - cs) * (uint32_t)sizeof(RecF);
-            mbar_arrive_tx(&W.bar[st], nb);
-            bulk_g2s(&W.stage[st][0], recs + cs, nb, &W.bar[st]);
+        const uint32_t tile = D.x & PK_MAX_TILES, sel = D.x >> 29, cand = D.y, s0 = D.w;
+        // the chunk at s0 + c * PK_CH, whole (slots past the array's end or a member's range are
+        // masked by the range)
+        auto copy_chunk = [&](uint32_t c, uint32_t st) {
+            mbar_arrive_tx(&W.bar[st], (uint32_t)sizeof(Chunk));
+            bulk_g2s(&W.stage[st], P.rec[sel] + s0 / PK_CH + c, (uint32_t)sizeof(Chunk), &W.bar[st]);
         };
         // one bulk copy of the members and of the chunks' bounding records, then the first two
         // listed chunks of records
         uint32_t pend = cand, first = 0;
-        const uint32_t nch = 32 - __clz(cand);  // (a listed tile has a chunk)
         if (lane == 0) {
+            const uint32_t g = D.z;
             const uint32_t mb = GROUP * (uint32_t)sizeof(MemberRec);
-            const uint32_t cb = nch * (uint32_t)sizeof(RecF);
+            const uint32_t cb = (32 - __clz(cand)) * (uint32_t)sizeof(RecF);
             mbar_arrive_tx(&W.mbar, mb + cb + (uint32_t)sizeof(float4));
             bulk_g2s(&W.ghdr, B.ghdr + 3 * (uint64_t)g, (uint32_t)sizeof(float4), &W.mbar);
             bulk_g2s(&W.mem[0], B.gmem + (uint64_t)g * GROUP, mb, &W.mbar);
             bulk_g2s(&W.cbox[0], P.box[sel] + s0 / PK_CH, cb, &W.mbar);
         }
+        pending = MEM;
 #pragma unroll
         for (int k = 0; k < PK_STAGES; k++) {
-            pending[k] = pend != 0u;
             if (pend) {
                 if (lane == 0) copy_chunk(__ffs(pend) - 1, k);
+                pending |= 1u << k;
                 first |= pend & (0u - pend);
                 pend &= pend - 1u;
             }
         }
-        mpending = true;
-        if (!mbar_wait_bounded(&W.mbar, mparity)) {
+        if (!mbar_wait_bounded(&W.mbar, (parity >> PK_STAGES) & 1u)) {
             abort = true;
             break;
         }
-        mparity ^= 1u;
-        mpending = false;
-        // a group's members belong to one request: its d bounds for the gap filter
-        const float4 GH = W.ghdr;
-        const float d_dn = GH.x, d2u = GH.y;
-        const uint32_t q_first = __float_as_uint(GH.z);
-        const uint32_t count = __float_as_uint(GH.w);
-        // the next tile's descriptor is copied into shared memory during the sweep
+        parity ^= MEM;
+        pending &= ~MEM;
+        // the next tile's entry is copied into shared memory during the sweep
         if (lane == 0 && t_next < ntiles) {
             asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(&W.dnext)),
                          "l"(B.tdesc + t_next)
                          : "memory");
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
-
-        // members of the group: one per lane, their expanded boxes and ranges in registers
-        uint32_t lo = 0, hi = 0, myq = 0;
-        float4 ea = make_float4(0.f, 0.f, 0.f, 0.f), eb = ea;
-        if ((uint32_t)lane < count) {
-            const MemberRec &M = W.mem[lane];
-            myq = M.qi;
-            lo = M.lo;
-            hi = M.hi;
-            if (M.sel != sel) lo = hi = 0;
-            ea = M.ea;
-            eb = M.eb;
+        // the listed chunks this lane's member meets: its range overlaps the chunk and its
+        // expanded box meets the chunk's bounding record
+        uint32_t mc = 0u;
+        if ((uint32_t)lane < __float_as_uint(W.ghdr.w) && W.mem[lane].sel == sel) {
+            const MemberRec M = W.mem[lane];
+            for (uint32_t rem = cand; rem; rem &= rem - 1u) {
+                const uint32_t c = __ffs(rem) - 1;
+                const uint32_t cs = s0 + c * PK_CH, ce = cs + PK_CH;
+                const bool meet = (M.lo < ce) & (M.hi > cs) & filter_box(W.cbox[c], M.ea, M.eb);
+                mc |= (uint32_t)meet << c;
+            }
         }
-        // the two axes of the stage-1 sweep, those on which the array's entries are least likely
-        // to meet the query: time and x for grid cells (a cell holds entries of every time), the
-        // two other axes for a subbin array (its entries overlap the query in the subbin's axis
-        // by construction), y and z for the temporal bins
-        const int dim = sel == SEL_GRID ? 3 : (sel == SEL_X || sel == SEL_T ? 1 : 0);
-        const int dim2 = sel == SEL_GRID ? 0 : (sel == SEL_Z ? 1 : 2);
-        auto comp = [](const float4 &v, int k) {
-            return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
-        };
-        const float fa = comp(ea, dim), fb = comp(eb, dim);
-        const float ga = comp(ea, dim2), gb = comp(eb, dim2);
+        __syncwarp();
 
-        // a candidate that passed the filters joins the exact-test queue
-        auto enqueue = [&](bool p, uint32_t qi, uint32_t pos) {
+        // a candidate that passed the filters joins the exact-test queue; its exact record, a
+        // gather from HBM, is on its way to L2 while it waits there
+        auto enqueue = [&](bool p, uint32_t qi, uint32_t e) {
             const unsigned bm = __ballot_sync(FULL, p);
             if (bm) {
                 if (p) {
                     const uint32_t j = qn + __popc(bm & lt_mask);
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(P.seg + e));
                     W.q_qi[j] = qi;
-                    W.q_pos[j] = pos;
-                    W.q_tile[j] = tw;
-                    W.q_ql[j] = qi - q_first;
+                    W.q_e[j] = e;
+                    W.q_tile[j] = tile;
+                    W.q_ql[j] = qi - __float_as_uint(W.ghdr.z);
                 }
                 qn += __popc(bm);
-                if (qn >= 32) {
-                    __syncwarp();
-                    flush(32);
-                }
             }
         };
 
-        // the listed chunks this lane's member meets: its range overlaps the chunk and its expanded
-        // box meets the chunk's bounding record
-        uint32_t mc = 0u;
-        for (uint32_t rem = cand; rem; rem &= rem - 1u) {
-            const uint32_t c = __ffs(rem) - 1;
-            const uint32_t cs = s0 + c * PK_CH, ce = cs + PK_CH;
-            const bool meet = (lo < ce) & (hi > cs) & filter_box(W.cbox[c], ea, eb);
-            mc |= (uint32_t)meet << c;
-        }
         // chunks to sweep, in order; the first PK_STAGES listed ones were copied already, later
         // ones are copied PK_STAGES sweeps ahead, so of these a chunk no member meets is neither
         // copied nor swept
         const uint32_t need = __reduce_or_sync(FULL, mc);
         uint32_t todo = need | first;
         pend &= need;
-        for (uint32_t k = 0; todo && !abort; k++) {
+        for (uint32_t st = 0; todo; st = st + 1 == PK_STAGES ? 0 : st + 1) {
             const uint32_t c = __ffs(todo) - 1;
             todo &= todo - 1u;
-            const int st = (int)(k % PK_STAGES);
-            if (!mbar_wait_bounded(&W.bar[st], parity[st])) {
+            if (!mbar_wait_bounded(&W.bar[st], (parity >> st) & 1u)) {
                 abort = true;
                 break;
             }
-            parity[st] ^= 1u;
-            pending[st] = false;
-            if (PASS == PASS_COUNT && lane == 0) W.sweep[0]++;
-            const uint32_t cs = s0 + c * PK_CH;
-            const uint32_t cn = min((uint32_t)PK_CH, n_rec - cs);
-            const bool mine = (mc >> c) & 1u;
-            // this lane's own range within the chunk, as bits of the 64 stage slots
-            const uint32_t va = max(lo, cs), vb = min(hi, cs + cn);
-            uint32_t v0 = 0u, v1 = 0u;
-            if (mine && vb > va) {
-                const uint32_t x = va - cs, y = vb - cs;  // 0 <= x < y <= 64
-                v0 = (y >= 32 ? FULL : ((1u << y) - 1u)) & (x >= 32 ? 0u : (FULL << x));
-                v1 = y <= 32 ? 0u : ((y >= 64 ? FULL : ((1u << (y - 32)) - 1u)) &
-                                     (x <= 32 ? FULL : (FULL << (x - 32))));
-            }
-            uint32_t m0 = 0u, m1 = 0u;
-            const unsigned act = __ballot_sync(FULL, (v0 | v1) != 0u);
-            if (!act) {
-                // (a chunk copied ahead of the member tests that no member meets)
-            } else if (__popc(act) <= PK_SPARSE) {
-                if (PASS == PASS_COUNT && lane == 0) W.sweep[2] += __popc(act);
-                // few members meet this chunk: one lane per slot (slots lane and lane + 32), the
-                // members that meet the chunk in turn, their boxes read as broadcasts
-                const bool in0 = (uint32_t)lane < cn, in1 = (uint32_t)lane + 32 < cn;
-                RecF r0 = W.stage[st][lane];
-                RecF r1 = W.stage[st][lane + 32];
-                if (!in0) r0.t0 = INFINITY;  // a slot past the chunk never passes the filter
-                if (!in1) r1.t0 = INFINITY;
-                const uint32_t pos0 = cs + lane, pos1 = cs + 32 + lane;
-                // the (member, slot) pairs that pass the box test are listed in shared memory
-                // (member by member, slot order) and go through the gap bound one per lane, so
-                // that the gap bound and the queue run on full warps
-                uint32_t npl = 0;  // listed pairs (warp-uniform)
-                auto drain = [&]() {
-                    __syncwarp();
-                    for (uint32_t b = 0; b < npl; b += 32) {
-                        bool p = false;
-                        uint32_t mq = 0, slot = 0;
-                        if (b + lane < npl) {
-                            const uint32_t e = W.plist[b + lane];
-                            const MemberRec &M = W.mem[e >> 8];
-                            slot = e & 63u;
-                            mq = M.qi;
-                            p = filter_gap_e(W.stage[st][slot], M.ea, M.eb, d_dn, d2u);
-                        }
-                        enqueue(p, mq, cs + slot);
-                    }
-                    npl = 0;
-                    __syncwarp();
-                };
-                for (unsigned rem = act; rem; rem &= rem - 1u) {
-                    // (a member in act has this tile's array: its range is its own)
-                    const uint32_t m = __ffs(rem) - 1;
-                    const MemberRec &M = W.mem[m];
-                    const float4 mea = M.ea, meb = M.eb;
-                    const uint32_t mlo = M.lo;
-                    const uint32_t w = M.hi - mlo;
-                    const bool p0 = ((pos0 - mlo) < w) & filter_box(r0, mea, meb);
-                    const bool p1 = ((pos1 - mlo) < w) & filter_box(r1, mea, meb);
-                    const unsigned b0 = __ballot_sync(FULL, p0), b1 = __ballot_sync(FULL, p1);
-                    if (!(b0 | b1)) continue;  // (the common case)
-                    if (p0) W.plist[npl + __popc(b0 & lt_mask)] = (m << 8) | (uint32_t)lane;
-                    if (p1)
-                        W.plist[npl + __popc(b0) + __popc(b1 & lt_mask)] =
-                            (m << 8) | (uint32_t)(lane + 32);
-                    npl += __popc(b0) + __popc(b1);
-                    if (npl > PK_PLIST - 64) drain();  // (room for one more member's 64 pairs)
-                }
-                if (npl) drain();
-            } else {
+            parity ^= 1u << st;
+            pending &= ~(1u << st);
+            if (PASS == PASS_COUNT && lane == 0) W.count[0]++;
+            const Chunk &C = W.stage[st];
+            const unsigned act = __ballot_sync(FULL, (mc >> c) & 1u);
+            // what is left of the chunk: members of the per-member pass, listed pairs [b, npl),
+            // survivors of the bitmask pass (none of them when no member meets a chunk that was
+            // copied ahead of the member tests)
+            unsigned rem = act;
+            uint32_t npl = 0, b = 0, m0 = 0u, m1 = 0u;
+            if (__popc(act) > PK_SPARSE) {
+                rem = 0u;
+                if (PASS == PASS_COUNT && lane == 0) W.count[1]++;
                 // stage 1: two axes of every slot against every member (slot i is read at a
                 // warp-uniform address, a shared-memory broadcast); bit i is set when the extents
-                // overlap on both. Four independent accumulators per half keep the OR chains
-                // short.
-                if (PASS == PASS_COUNT && lane == 0) W.sweep[1]++;
-                const float2 *ax = reinterpret_cast<const float2 *>(&W.stage[st][0]) + dim;
-                const float2 *ax2 = reinterpret_cast<const float2 *>(&W.stage[st][0]) + dim2;
-                uint32_t a[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+                // overlap on both. 16 slots at a time and two accumulators: unrolled further, the
+                // loads in flight take the registers of more warps. The two axes are those on
+                // which the array's entries are least likely to meet the query: time and x for
+                // grid cells (a cell holds entries of every time), the two other axes for a subbin
+                // array (its entries overlap the query in the subbin's axis by construction), y
+                // and z for the temporal bins.
+                const uint32_t dim = sel == SEL_GRID ? 3 : (sel == SEL_X || sel == SEL_T ? 1 : 0);
+                const uint32_t dim2 = sel == SEL_GRID ? 0 : (sel == SEL_Z ? 1 : 2);
+                const MemberRec &M = W.mem[lane];
+                const float *ma = reinterpret_cast<const float *>(&M.ea);
+                const float *mb = reinterpret_cast<const float *>(&M.eb);
+                const float fa = ma[dim], fb = mb[dim], ga = ma[dim2], gb = mb[dim2];
+                const float2 *ax = reinterpret_cast<const float2 *>(&C.r[0]) + dim;
+                const float2 *ax2 = reinterpret_cast<const float2 *>(&C.r[0]) + dim2;
+#pragma unroll 1
+                for (int j = 0; j < 4; j++) {
+                    uint32_t a[2] = {0u, 0u};
 #pragma unroll
-                for (int i = 0; i < 64; i++) {
-                    const float2 v = ax[4 * i], u = ax2[4 * i];
-                    if ((v.y >= fa) & (v.x <= fb) & (u.y >= ga) & (u.x <= gb))
-                        a[(i >> 5) * 4 + (i & 3)] |= 1u << (i & 31);
-                }
-                m0 = ((a[0] | a[1]) | (a[2] | a[3])) & v0;
-                m1 = ((a[4] | a[5]) | (a[6] | a[7])) & v1;
-            }
-            // stage 2: the survivors, one per lane per round, through the full box and gap
-            // filters and into the exact-test queue
-            for (;;) {
-                const bool have = (m0 | m1) != 0u;
-                const unsigned hv = __ballot_sync(FULL, have);
-                if (!hv) break;
-                if (PASS == PASS_COUNT && lane == 0) W.sweep[3] += __popc(hv);
-                bool p = false;
-                uint32_t i = 0;
-                if (have) {
-                    if (m0) {
-                        i = __ffs(m0) - 1;
-                        m0 &= m0 - 1u;
-                    } else {
-                        i = 31 + __ffs(m1);
-                        m1 &= m1 - 1u;
+                    for (int i = 0; i < 16; i++) {
+                        const float2 v = ax[64 * j + 4 * i], u = ax2[64 * j + 4 * i];
+                        if ((v.y >= fa) & (v.x <= fb) & (u.y >= ga) & (u.x <= gb))
+                            a[i & 1] |= 1u << i;
                     }
-                    const RecF r = W.stage[st][i];
-                    p = filter_box(r, ea, eb) & filter_gap_e(r, ea, eb, d_dn, d2u);
+                    m0 = (m0 >> 16) | (m1 << 16);  // the 64 bits move down, these join on top
+                    m1 = (m1 >> 16) | ((a[0] | a[1]) << 16);
                 }
-                enqueue(p, myq, cs + i);
+                // this lane's own range within the chunk, as bits of the 64 slots
+                const uint32_t cs = s0 + c * PK_CH;
+                const uint32_t x = max(M.lo, cs) - cs, y = min(M.hi - cs, (uint32_t)PK_CH);
+                if ((act >> lane) & 1u) {
+                    m0 &= (y >= 32 ? FULL : ((1u << y) - 1u)) & (x >= 32 ? 0u : (FULL << x));
+                    m1 &= y <= 32 ? 0u : ((y >= 64 ? FULL : ((1u << (y - 32)) - 1u)) &
+                                          (x <= 32 ? FULL : (FULL << (x - 32))));
+                } else {
+                    m0 = m1 = 0u;
+                }
+            } else if (PASS == PASS_COUNT && lane == 0) {
+                W.count[2] += __popc(act);
+            }
+            for (bool more = true; more;) {
+                while (qn <= PK_QUEUE - 32) {
+                    bool p = false;
+                    uint32_t qi = 0, e = 0;
+                    if (b < npl) {
+                        // the listed pairs go through the gap bound one per lane, so that the gap
+                        // bound and the queue run on full warps
+                        if (b + lane < npl) {
+                            const uint32_t x = W.plist[b + lane];
+                            const MemberRec &M = W.mem[x >> 8];
+                            qi = M.qi;
+                            e = C.id[x & 63u];
+                            p = filter_gap_e(C.r[x & 63u], M.ea, M.eb, W.ghdr.x, W.ghdr.y);
+                        }
+                        b += 32;
+                    } else if (rem) {
+                        // few members meet this chunk: one lane per slot (slots lane and lane +
+                        // 32), the members that meet the chunk in turn, their boxes read as
+                        // broadcasts; the (member, slot) pairs that pass the box test are listed
+                        // in shared memory (member by member, slot order)
+                        __syncwarp();
+                        const uint32_t pos = s0 + c * PK_CH + lane;
+                        const RecF r0 = C.r[lane], r1 = C.r[lane + 32];
+                        npl = b = 0;
+                        // (room for one more member's 64 pairs)
+                        for (; rem && npl <= PK_PLIST - 64; rem &= rem - 1u) {
+                            const uint32_t m = __ffs(rem) - 1;
+                            const MemberRec &M = W.mem[m];
+                            const float4 mea = M.ea, meb = M.eb;
+                            // (a member in act has this tile's array: its range is its own)
+                            const uint32_t off = pos - M.lo, w = M.hi - M.lo;
+                            const bool p0 = (off < w) & filter_box(r0, mea, meb);
+                            const bool p1 = (off + 32 < w) & filter_box(r1, mea, meb);
+                            const unsigned b0 = __ballot_sync(FULL, p0);
+                            const unsigned b1 = __ballot_sync(FULL, p1);
+                            if (!(b0 | b1)) continue;
+                            if (p0)
+                                W.plist[npl + __popc(b0 & lt_mask)] = (m << 8) | (uint32_t)lane;
+                            if (p1)
+                                W.plist[npl + __popc(b0) + __popc(b1 & lt_mask)] =
+                                    (m << 8) | (uint32_t)(lane + 32);
+                            npl += __popc(b0) + __popc(b1);
+                        }
+                        __syncwarp();
+                        continue;
+                    } else {
+                        // stage 2: the bitmasks' survivors, one per lane per round, through the
+                        // full box and gap filters
+                        const bool have = (m0 | m1) != 0u;
+                        const unsigned hv = __ballot_sync(FULL, have);
+                        if (!hv) {
+                            more = false;
+                            break;
+                        }
+                        if (PASS == PASS_COUNT && lane == 0) W.count[3] += __popc(hv);
+                        if (have) {
+                            uint32_t i;
+                            if (m0) {
+                                i = __ffs(m0) - 1;
+                                m0 &= m0 - 1u;
+                            } else {
+                                i = 31 + __ffs(m1);
+                                m1 &= m1 - 1u;
+                            }
+                            const MemberRec &M = W.mem[lane];
+                            const RecF r = C.r[i];
+                            e = C.id[i];
+                            qi = M.qi;
+                            p = filter_box(r, M.ea, M.eb) &
+                                filter_gap_e(r, M.ea, M.eb, W.ghdr.x, W.ghdr.y);
+                        }
+                    }
+                    enqueue(p, qi, e);
+                }
+                if (qn >= 32) qn = pair_flush<PASS>(qn, false);
             }
             __syncwarp();
             if (pend) {
-                const uint32_t cnext = __ffs(pend) - 1;
+                if (lane == 0) copy_chunk(__ffs(pend) - 1, st);
                 pend &= pend - 1u;
-                if (lane == 0) copy_chunk(cnext, st);
-                pending[st] = true;
+                pending |= 1u << st;
             }
         }
+        if (abort) break;
         if (lane == 0) asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
         t = __shfl_sync(FULL, t_next, 0);
         D = W.dnext;
         __syncwarp();  // (read by every lane before the next copy)
     }
-    if (!abort && qn) {
-        __syncwarp();
-        flush(qn);
-    }
+    if (!abort && qn) pair_flush<PASS>(qn, true);
+    // the unused slots of this warp's part hold no hit
+    __syncwarp();
+    if (PASS == PASS_COUNT)
+        for (uint32_t j = W.sc_at + lane; j < W.sc_end; j += 32) B.s_tile[j] = 0xffffffffu;
     if (abort) {
-        if (lane == 0) atomicOr(B.status, DEV_ERR_TIMEOUT);
+        if (lane == 0) {
+            atomicOr(B.status, DEV_ERR_TIMEOUT);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        }
         // let copies still in flight land before the shared memory is released
         for (int st = 0; st < PK_STAGES; st++)
-            if (pending[st]) mbar_wait_bounded(&W.bar[st], parity[st]);
-        if (mpending) mbar_wait_bounded(&W.mbar, mparity);
+            if ((pending >> st) & 1u) mbar_wait_bounded(&W.bar[st], (parity >> st) & 1u);
+        if (pending & MEM) mbar_wait_bounded(&W.mbar, (parity >> PK_STAGES) & 1u);
     }
     if (PASS == PASS_COUNT) {
         // the block's counts are summed in shared memory: one atomic per counter and block
         // (warps finish together, so per-warp atomics on these few addresses would queue)
-        if (lane == 0) {
-            W.sweep[4] = acc_exact;
-            W.sweep[5] = acc_hits;
-        }
         __syncthreads();
         if (threadIdx.x < 6) {
             const WarpSmem *all = reinterpret_cast<const WarpSmem *>(smem_raw);
             unsigned long long v = 0;
-            for (int w = 0; w < PK_WARPS; w++) v += all[w].sweep[threadIdx.x];
+            for (int w = 0; w < PK_WARPS; w++) v += all[w].count[threadIdx.x];
             const int slot = threadIdx.x < 4 ? ST_CHUNKS + (int)threadIdx.x
                                              : (threadIdx.x == 4 ? ST_EXACT : ST_HITS);
             if (v) atomicAdd(&B.stats[slot], v);
@@ -1212,21 +1274,49 @@ __global__ void k_place(PipeBufs b, uint64_t scap, uint64_t tcap, uint64_t rows_
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(b.status, DEV_ERR_OVERFLOW);
         return;
     }
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t t = b.s_tile[i];
-        const uint64_t o = b.tile_off[t] + b.s_rank[i];
-        if (t >= T || o >= b.tile_off[t + 1]) {
-            atomicOr(b.status, DEV_ERR_INTERNAL);
-            continue;
+    // four hits per thread at a time, their loads independent: a hit's tile offset waits for its
+    // tile, and one such chain per thread left HBM idle (978 M hits, 56 B each at least: 23.3 ms
+    // with one, 16.6 ms with four and a grid of several waves, 3.3 TB/s)
+    const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * nth) {
+        uint32_t t[4], rank[4], q[4], e[4];
+        double tin[4], tout[4];
+        uint64_t o[4], end[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint64_t i = i0 + k * nth;
+            t[k] = i < n ? __ldcs(b.s_tile + i) : 0xffffffffu;  // (a slot without a hit)
         }
-        b.out_q[o] = b.s_q[i];
-        b.out_e[o] = b.s_e[i];
-        b.out_tin[o] = b.s_tin[i];
-        b.out_tout[o] = b.s_tout[i];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint64_t i = i0 + k * nth;
+            const bool on = t[k] != 0xffffffffu;
+            const uint32_t tk = on && t[k] < T ? t[k] : 0u;
+            rank[k] = on ? __ldcs(b.s_rank + i) : 0u;
+            q[k] = on ? __ldcs(b.s_q + i) : 0u;
+            e[k] = on ? __ldcs(b.s_e + i) : 0u;
+            tin[k] = on ? __ldcs(b.s_tin + i) : 0.0;
+            tout[k] = on ? __ldcs(b.s_tout + i) : 0.0;
+            o[k] = on ? b.tile_off[tk] : 0ull;
+            end[k] = on ? b.tile_off[tk + 1] : 0ull;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (t[k] == 0xffffffffu) continue;
+            const uint64_t at = o[k] + rank[k];
+            if (t[k] >= T || at >= end[k]) {
+                atomicOr(b.status, DEV_ERR_INTERNAL);
+                continue;
+            }
+            b.out_q[at] = q[k];
+            b.out_e[at] = e[k];
+            b.out_tin[at] = tin[k];
+            b.out_tout[at] = tout[k];
+        }
     }
 }
 
+constexpr size_t PAIR_SMEM = PK_WARPS * sizeof(WarpSmem) + sizeof(PairParams);
 int g_pair_blocks = 0;
 
 ts_status pair_grid(int *blocks)
@@ -1238,7 +1328,7 @@ ts_status pair_grid(int *blocks)
     int dev = 0, sms = 0, per = 0;
     TS_CUDA(cudaGetDevice(&dev));
     TS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int smem = (int)sizeof(WarpSmem) * PK_WARPS;
+    const int smem = (int)PAIR_SMEM;
     TS_CUDA(cudaFuncSetAttribute(k_pair<PASS_COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     TS_CUDA(cudaFuncSetAttribute(k_pair<PASS_WRITE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     TS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<PASS_COUNT>, PK_THREADS, smem));
@@ -1255,18 +1345,15 @@ void fill_pair_params(PairParams &P, const Index *ix, const ReqDesc *reqs, const
     P.reqs = reqs;
     for (int k = 0; k < 3; k++) {
         P.rec[k] = ix->st_rec[k];
-        P.ids[k] = ix->st_ids[k];
         P.box[k] = ix->st_box[k];
         P.len[k] = (uint32_t)ix->st_len[k];
     }
     // ranges over the start-time order cover whole bins: they are swept in the copy in Morton
     // order inside every bin, chunk by chunk with the chunks' bounding records
     P.rec[SEL_T] = ix->trec;
-    P.ids[SEL_T] = ix->tid;
     P.box[SEL_T] = ix->tbox;
     P.len[SEL_T] = (uint32_t)ix->n;
     P.rec[SEL_GRID] = ix->ga_rec;
-    P.ids[SEL_GRID] = ix->ga;
     P.box[SEL_GRID] = ix->gbox;
     P.len[SEL_GRID] = (uint32_t)ix->g_len;
     P.seg = ix->seg;
@@ -1479,7 +1566,7 @@ ts_status pipe_count(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, co
         TS_LAUNCH_PDL(k_tile_desc, dim3(dblk), dim3(TPB), 0, s,
                       c.groups, c.tiles, c.tile, box, b);
         TS_LAUNCH_PDL(k_pair<PASS_COUNT>, dim3(blocks), dim3(PK_THREADS),
-                      sizeof(WarpSmem) * PK_WARPS, s, P);
+                      PAIR_SMEM, s, P);
     }
     return TS_OK;
 }
@@ -1501,11 +1588,11 @@ ts_status pipe_write(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, co
     fill_pair_params(P, ix, reqs, b, c);
     if (c.tiles) {
         if (c.scratch) {
-            TS_LAUNCH_PDL(k_place, dim3(152 * 4), dim3(TPB), 0, s,
+            TS_LAUNCH_PDL(k_place, dim3(152 * 32), dim3(TPB), 0, s,
                           b, c.scratch, c.tiles, c.rows);
         }
         TS_LAUNCH_PDL(k_pair<PASS_WRITE>, dim3(blocks), dim3(PK_THREADS),
-                      sizeof(WarpSmem) * PK_WARPS, s, P);
+                      PAIR_SMEM, s, P);
     }
     return TS_OK;
 }
@@ -1731,8 +1818,12 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     b.tdesc = w.tdesc.as<uint4>();
     b.tile_hits = w.tiles.as<uint32_t>();
     // hits kept by the count pass and placed after the scan (a second sweep when they overflow)
-    c.scratch = std::min<uint64_t>(4 * nq + (1ull << 20), SCRATCH_MAX);
-    TS_CHECK(w.scratch.alloc(32 * c.scratch, s));
+    c.scratch = scratch_slots(std::min<uint64_t>(std::max<uint64_t>(4 * nq + (1ull << 20), 512 * nq),
+                                                 SCRATCH_MAX));
+    if (w.scratch.alloc(32 * c.scratch, s) != TS_OK) {  // (short of memory: sweep twice instead)
+        c.scratch = std::min<uint64_t>(4 * nq + (1ull << 20), SCRATCH_MAX);
+        TS_CHECK(w.scratch.alloc(32 * c.scratch, s));
+    }
     b.s_tile = w.scratch.as<uint32_t>();
     b.s_rank = b.s_tile + c.scratch;
     b.s_q = b.s_rank + c.scratch;

@@ -16,11 +16,11 @@
 
 namespace ts {
 
-constexpr int PK_WARPS = 8;
+constexpr int PK_WARPS = 10;
 constexpr int PK_THREADS = PK_WARPS * 32;
-constexpr int PK_CH = 64;      // records per bulk-copy stage (2 KB): 2 per lane
+constexpr int PK_CH = CHUNK;   // records per bulk-copy stage (2.25 KB): 2 per lane
 constexpr int PK_STAGES = 2;   // chunk stages per warp (copies in flight while one is swept)
-constexpr int PK_QUEUE = 64;   // exact-test queue per warp (drained at 32)
+constexpr int PK_QUEUE = 128;  // exact-test queue per warp (drained at a chunk's end)
 constexpr uint32_t PK_PLIST = 128;  // box-test survivors of a chunk awaiting the gap bound
 constexpr uint32_t PK_MAX_TILES = (1u << 29) - 1;  // tile index bits of a queued candidate
 constexpr int PK_SPARSE = 8;  // chunks met by at most this many members: per-member sweep
@@ -99,6 +99,12 @@ struct PipeCaps {
     uint64_t stall_ns = 0;    // plain searches only, tests of the timeout path (inject_stall)
 };
 constexpr uint64_t SCRATCH_MAX = 1ull << 24;  // rows (32 B each)
+// Slots that keep n hits: the count pass's warps take their parts in advance, so some slots of each
+// stay empty (at most 32, or a third of what it has had, or 256).
+inline uint64_t scratch_slots(uint64_t n)
+{
+    return n + (n / 2 + 100000 < 700000 ? n / 2 + 100000 : 700000);
+}
 
 // Result of one search (device arrays owned by the ts_result handle).
 struct SearchOut {
