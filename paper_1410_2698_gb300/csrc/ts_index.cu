@@ -569,7 +569,7 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     }
 
     // sort by start time (stable: ties in input order)
-    TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, 64, s));
+    TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, 64, s, nullptr, false));
     TS_CHECK(ix->alloc(&ix->seg, n));
     TS_CHECK(ix->alloc(&ix->rec, n));
     TS_CHECK(ix->alloc(&ix->orig, n));
@@ -631,7 +631,7 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
                                             tkeys.as<uint64_t>(), tvals.as<uint32_t>());
         TS_LAUNCHED();
         TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), tvals.as<uint32_t>(), n,
-                                3 * mm.bits + bits_for((uint64_t)ix->m - 1), s));
+                                3 * mm.bits + bits_for((uint64_t)ix->m - 1), s, nullptr, false));
         TS_CHECK(ix->alloc(&ix->trec, (n + CHUNK - 1) / CHUNK));
         TS_CHECK(ix->alloc(&ix->tid, n));
         TS_CUDA(cudaMemcpyAsync(ix->tid, tvals.p, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice,

@@ -243,11 +243,12 @@ ts_status scan_u32_to_u64(const uint32_t *in, uint64_t *out, uint64_t n, cudaStr
 // total does not fit in 32 bits
 ts_status scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *status,
                    cudaStream_t s, const uint32_t *n_dev = nullptr);
-// stable LSD radix sort of (key, value) pairs by the low `bits` bits of the key
+// stable LSD radix sort of (key, value) pairs by the low `bits` bits of the key; without keys_out
+// the keys are left in no particular order
 ts_status radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                         const uint32_t *n_dev = nullptr);
+                         const uint32_t *n_dev = nullptr, bool keys_out = true);
 ts_status radix_sort_u32(uint32_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                         const uint32_t *n_dev = nullptr);
+                         const uint32_t *n_dev = nullptr, bool keys_out = true);
 
 }  // namespace ts
 

@@ -113,7 +113,7 @@ ts_status DevBuf::alloc(size_t nbytes, cudaStream_t stream)
 // ---------------------------------------------------------------------------------------------
 // scan
 // ---------------------------------------------------------------------------------------------
-constexpr int SCAN_THREADS = 256;
+constexpr int SCAN_THREADS = 512;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
@@ -130,23 +130,23 @@ __device__ inline T warp_incl_scan(T v)
 }
 
 // Block-wide exclusive scan of one value per thread; returns the exclusive prefix, *total the sum.
-template <class T>
+template <class T, int THREADS = SCAN_THREADS>
 __device__ inline T block_excl_scan(T v, T *total)
 {
-    __shared__ T warp_sums[SCAN_THREADS / 32 + 1];
+    __shared__ T warp_sums[THREADS / 32 + 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     T incl = warp_incl_scan(v);
     if (lane == 31) warp_sums[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-        T w = lane < SCAN_THREADS / 32 ? warp_sums[lane] : T(0);
+        T w = lane < THREADS / 32 ? warp_sums[lane] : T(0);
         T wi = warp_incl_scan(w);
-        if (lane < SCAN_THREADS / 32) warp_sums[lane] = wi - w;
-        if (lane == SCAN_THREADS / 32 - 1) warp_sums[SCAN_THREADS / 32] = wi;  // total
+        if (lane < THREADS / 32) warp_sums[lane] = wi - w;
+        if (lane == THREADS / 32 - 1) warp_sums[THREADS / 32] = wi;  // total
     }
     __syncthreads();
     T excl = warp_sums[wid] + incl - v;
-    if (total) *total = warp_sums[SCAN_THREADS / 32];
+    if (total) *total = warp_sums[THREADS / 32];
     __syncthreads();
     return excl;
 }
@@ -158,9 +158,20 @@ __device__ __forceinline__ uint64_t dev_count(uint64_t cap, const uint32_t *n_de
     return n_dev ? min(cap, (uint64_t)*n_dev) : cap;
 }
 
-template <class Tin, class Tout>
+// An offset as it is stored: 64 bits as they are, 32 bits checked.
+__device__ __forceinline__ void put_off(uint64_t *out, uint64_t v, uint32_t *) { *out = v; }
+__device__ __forceinline__ void put_off(uint32_t *out, uint64_t v, uint32_t *status)
+{
+    if (v > 0xffffffffull) {
+        atomicOr(status, DEV_ERR_OVERFLOW);
+        v = 0xffffffffull;
+    }
+    *out = (uint32_t)v;
+}
+
+template <class Tin>
 __global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
-                            Tout *sums)
+                            uint64_t *sums)
 {
     pdl_enter();
     const uint64_t n = dev_count(ncap, n_dev);
@@ -169,314 +180,237 @@ __global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev,
         if (threadIdx.x == 0) sums[blockIdx.x] = 0;
         return;
     }
-    Tout acc = 0;
+    uint64_t acc = 0;
+#pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         uint64_t i = base + (uint64_t)k * SCAN_THREADS + threadIdx.x;
-        if (i < n) acc += (Tout)(in[i] & mask);
+        if (i < n) acc += (uint64_t)(in[i] & mask);
     }
-    Tout total;
-    block_excl_scan<Tout>(acc, &total);
+    uint64_t total;
+    block_excl_scan<uint64_t>(acc, &total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// Scan one tile per block with the tile's starting offset taken from `tile_off` (or 0), writing
-// out[i] = exclusive prefix; the block whose tile holds index n writes out[n] = total.
-template <class Tin, class Tout>
-__global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
-                            const Tout *tile_off, Tout *out)
-{
-    pdl_enter();
-    const uint64_t n = dev_count(ncap, n_dev);
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
-    if (base > n) return;
-    Tout v[SCAN_ITEMS];
-    Tout acc = 0;
-    // thread-contiguous items for a stable sequential order within a thread
-    uint64_t tbase = base + (uint64_t)threadIdx.x * SCAN_ITEMS;
-#pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; k++) {
-        uint64_t i = tbase + k;
-        v[k] = i < n ? (Tout)(in[i] & mask) : Tout(0);
-        acc += v[k];
-    }
-    Tout total;
-    Tout pre = block_excl_scan<Tout>(acc, &total);
-    Tout off = (tile_off ? tile_off[blockIdx.x] : Tout(0)) + pre;
-#pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; k++) {
-        uint64_t i = tbase + k;
-        if (i < n) out[i] = off;
-        off += v[k];
-    }
-    if (threadIdx.x == 0 && n < base + SCAN_TILE)
-        out[n] = (tile_off ? tile_off[blockIdx.x] : Tout(0)) + total;
-}
-
-// Second pass of a two-kernel scan: every block first adds up the totals of the tiles before its
-// own (at most SCAN_LOOKBACK of them, read by the whole block), then scans its tile.
+// Scan of one tile per block, out[i] = exclusive prefix; the block whose tile holds index n writes
+// out[n] = total. The tiles before: `tile_off` holds their scanned sums, or `sums` the sums
+// themselves, which every block adds up (at most SCAN_LOOKBACK of them), or neither (one tile).
 constexpr uint64_t SCAN_LOOKBACK = 4096;
 
 template <class Tin, class Tout>
-__global__ void k_tile_scan_lb(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
-                               const Tout *sums, Tout *out)
+__global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
+                            const uint64_t *tile_off, const uint64_t *sums, Tout *out,
+                            uint32_t *status)
 {
     pdl_enter();
     const uint64_t n = dev_count(ncap, n_dev);
     const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
     if (base > n) return;
-    Tout pre = 0;
-    for (uint32_t j = threadIdx.x; j < blockIdx.x; j += SCAN_THREADS) pre += sums[j];
-    Tout before;
-    block_excl_scan<Tout>(pre, &before);
-    Tout v[SCAN_ITEMS];
-    Tout acc = 0;
+    // thread-contiguous items for a stable sequential order within a thread
+    uint64_t v[SCAN_ITEMS], acc = 0;
     const uint64_t tbase = base + (uint64_t)threadIdx.x * SCAN_ITEMS;
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         const uint64_t i = tbase + k;
-        v[k] = i < n ? (Tout)(in[i] & mask) : Tout(0);
+        v[k] = i < n ? (uint64_t)(in[i] & mask) : 0ull;
         acc += v[k];
     }
-    Tout total;
-    Tout off = before + block_excl_scan<Tout>(acc, &total);
+    uint64_t before = tile_off ? tile_off[blockIdx.x] : 0ull;
+    if (sums) {
+        uint64_t pre = 0;
+        for (uint32_t j = threadIdx.x; j < blockIdx.x; j += SCAN_THREADS) pre += sums[j];
+        block_excl_scan<uint64_t>(pre, &before);
+    }
+    uint64_t total;
+    uint64_t off = before + block_excl_scan<uint64_t>(acc, &total);
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; k++) {
         const uint64_t i = tbase + k;
-        if (i < n) out[i] = off;
+        if (i < n) put_off(out + i, off, status);
         off += v[k];
     }
-    if (threadIdx.x == 0 && n < base + SCAN_TILE) out[n] = before + total;
+    if (threadIdx.x == 0 && n < base + SCAN_TILE) put_off(out + n, before + total, status);
 }
 
 // Exclusive scan of n (or *n_dev <= n) values: out[0..n] with out[n] = total. One block per tile
-// of SCAN_TILE values plus one, so that the tile holding index n always exists.
+// of SCAN_TILE values plus one, so that the tile holding index n always exists. 32-bit offsets are
+// written by the scan itself: the 64-bit array and the kernel that narrowed it are gone.
 template <class Tin, class Tout>
 static ts_status scan_impl(const Tin *in, Tout *out, uint64_t n, const uint32_t *n_dev,
-                           cudaStream_t s, Tin mask = ~Tin(0))
+                           cudaStream_t s, Tin mask, uint32_t *status)
 {
     if (n == 0) {
         TS_CUDA(cudaMemsetAsync(out, 0, sizeof(Tout), s));
         return TS_OK;
     }
     const uint64_t nt = n / SCAN_TILE + 1;
-    if (nt == 1) {
-        TS_LAUNCH_PDL(k_tile_scan<Tin, Tout>, dim3(1), dim3(SCAN_THREADS), 0, s,
-                      in, n, n_dev, mask, nullptr, out);
-        return TS_OK;
+    DevBuf sums, offs;
+    if (nt > 1) {
+        TS_CHECK(sums.alloc(sizeof(uint64_t) * nt, s));
+        TS_LAUNCH_PDL(k_tile_sums<Tin>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
+                      in, n, n_dev, mask, sums.as<uint64_t>());
     }
-    DevBuf sums;
-    TS_CHECK(sums.alloc(sizeof(Tout) * nt, s));
-    TS_LAUNCH_PDL(k_tile_sums<Tin, Tout>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                  in, n, n_dev, mask, sums.as<Tout>());
-    if (nt <= SCAN_LOOKBACK) {
-        TS_LAUNCH_PDL(k_tile_scan_lb<Tin, Tout>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                      in, n, n_dev, mask, sums.as<Tout>(), out);
-        return TS_OK;
+    if (nt > SCAN_LOOKBACK) {
+        TS_CHECK(offs.alloc(sizeof(uint64_t) * (nt + 1), s));
+        TS_CHECK((scan_impl<uint64_t, uint64_t>(sums.as<uint64_t>(), offs.as<uint64_t>(), nt,
+                                                nullptr, s, ~0ull, nullptr)));
     }
-    DevBuf offs;
-    TS_CHECK(offs.alloc(sizeof(Tout) * (nt + 1), s));
-    TS_CHECK((scan_impl<Tout, Tout>(sums.as<Tout>(), offs.as<Tout>(), nt, nullptr, s)));
-    TS_LAUNCH_PDL(k_tile_scan<Tin, Tout>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                  in, n, n_dev, mask, offs.as<Tout>(), out);
+    TS_LAUNCH_PDL((k_tile_scan<Tin, Tout>), dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
+                  in, n, n_dev, mask, nt > SCAN_LOOKBACK ? offs.as<uint64_t>() : nullptr,
+                  nt > 1 && nt <= SCAN_LOOKBACK ? sums.as<uint64_t>() : nullptr, out, status);
     return TS_OK;
 }
 
 ts_status scan_u32_to_u64(const uint32_t *in, uint64_t *out, uint64_t n, cudaStream_t s,
                           const uint32_t *n_dev, uint32_t mask)
 {
-    return scan_impl<uint32_t, uint64_t>(in, out, n, n_dev, s, mask);
-}
-
-__global__ void k_narrow_u64(const uint64_t *in, uint32_t *out, uint64_t ncap,
-                             const uint32_t *n_dev, uint32_t *status)
-{
-    pdl_enter();
-    const uint64_t n = dev_count(ncap, n_dev);
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > n) return;
-    uint64_t v = in[i];
-    if (v > 0xffffffffull) {
-        atomicOr(status, DEV_ERR_OVERFLOW);
-        v = 0xffffffffull;
-    }
-    out[i] = (uint32_t)v;
+    return scan_impl<uint32_t, uint64_t>(in, out, n, n_dev, s, mask, nullptr);
 }
 
 ts_status scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *status,
                    cudaStream_t s, const uint32_t *n_dev)
 {
-    DevBuf wide;
-    TS_CHECK(wide.alloc(sizeof(uint64_t) * (n + 1), s));
-    TS_CHECK(scan_u32_to_u64(in, wide.as<uint64_t>(), n, s, n_dev));
-    TS_LAUNCH_PDL(k_narrow_u64, dim3((unsigned)((n + 1 + 255) / 256)), dim3(256), 0, s,
-                  wide.as<uint64_t>(), out, n, n_dev, status);
-    return TS_OK;
+    return scan_impl<uint32_t, uint32_t>(in, out, n, n_dev, s, ~0u, status);
 }
 
 // ---------------------------------------------------------------------------------------------
-// radix sort: LSD, 8-bit digits, 256 threads x 8 keys per block tile. Each pass: per-tile digit
-// histograms (digit-major), an exclusive scan of them, and a stable scatter in which every warp
-// ranks its 256 consecutive keys with __match_any_sync and the block adds the earlier warps'
-// counts.
+// radix sort: LSD, 8-bit digits, 1024 threads x 4 keys per block tile. Each pass: per-tile digit
+// histograms, and a stable scatter in which every warp ranks its 128 consecutive keys with
+// __match_any_sync and the block adds the earlier warps' counts. Up to RS_FUSED_TILES tiles (2M
+// keys) the scatter adds up the histograms itself: four groups of threads, a thread per digit,
+// read them tile by tile, coalesced, while the block's keys arrive. (With 2048 keys a tile and a
+// thread reading a digit's counts of all tiles one after the other, that took 25 of the 31 us of
+// a pass over 300,000 keys.) Above, a scan kernel turns digit-major histograms into offsets.
+// Bound: L2 latency for the sizes of a search's units, HBM for an index's keys.
 // ---------------------------------------------------------------------------------------------
-constexpr int RS_THREADS = 256;
+constexpr int RS_THREADS = 1024;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ITEMS = 8;
+constexpr int RS_ITEMS = 4;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
 constexpr int RS_RADIX = 256;
+constexpr uint32_t RS_FUSED_TILES = 512;
 
-template <class K>
-__global__ void k_rs_hist(const K *keys, uint64_t ncap, const uint32_t *n_dev, int shift,
-                          uint32_t *hist, uint32_t ntiles)
+template <class K, bool FUSED>
+__global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const K *keys, uint64_t ncap,
+                                                        const uint32_t *n_dev, int shift,
+                                                        uint32_t *hist, uint32_t ntiles)
 {
     pdl_enter();
     __shared__ uint32_t h[RS_RADIX];
     const uint64_t n = dev_count(ncap, n_dev);
-    for (int i = threadIdx.x; i < RS_RADIX; i += RS_THREADS) h[i] = 0;
-    __syncthreads();
-    uint64_t base = (uint64_t)blockIdx.x * RS_TILE;
+    const uint64_t base = (uint64_t)blockIdx.x * RS_TILE;
+    if (FUSED && base >= n) return;
+    if (threadIdx.x < RS_RADIX) h[threadIdx.x] = 0;
+    K key[RS_ITEMS];
+#pragma unroll
     for (int k = 0; k < RS_ITEMS; k++) {
-        uint64_t i = base + (uint64_t)k * RS_THREADS + threadIdx.x;
-        if (i < n) atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 0xffu], 1u);
+        const uint64_t i = base + (uint64_t)k * RS_THREADS + threadIdx.x;
+        key[k] = i < n ? keys[i] : K(0);
     }
     __syncthreads();
-    for (int dgt = threadIdx.x; dgt < RS_RADIX; dgt += RS_THREADS)
-        hist[(uint64_t)dgt * ntiles + blockIdx.x] = h[dgt];
+#pragma unroll
+    for (int k = 0; k < RS_ITEMS; k++) {
+        const uint64_t i = base + (uint64_t)k * RS_THREADS + threadIdx.x;
+        const bool ok = i < n;
+        const uint32_t d = (uint32_t)(key[k] >> shift) & 0xffu;
+        // the lanes of a warp often share their digit (the high digits of sorted starts)
+        const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+        if (__all_sync(0xffffffffu, ok && d == d0)) {
+            if ((threadIdx.x & 31) == 0) atomicAdd(&h[d], 32u);
+        } else if (ok) {
+            atomicAdd(&h[d], 1u);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < RS_RADIX) {
+        const uint64_t d = threadIdx.x;
+        hist[FUSED ? (uint64_t)blockIdx.x * RS_RADIX + d : d * ntiles + blockIdx.x] = h[d];
+    }
 }
 
-template <class K>
+// off: the tiles' histograms (FUSED), or the scanned digit-major ones.
+template <class K, bool FUSED>
 __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const K *keys_in, const uint32_t *vals_in,
                                                            K *keys_out, uint32_t *vals_out,
                                                            uint64_t ncap, const uint32_t *n_dev,
-                                                           int shift, const uint64_t *digit_off,
+                                                           int shift, const uint32_t *hist,
+                                                           const uint64_t *digit_off,
                                                            uint32_t ntiles)
 {
     pdl_enter();
     __shared__ uint32_t wcnt[RS_WARPS][RS_RADIX];
+    __shared__ uint32_t part[2][RS_THREADS];
+    __shared__ uint64_t dbase[RS_RADIX];
     const uint64_t n = dev_count(ncap, n_dev);
     if ((uint64_t)blockIdx.x * RS_TILE >= n) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < RS_WARPS * RS_RADIX; i += RS_THREADS) (&wcnt[0][0])[i] = 0;
-    __syncthreads();
     const uint64_t wbase = (uint64_t)blockIdx.x * RS_TILE + (uint64_t)wid * (RS_ITEMS * 32);
     K key[RS_ITEMS];
-    uint32_t val[RS_ITEMS];
-    uint32_t rank[RS_ITEMS];
+    uint32_t val[RS_ITEMS], rank[RS_ITEMS];
+#pragma unroll
+    for (int k = 0; k < RS_ITEMS; k++) {
+        const uint64_t i = wbase + (uint64_t)k * 32 + lane;
+        key[k] = i < n ? keys_in[i] : K(0);
+        val[k] = i < n ? vals_in[i] : 0u;
+    }
+    for (int i = threadIdx.x; i < RS_WARPS * RS_RADIX; i += RS_THREADS) (&wcnt[0][0])[i] = 0;
+    if (FUSED) {
+        const uint32_t nt = (uint32_t)((n + RS_TILE - 1) / RS_TILE);
+        const uint32_t d = threadIdx.x & (RS_RADIX - 1), grp = threadIdx.x / RS_RADIX;
+        uint32_t tot = 0, pre = 0;
+#pragma unroll 8
+        for (uint32_t t = grp; t < nt; t += RS_THREADS / RS_RADIX) {
+            const uint32_t v = hist[(uint64_t)t * RS_RADIX + d];
+            tot += v;
+            pre += t < blockIdx.x ? v : 0u;
+        }
+        part[0][threadIdx.x] = tot;
+        part[1][threadIdx.x] = pre;
+        __syncthreads();
+        tot = pre = 0;
+        if (threadIdx.x < RS_RADIX)
+            for (int g = 0; g < RS_THREADS / RS_RADIX; g++) {
+                tot += part[0][g * RS_RADIX + threadIdx.x];
+                pre += part[1][g * RS_RADIX + threadIdx.x];
+            }
+        const uint32_t base = block_excl_scan<uint32_t, RS_THREADS>(tot, nullptr);
+        if (threadIdx.x < RS_RADIX) dbase[threadIdx.x] = base + pre;
+    } else {
+        if (threadIdx.x < RS_RADIX)
+            dbase[threadIdx.x] = digit_off[(uint64_t)threadIdx.x * ntiles + blockIdx.x];
+        __syncthreads();
+    }
     const uint32_t lt_mask = (1u << lane) - 1u;
 #pragma unroll
     for (int k = 0; k < RS_ITEMS; k++) {
-        uint64_t i = wbase + (uint64_t)k * 32 + lane;
-        bool ok = i < n;
-        key[k] = ok ? keys_in[i] : K(0);
-        val[k] = ok ? vals_in[i] : 0u;
-        uint32_t dgt = ok ? ((uint32_t)(key[k] >> shift) & 0xffu) : 0x100u;
-        uint32_t peers = __match_any_sync(0xffffffffu, dgt);
-        uint32_t before = __popc(peers & lt_mask);
-        uint32_t leader = __ffs(peers) - 1;
+        const bool ok = wbase + (uint64_t)k * 32 + lane < n;
+        const uint32_t dgt = ok ? ((uint32_t)(key[k] >> shift) & 0xffu) : 0x100u;
+        const uint32_t peers = __match_any_sync(0xffffffffu, dgt);
+        const uint32_t leader = __ffs(peers) - 1;
         uint32_t cur = 0;
         if (ok && lane == (int)leader) {
             cur = wcnt[wid][dgt];
             wcnt[wid][dgt] = cur + __popc(peers);
         }
-        cur = __shfl_sync(0xffffffffu, cur, leader);
-        rank[k] = cur + before;
+        rank[k] = __shfl_sync(0xffffffffu, cur, leader) + __popc(peers & lt_mask);
         __syncwarp();
     }
     __syncthreads();
     // exclusive prefix over warps, per digit
-    for (int dgt = threadIdx.x; dgt < RS_RADIX; dgt += RS_THREADS) {
+    if (threadIdx.x < RS_RADIX) {
         uint32_t run = 0;
+#pragma unroll 8
         for (int w = 0; w < RS_WARPS; w++) {
-            uint32_t c = wcnt[w][dgt];
-            wcnt[w][dgt] = run;
+            const uint32_t c = wcnt[w][threadIdx.x];
+            wcnt[w][threadIdx.x] = run;
             run += c;
         }
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < RS_ITEMS; k++) {
-        uint64_t i = wbase + (uint64_t)k * 32 + lane;
-        if (i >= n) continue;
-        uint32_t dgt = (uint32_t)(key[k] >> shift) & 0xffu;
-        uint64_t dst = digit_off[(uint64_t)dgt * ntiles + blockIdx.x] + wcnt[wid][dgt] + rank[k];
-        keys_out[dst] = key[k];
-        vals_out[dst] = val[k];
-    }
-}
-
-// Scatter of one pass that computes its own digit offsets from the per-tile histograms (for at
-// most RS_FUSED_TILES tiles): thread d adds up digit d over all tiles and over the tiles before
-// this block's, and a block scan over the digit totals gives every digit's first position.
-constexpr uint32_t RS_FUSED_TILES = 256;
-
-template <class K>
-__global__ void __launch_bounds__(RS_THREADS) k_rs_scatter_fused(const K *keys_in,
-                                                                 const uint32_t *vals_in,
-                                                                 K *keys_out, uint32_t *vals_out,
-                                                                 uint64_t ncap, const uint32_t *n_dev,
-                                                                 int shift, const uint32_t *hist,
-                                                                 uint32_t ntiles)
-{
-    pdl_enter();
-    __shared__ uint32_t wcnt[RS_WARPS][RS_RADIX];
-    __shared__ uint32_t dbase[RS_RADIX];
-    const uint64_t n = dev_count(ncap, n_dev);
-    if ((uint64_t)blockIdx.x * RS_TILE >= n) return;
-    {
-        const int d = threadIdx.x;  // RS_THREADS == RS_RADIX
-        uint32_t tot = 0, pre = 0;
-        for (uint32_t t = 0; t < ntiles; t++) {
-            const uint32_t v = hist[(uint64_t)d * ntiles + t];
-            tot += v;
-            pre += t < blockIdx.x ? v : 0u;
-        }
-        uint32_t all;
-        const uint32_t base = block_excl_scan<uint32_t>(tot, &all);
-        dbase[d] = base + pre;
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < RS_WARPS * RS_RADIX; i += RS_THREADS) (&wcnt[0][0])[i] = 0;
-    __syncthreads();
-    const uint64_t wbase = (uint64_t)blockIdx.x * RS_TILE + (uint64_t)wid * (RS_ITEMS * 32);
-    K key[RS_ITEMS];
-    uint32_t val[RS_ITEMS];
-    uint32_t rank[RS_ITEMS];
-    const uint32_t lt_mask = (1u << lane) - 1u;
-#pragma unroll
-    for (int k = 0; k < RS_ITEMS; k++) {
-        uint64_t i = wbase + (uint64_t)k * 32 + lane;
-        bool ok = i < n;
-        key[k] = ok ? keys_in[i] : K(0);
-        val[k] = ok ? vals_in[i] : 0u;
-        uint32_t dgt = ok ? ((uint32_t)(key[k] >> shift) & 0xffu) : 0x100u;
-        uint32_t peers = __match_any_sync(0xffffffffu, dgt);
-        uint32_t before = __popc(peers & lt_mask);
-        uint32_t leader = __ffs(peers) - 1;
-        uint32_t cur = 0;
-        if (ok && lane == (int)leader) {
-            cur = wcnt[wid][dgt];
-            wcnt[wid][dgt] = cur + __popc(peers);
-        }
-        cur = __shfl_sync(0xffffffffu, cur, leader);
-        rank[k] = cur + before;
-        __syncwarp();
-    }
-    __syncthreads();
-    for (int dgt = threadIdx.x; dgt < RS_RADIX; dgt += RS_THREADS) {
-        uint32_t run = 0;
-        for (int w = 0; w < RS_WARPS; w++) {
-            uint32_t c = wcnt[w][dgt];
-            wcnt[w][dgt] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < RS_ITEMS; k++) {
-        uint64_t i = wbase + (uint64_t)k * 32 + lane;
-        if (i >= n) continue;
-        uint32_t dgt = (uint32_t)(key[k] >> shift) & 0xffu;
-        uint64_t dst = (uint64_t)dbase[dgt] + wcnt[wid][dgt] + rank[k];
+        if (wbase + (uint64_t)k * 32 + lane >= n) continue;
+        const uint32_t dgt = (uint32_t)(key[k] >> shift) & 0xffu;
+        const uint64_t dst = dbase[dgt] + wcnt[wid][dgt] + rank[k];
         keys_out[dst] = key[k];
         vals_out[dst] = val[k];
     }
@@ -490,14 +424,14 @@ __global__ void k_copy_kv(const K *ks, const uint32_t *vs, K *kd, uint32_t *vd, 
     const uint64_t n = dev_count(ncap, n_dev);
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        kd[i] = ks[i];
+        if (kd) kd[i] = ks[i];
         vd[i] = vs[i];
     }
 }
 
 template <class K>
 static ts_status radix_sort_impl(K *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                                 const uint32_t *n_dev)
+                                 const uint32_t *n_dev, bool keys_out)
 {
     if (n <= 1 || bits <= 0) return TS_OK;
     uint32_t ntiles = (uint32_t)((n + RS_TILE - 1) / RS_TILE);
@@ -506,48 +440,46 @@ static ts_status radix_sort_impl(K *keys, uint32_t *vals, uint64_t n, int bits, 
     TS_CHECK(vb.alloc(sizeof(uint32_t) * n, s));
     uint64_t nh = (uint64_t)RS_RADIX * ntiles;
     TS_CHECK(hist.alloc(sizeof(uint32_t) * nh, s));
-    const bool fused = ntiles <= RS_FUSED_TILES && n < (1ull << 32);
+    const bool fused = ntiles <= RS_FUSED_TILES;
     if (!fused) TS_CHECK(off.alloc(sizeof(uint64_t) * (nh + 1), s));
     K *ka = keys, *kbp = kb.as<K>();
     uint32_t *va = vals, *vbp = vb.as<uint32_t>();
     int passes = (bits + 7) / 8;
     for (int p = 0; p < passes; p++) {
         int shift = 8 * p;
-        TS_LAUNCH_PDL(k_rs_hist<K>, dim3(ntiles), dim3(RS_THREADS), 0, s, ka, n, n_dev, shift,
-                      hist.as<uint32_t>(), ntiles);
         if (fused) {
-            TS_LAUNCH_PDL(k_rs_scatter_fused<K>, dim3(ntiles), dim3(RS_THREADS), 0, s, ka, va, kbp,
-                          vbp, n, n_dev, shift, hist.as<uint32_t>(), ntiles);
+            TS_LAUNCH_PDL((k_rs_hist<K, true>), dim3(ntiles), dim3(RS_THREADS), 0, s, ka, n, n_dev,
+                          shift, hist.as<uint32_t>(), ntiles);
+            TS_LAUNCH_PDL((k_rs_scatter<K, true>), dim3(ntiles), dim3(RS_THREADS), 0, s, ka, va,
+                          kbp, vbp, n, n_dev, shift, hist.as<uint32_t>(), nullptr, ntiles);
         } else {
+            TS_LAUNCH_PDL((k_rs_hist<K, false>), dim3(ntiles), dim3(RS_THREADS), 0, s, ka, n, n_dev,
+                          shift, hist.as<uint32_t>(), ntiles);
             TS_CHECK(scan_u32_to_u64(hist.as<uint32_t>(), off.as<uint64_t>(), nh, s));
-            TS_LAUNCH_PDL(k_rs_scatter<K>, dim3(ntiles), dim3(RS_THREADS), 0, s, ka, va, kbp, vbp,
-                          n, n_dev, shift, off.as<uint64_t>(), ntiles);
+            TS_LAUNCH_PDL((k_rs_scatter<K, false>), dim3(ntiles), dim3(RS_THREADS), 0, s, ka, va,
+                          kbp, vbp, n, n_dev, shift, nullptr, off.as<uint64_t>(), ntiles);
         }
         K *tk = ka; ka = kbp; kbp = tk;
         uint32_t *tv = va; va = vbp; vbp = tv;
     }
     if (ka != keys) {
-        if (n_dev) {
-            const unsigned cb = (unsigned)std::min<uint64_t>((n + 255) / 256, 152 * 8);
-            TS_LAUNCH_PDL(k_copy_kv<K>, dim3(cb), dim3(256), 0, s, ka, va, keys, vals, n, n_dev);
-        } else {
-            TS_CUDA(cudaMemcpyAsync(keys, ka, sizeof(K) * n, cudaMemcpyDeviceToDevice, s));
-            TS_CUDA(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
-        }
+        const unsigned cb = (unsigned)std::min<uint64_t>((n + 255) / 256, 152 * 8);
+        TS_LAUNCH_PDL(k_copy_kv<K>, dim3(cb), dim3(256), 0, s, ka, va, keys_out ? keys : nullptr,
+                      vals, n, n_dev);
     }
     return TS_OK;
 }
 
 ts_status radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                         const uint32_t *n_dev)
+                         const uint32_t *n_dev, bool keys_out)
 {
-    return radix_sort_impl<uint64_t>(keys, vals, n, bits, s, n_dev);
+    return radix_sort_impl<uint64_t>(keys, vals, n, bits, s, n_dev, keys_out);
 }
 
 ts_status radix_sort_u32(uint32_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                         const uint32_t *n_dev)
+                         const uint32_t *n_dev, bool keys_out)
 {
-    return radix_sort_impl<uint32_t>(keys, vals, n, bits, s, n_dev);
+    return radix_sort_impl<uint32_t>(keys, vals, n, bits, s, n_dev, keys_out);
 }
 
 }  // namespace ts

@@ -1535,7 +1535,7 @@ ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const 
     const KeyFmt f = key_fmt(ix, c.nreq);
     const int bits =
         3 * f.morton + f.lo_bits + f.sel_bits + bits_for(c.nreq > 1 ? c.nreq - 1 : 0) + 1;
-    TS_CHECK(radix_sort_u64(b.keys, b.vals, c.units, bits, s, b.hdr + HDR_NU));
+    TS_CHECK(radix_sort_u64(b.keys, b.vals, c.units, bits, s, b.hdr + HDR_NU, false));
     TS_LAUNCH_PDL(k_req_scan, dim3(1), dim3(32), 0, s,
                   nreq, b);
     const unsigned gblk = (unsigned)std::min<uint64_t>((c.groups * 32 + TPB - 1) / TPB, 152 * 16);
