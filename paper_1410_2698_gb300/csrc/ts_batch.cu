@@ -67,21 +67,6 @@ __global__ void k_req_rows(const uint32_t *run, uint32_t nreq_cap, uint64_t tcap
     if (threadIdx.x == 0) out->status = b.status[0];
 }
 
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-// Carves one device allocation into the plan's buffers.
-struct Carver {
-    size_t off = 0;
-    unsigned char *base = nullptr;
-    template <class T>
-    T *take(uint64_t count)
-    {
-        size_t at = off;
-        off += align256(sizeof(T) * (count ? count : 1));
-        return base ? reinterpret_cast<T *>(base + at) : nullptr;
-    }
-};
-
 }  // namespace
 
 // Layout of the device memory and pointers of a plan (the same code sizes and carves).
@@ -150,8 +135,6 @@ void destroy_plan(BatchPlan *p)
     if (p->dmem) cudaFree(p->dmem);
     if (p->hmem) cudaFreeHost(p->hmem);
     if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
-    for (int e = 0; e < 4; e++)
-        if (p->ev[e]) cudaEventDestroy(p->ev[e]);
     if (p->done) cudaEventDestroy(p->done);
     p->magic = 0;
     delete p;
@@ -237,7 +220,6 @@ ts_status create_plan(const Index *ix, const ts_batch_params *prm, cudaStream_t 
     }
     TS_CUDA(cudaMemsetAsync(p->dmem, 0, p->dbytes, p->stream));
     TS_CUDA(cudaStreamSynchronize(p->stream));
-    for (int e = 0; e < 4; e++) TS_CUDA(cudaEventCreate(&p->ev[e]));
     TS_CUDA(cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming));
     *out = p.release();
     return TS_OK;
@@ -309,18 +291,6 @@ static ts_status stage_requests(BatchPlan *p, uint32_t nreq, const ts_segments *
 
 // Enqueue the run (no host synchronisation; graph-capturable). With write = false the run stops
 // after the scan (one-shot batches size their rows first).
-// Records a timing event; inside a stream capture the event becomes an event-record node of the
-// graph (cudaEventRecordExternal), so that replays time the passes too.
-static cudaError_t record_ev(cudaEvent_t e, cudaStream_t s)
-{
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaError_t ce = cudaStreamIsCapturing(s, &cs);
-    if (ce != cudaSuccess) return ce;
-    return cs == cudaStreamCaptureStatusActive
-               ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal)
-               : cudaEventRecord(e, s);
-}
-
 static ts_status enqueue_run(BatchPlan *p, cudaStream_t s, bool write)
 {
     const PipeCaps &k = p->caps;
@@ -341,15 +311,11 @@ static ts_status enqueue_run(BatchPlan *p, cudaStream_t s, bool write)
         TS_CHECK(pipe_grid_units(p->ix, k.nq, b, k, s));
     }
     TS_CHECK(pipe_group(p->ix, p->d_reqs, k.nreq, b, k, false, s));
-    TS_CUDA(record_ev(p->ev[0], s));
     TS_CHECK(pipe_count(p->ix, p->d_reqs, b, k, s));
-    TS_CUDA(record_ev(p->ev[1], s));
     TS_CHECK(pipe_scan_rows(b, k, s));
     if (write) {
-        TS_CUDA(record_ev(p->ev[2], s));
-        TS_CHECK(pipe_write(p->ix, p->d_reqs, b, k, s));
-        TS_CUDA(record_ev(p->ev[3], s));
-    }
+            TS_CHECK(pipe_write(p->ix, p->d_reqs, b, k, s));
+        }
     TS_LAUNCH_PDL(k_req_rows, dim3(1), dim3(256), 0, s,
                   p->d_run, k.nreq, k.tiles, b, p->dh_row0, p->dh_out);
     return TS_OK;
@@ -408,6 +374,8 @@ static void fill_stats(const BatchOut *o, ts_search_stats *s)
     s->n_dense = o->stats[ST_DENSE];
     s->n_sparse = o->stats[ST_SPARSE];
     s->n_stage2 = o->stats[ST_STAGE2];
+    s->ms_count_pass = stamp_ms(o->stats[ST_CNT0], o->stats[ST_CNT1]);
+    s->ms_write_pass = stamp_ms(o->stats[ST_WR0], o->stats[ST_WR1]);
 }
 
 ts_status plan_wait(BatchPlan *p, ts_batch_status *out)
@@ -426,10 +394,6 @@ ts_status plan_wait(BatchPlan *p, ts_batch_status *out)
     bs.overflow = (st & DEV_ERR_OVERFLOW) ? 1 : 0;
     fill_stats(p->h_out, &bs.stats);
     bs.stats.n_queries = p->h_run[0];
-    float ms = 0.f;
-    if (cudaEventElapsedTime(&ms, p->ev[0], p->ev[1]) == cudaSuccess) bs.stats.ms_count_pass = ms;
-    if (cudaEventElapsedTime(&ms, p->ev[2], p->ev[3]) == cudaSuccess) bs.stats.ms_write_pass = ms;
-    cudaGetLastError();  // a run without a write pass leaves ev[2..3] unrecorded
     if (out) *out = bs;
     if (st & ~DEV_ERR_OVERFLOW) return read_dev_status(st & ~DEV_ERR_OVERFLOW);
     return TS_OK;

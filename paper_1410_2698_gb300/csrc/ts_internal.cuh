@@ -83,7 +83,9 @@ enum : int {
     // visits of the sparse path, survivors of the bitmask given the full FP32 filters
     ST_CHUNKS = 8, ST_DENSE = 9, ST_SPARSE = 10, ST_STAGE2 = 11,
     ST_LOST = 12,  // some hit found no slot of the scratch
-    ST_NSLOTS = 13
+    // device clock (ns): count pass begun and ended, write pass begun and ended
+    ST_CNT0 = 13, ST_CNT1 = 14, ST_WR0 = 15, ST_WR1 = 16,
+    ST_NSLOTS = 17
 };
 
 // ---------------------------------------------------------------------------------------------

@@ -416,6 +416,92 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const K *keys_in, con
     }
 }
 
+// The whole sort of up to RS_SMALL keys in one block, pass by pass through shared memory (two
+// launches and two rounds through L2 a pass cost 5 us each on a few keys).
+constexpr int RS_SMALL_ITEMS = 2;
+constexpr int RS_SMALL = RS_THREADS * RS_SMALL_ITEMS;
+
+template <class K>
+__global__ void __launch_bounds__(RS_THREADS) k_rs_small(K *keys, uint32_t *vals, uint64_t ncap,
+                                                         const uint32_t *n_dev, int passes)
+{
+    pdl_enter();
+    __shared__ K skey[RS_SMALL];
+    __shared__ uint32_t sval[RS_SMALL];
+    __shared__ uint16_t wcnt[RS_WARPS][RS_RADIX];
+    __shared__ uint32_t dbase[RS_RADIX];
+    const uint32_t n = (uint32_t)dev_count(ncap, n_dev);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t at = wid * (RS_SMALL_ITEMS * 32) + lane;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    K key[RS_SMALL_ITEMS];
+    uint32_t val[RS_SMALL_ITEMS], rank[RS_SMALL_ITEMS];
+#pragma unroll
+    for (int k = 0; k < RS_SMALL_ITEMS; k++) {
+        const uint32_t i = at + k * 32;
+        key[k] = i < n ? keys[i] : K(0);
+        val[k] = i < n ? vals[i] : 0u;
+    }
+    for (int p = 0; p < passes; p++) {
+        for (int i = threadIdx.x; i < RS_WARPS * RS_RADIX / 2; i += RS_THREADS)
+            reinterpret_cast<uint32_t *>(&wcnt[0][0])[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < RS_SMALL_ITEMS; k++) {
+            const bool ok = at + k * 32 < n;
+            const uint32_t dgt = ok ? ((uint32_t)(key[k] >> (8 * p)) & 0xffu) : 0x100u;
+            const uint32_t peers = __match_any_sync(0xffffffffu, dgt);
+            const uint32_t leader = __ffs(peers) - 1;
+            uint32_t cur = 0;
+            if (ok && lane == (int)leader) {
+                cur = wcnt[wid][dgt];
+                wcnt[wid][dgt] = (uint16_t)(cur + __popc(peers));
+            }
+            rank[k] = __shfl_sync(0xffffffffu, cur, leader) + __popc(peers & lt_mask);
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t run = 0;
+        if (threadIdx.x < RS_RADIX) {
+#pragma unroll 8
+            for (int w = 0; w < RS_WARPS; w++) {
+                const uint32_t c = wcnt[w][threadIdx.x];
+                wcnt[w][threadIdx.x] = (uint16_t)run;
+                run += c;
+            }
+        }
+        const uint32_t base = block_excl_scan<uint32_t, RS_THREADS>(run, nullptr);
+        if (threadIdx.x < RS_RADIX) dbase[threadIdx.x] = base;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < RS_SMALL_ITEMS; k++) {
+            if (at + k * 32 >= n) continue;
+            const uint32_t dgt = (uint32_t)(key[k] >> (8 * p)) & 0xffu;
+            const uint32_t dst = dbase[dgt] + wcnt[wid][dgt] + rank[k];
+            skey[dst] = key[k];
+            sval[dst] = val[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < RS_SMALL_ITEMS; k++) {
+            const uint32_t i = at + k * 32;
+            if (i < n) {
+                key[k] = skey[i];
+                val[k] = sval[i];
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < RS_SMALL_ITEMS; k++) {
+        const uint32_t i = at + k * 32;
+        if (i < n) {
+            keys[i] = key[k];
+            vals[i] = val[k];
+        }
+    }
+}
+
 template <class K>
 __global__ void k_copy_kv(const K *ks, const uint32_t *vs, K *kd, uint32_t *vd, uint64_t ncap,
                           const uint32_t *n_dev)
@@ -434,6 +520,11 @@ static ts_status radix_sort_impl(K *keys, uint32_t *vals, uint64_t n, int bits, 
                                  const uint32_t *n_dev, bool keys_out)
 {
     if (n <= 1 || bits <= 0) return TS_OK;
+    if (n <= RS_SMALL) {
+        TS_LAUNCH_PDL(k_rs_small<K>, dim3(1), dim3(RS_THREADS), 0, s, keys, vals, n, n_dev,
+                      (bits + 7) / 8);
+        return TS_OK;
+    }
     uint32_t ntiles = (uint32_t)((n + RS_TILE - 1) / RS_TILE);
     DevBuf kb, vb, hist, off;
     TS_CHECK(kb.alloc(sizeof(K) * n, s));

@@ -28,6 +28,8 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cstddef>
+#include <mutex>
 #include <vector>
 
 #include "ts_device.cuh"
@@ -449,6 +451,7 @@ __global__ void k_grid_units(uint64_t nqcap, uint64_t ucap, KeyFmt kf, uint32_t 
 // groups
 // ---------------------------------------------------------------------------------------------
 // Per request: unit starts (exclusive scan of its unit count) and group starts (ceil(units/32)).
+// (With one request k_groups needs neither.)
 __global__ void k_req_scan(uint32_t nreq_cap, PipeBufs b)
 {
     pdl_enter();
@@ -482,7 +485,17 @@ __global__ void k_groups(uint32_t nreq_cap, uint64_t gcap, uint32_t tile, const 
     // of their boxes, against which k_tile_desc tests the chunks' bounding records)
     const unsigned FULL = 0xffffffffu;
     const uint32_t nreq = b.run ? min(b.run[1], nreq_cap) : nreq_cap;
-    const uint32_t G = b.hdr[HDR_G];
+    uint32_t G = b.hdr[HDR_G];
+    if (nreq_cap == 1) {  // (what k_req_scan finds for several)
+        const uint32_t nu = nreq ? b.req_units[0] : 0u;
+        G = (nu + GROUP - 1) / GROUP;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            b.gstart[0] = 0;
+            b.gstart[1] = G;
+            b.hdr[HDR_U] = nu;
+            b.hdr[HDR_G] = G;
+        }
+    }
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     unsigned long long n_cand = 0;  // candidates of this lane's members
@@ -492,14 +505,18 @@ __global__ void k_groups(uint32_t nreq_cap, uint64_t gcap, uint32_t tile, const 
             if (lane == 0) b.ntiles[g] = 0;
             continue;
         }
-        uint32_t lo = 0, hi = nreq;  // last r with gstart[r] <= g
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) / 2;
-            if (b.gstart[mid] <= g) lo = mid; else hi = mid;
+        uint32_t r = 0, first = GROUP * (uint32_t)g, end = b.req_units[0];
+        if (nreq_cap > 1) {
+            uint32_t lo = 0, hi = nreq;  // last r with gstart[r] <= g
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) / 2;
+                if (b.gstart[mid] <= g) lo = mid; else hi = mid;
+            }
+            r = lo;
+            first = b.ustart[r] + GROUP * ((uint32_t)g - b.gstart[r]);
+            end = b.ustart[r] + b.req_units[r];
         }
-        const uint32_t r = lo;
-        const uint32_t first = b.ustart[r] + GROUP * ((uint32_t)g - b.gstart[r]);
-        const uint32_t end = min(first + GROUP, b.ustart[r] + b.req_units[r]);
+        end = min(first + GROUP, end);
         const uint32_t n = end - first;
         if (lane == 0) {
             b.g_first[g] = first;
@@ -638,6 +655,7 @@ __global__ void k_tile_desc(uint64_t gcap, uint64_t tcap, uint32_t tile, ArrayPt
                             PipeBufs b)
 {
     pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.stats[ST_CNT0] = globaltimer_ns();
     const uint32_t G = b.hdr[HDR_G];
     const uint64_t T = b.tile_base[min((uint64_t)G, gcap)];
     if (blockIdx.x == 0 && threadIdx.x == 0) {  // the run header's tile count (as k_hdr)
@@ -965,6 +983,8 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
     uint32_t parity = 0u, pending = 0u;
     constexpr uint32_t MEM = 1u << PK_STAGES;
     bool abort = false;
+    if (PASS == PASS_WRITE && !P.scap && blockIdx.x == 0 && threadIdx.x == 0)
+        B.stats[ST_WR0] = globaltimer_ns();
     if (P.stall_ns && blockIdx.x == 0 && wid == 0)
         abort = !mbar_wait_bounded(&W.xbar, 0u, P.stall_ns);  // (never arrived on: times out)
 
@@ -1245,10 +1265,12 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
             if ((pending >> st) & 1u) mbar_wait_bounded(&W.bar[st], (parity >> st) & 1u);
         if (pending & MEM) mbar_wait_bounded(&W.mbar, (parity >> PK_STAGES) & 1u);
     }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        atomicMax(&B.stats[PASS == PASS_COUNT ? ST_CNT1 : ST_WR1], (unsigned long long)globaltimer_ns());
     if (PASS == PASS_COUNT) {
         // the block's counts are summed in shared memory: one atomic per counter and block
         // (warps finish together, so per-warp atomics on these few addresses would queue)
-        __syncthreads();
         if (threadIdx.x < 6) {
             const WarpSmem *all = reinterpret_cast<const WarpSmem *>(smem_raw);
             unsigned long long v = 0;
@@ -1267,6 +1289,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
 __global__ void k_place(PipeBufs b, uint64_t scap, uint64_t tcap, uint64_t rows_cap)
 {
     pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.stats[ST_WR0] = globaltimer_ns();
     const unsigned long long n = min((unsigned long long)scap, b.stats[ST_SCRATCH]);
     const uint64_t T = (uint64_t)b.hdr[HDR_T_LO] | ((uint64_t)b.hdr[HDR_T_HI] << 32);
     if (T > tcap || T > PK_MAX_TILES) return;  // overflow already flagged
@@ -1367,28 +1390,6 @@ void fill_pair_params(PairParams &P, const Index *ix, const ReqDesc *reqs, const
 
 // A stall requested for the next count pass (tests of the timeout path), taken by that launch.
 std::atomic<uint64_t> g_stall_ns{0};
-
-// Two CUDA events bracketing one kernel launch on its stream.
-struct EventPair {
-    cudaEvent_t a = nullptr, b = nullptr;
-    ts_status create()
-    {
-        TS_CUDA(cudaEventCreate(&a));
-        TS_CUDA(cudaEventCreate(&b));
-        return TS_OK;
-    }
-    double ms() const
-    {
-        float v = 0.f;
-        if (a && b && cudaEventElapsedTime(&v, a, b) == cudaSuccess) return (double)v;
-        return 0.0;
-    }
-    ~EventPair()
-    {
-        if (a) cudaEventDestroy(a);
-        if (b) cudaEventDestroy(b);
-    }
-};
 
 // Smallest float >= x (host).
 float float_up(double x)
@@ -1536,8 +1537,10 @@ ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const 
     const int bits =
         3 * f.morton + f.lo_bits + f.sel_bits + bits_for(c.nreq > 1 ? c.nreq - 1 : 0) + 1;
     TS_CHECK(radix_sort_u64(b.keys, b.vals, c.units, bits, s, b.hdr + HDR_NU, false));
-    TS_LAUNCH_PDL(k_req_scan, dim3(1), dim3(32), 0, s,
-                  nreq, b);
+    if (nreq > 1) {
+        TS_LAUNCH_PDL(k_req_scan, dim3(1), dim3(32), 0, s,
+                      nreq, b);
+    }
     const unsigned gblk = (unsigned)std::min<uint64_t>((c.groups * 32 + TPB - 1) / TPB, 152 * 16);
     TS_LAUNCH_PDL(k_groups, dim3(gblk), dim3(TPB), 0, s,
                   nreq, c.groups, c.tile, reqs, b);
@@ -1759,12 +1762,20 @@ ts_status plain_prepare(const Index *ix, const double *const cols[8], uint64_t n
     return TS_OK;
 }
 
+void fill_stats(const unsigned long long *h, ts_search_stats *st);
+
 ts_status copy_stats(const PipeBufs &b, cudaStream_t s, ts_search_stats *st, uint32_t *status)
 {
     unsigned long long h[ST_NSLOTS];
     TS_CUDA(cudaMemcpyAsync(h, b.stats, sizeof(h), cudaMemcpyDeviceToHost, s));
     TS_CUDA(cudaMemcpyAsync(status, b.status, 4, cudaMemcpyDeviceToHost, s));
     TS_CUDA(cudaStreamSynchronize(s));
+    fill_stats(h, st);
+    return TS_OK;
+}
+
+void fill_stats(const unsigned long long *h, ts_search_stats *st)
+{
     st->n_qsegs = h[ST_QSEGS];
     st->n_tests = h[ST_TESTS];
     st->n_exact = h[ST_EXACT];
@@ -1776,6 +1787,294 @@ ts_status copy_stats(const PipeBufs &b, cudaStream_t s, ts_search_stats *st, uin
     st->n_dense = h[ST_DENSE];
     st->n_sparse = h[ST_SPARSE];
     st->n_stage2 = h[ST_STAGE2];
+    st->ms_count_pass = stamp_ms(h[ST_CNT0], h[ST_CNT1]);
+    st->ms_write_pass = stamp_ms(h[ST_WR0], h[ST_WR1]);
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------------------------
+// a search in one go: every kernel enqueued at once on guessed capacities, one wait
+// ---------------------------------------------------------------------------------------------
+namespace {
+
+constexpr uint64_t ONE_GO_QUERIES = 1ull << 16;  // above, the kernels dwarf the waits
+constexpr uint64_t ONE_GO_ROWS = 1ull << 16;     // rows a result may have room for unasked
+constexpr uint64_t STAGE_QUERIES = 1024;         // host queries read in place from pinned memory
+
+// What the host reads after the wait.
+struct PlainOut {
+    uint32_t hdr[8];
+    unsigned long long stats[ST_NSLOTS];
+    unsigned long long total;
+    uint32_t status, units;
+};
+
+// Pinned, mapped memory of one search in flight: its outcome and its small host query set.
+struct HostSlot {
+    PlainOut out;
+    alignas(256) double stage[8 * STAGE_QUERIES];
+};
+
+// A fixed number of slots for the searches in flight, allocated once; a search that finds none
+// free takes the stepwise path.
+class SlotPool {
+public:
+    HostSlot *take()
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        if (!base_ && !failed_) {
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, sizeof(HostSlot) * SLOTS,
+                              cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
+                base_ = static_cast<HostSlot *>(p);
+            } else {
+                cudaGetLastError();
+                failed_ = true;
+            }
+        }
+        for (int k = 0; base_ && k < SLOTS; k++)
+            if (!((used_ >> k) & 1u)) {
+                used_ |= 1u << k;
+                return base_ + k;
+            }
+        return nullptr;
+    }
+    void give(HostSlot *h)
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        used_ &= ~(1u << (h - base_));
+    }
+
+private:
+    static constexpr int SLOTS = 16;
+    std::mutex mu_;
+    HostSlot *base_ = nullptr;
+    uint32_t used_ = 0;
+    bool failed_ = false;
+};
+SlotPool g_slots;
+
+__global__ void k_plain_start(ReqDesc rd, ReqDesc *reqs, PipeBufs b)
+{
+    pdl_enter();
+    const uint32_t t = threadIdx.x;
+    if (t < 8) b.hdr[t] = 0;
+    if (t < ST_NSLOTS) b.stats[t] = 0;
+    if (t < 3) b.counters[t] = 0;
+    if (t == 0) {
+        *b.status = 0;
+        b.req_units[0] = 0;
+        *reqs = rd;
+    }
+}
+
+__global__ void k_plain_out(uint64_t nq, uint64_t tcap, PipeBufs b, PlainOut *out)
+{
+    pdl_enter();
+    const uint32_t t = threadIdx.x;
+    const uint64_t T = (uint64_t)b.hdr[HDR_T_LO] | ((uint64_t)b.hdr[HDR_T_HI] << 32);
+    if (t < 8) out->hdr[t] = b.hdr[t];
+    if (t < ST_NSLOTS) out->stats[t] = b.stats[t];
+    if (t == 0) {
+        out->total = T <= tcap ? b.tile_off[T] : 0ull;
+        out->status = *b.status;
+        out->units = b.quoff ? b.quoff[nq] : 0u;
+    }
+}
+
+void plain_layout(Carver &k, const PipeCaps &c, bool grid, PipeBufs &b, ReqDesc **reqs)
+{
+    *reqs = k.take<ReqDesc>(1);
+    b.hdr = k.take<uint32_t>(8);
+    b.stats = k.take<unsigned long long>(ST_NSLOTS);
+    b.status = k.take<uint32_t>(4);
+    b.counters = b.status + 1;
+    b.req_units = k.take<uint32_t>(8);
+    b.ustart = b.req_units + 1;
+    b.req_groups = b.req_units + 3;
+    b.gstart = b.req_units + 4;
+    b.qd = k.take<QueryD>(c.nq);
+    b.qf = k.take<float4>(2 * c.nq);
+    b.qreq = k.take<uint32_t>(c.nq);
+    b.qcell = grid ? k.take<uint32_t>(2 * c.nq) : nullptr;
+    b.qnu = grid ? k.take<uint32_t>(c.nq) : nullptr;
+    b.quoff = grid ? k.take<uint32_t>(c.nq + 1) : nullptr;
+    b.u_q = k.take<uint32_t>(c.units);
+    b.u_lo = k.take<uint32_t>(c.units);
+    b.u_hi = k.take<uint32_t>(c.units);
+    b.u_sel = k.take<uint32_t>(c.units);
+    b.keys = k.take<uint64_t>(c.units);
+    b.vals = k.take<uint32_t>(c.units);
+    b.g_first = k.take<uint32_t>(c.groups);
+    b.g_count = k.take<uint32_t>(c.groups);
+    b.g_nseg = k.take<uint32_t>(c.groups);
+    b.gmem = k.take<MemberRec>(GROUP * c.groups);
+    b.ghdr = k.take<float4>(3 * c.groups);
+    b.seg_lo = k.take<uint32_t>(GROUP * c.groups);
+    b.seg_hi = k.take<uint32_t>(GROUP * c.groups);
+    b.seg_sel = k.take<uint32_t>(GROUP * c.groups);
+    b.seg_t0 = k.take<uint32_t>(GROUP * c.groups);
+    b.ntiles = k.take<uint32_t>(c.groups);
+    b.tile_base = k.take<uint64_t>(c.groups + 1);
+    b.tdesc = k.take<uint4>(c.tiles);
+    b.tile_hits = k.take<uint32_t>(c.tiles);
+    b.tile_off = k.take<uint64_t>(c.tiles + 1);
+    b.s_tile = k.take<uint32_t>(c.scratch);
+    b.s_rank = k.take<uint32_t>(c.scratch);
+    b.s_q = k.take<uint32_t>(c.scratch);
+    b.s_e = k.take<uint32_t>(c.scratch);
+    b.s_tin = k.take<double>(c.scratch);
+    b.s_tout = k.take<double>(c.scratch);
+}
+
+void free_rows(SearchOut *out, cudaStream_t s)
+{
+    for (void *p : {(void *)out->q, (void *)out->e, (void *)out->tin, (void *)out->tout})
+        if (p) cudaFreeAsync(p, s);
+    out->q = out->e = nullptr;
+    out->tin = out->tout = nullptr;
+}
+
+ts_status alloc_rows(SearchOut *out, uint64_t n, cudaStream_t s, PipeBufs &b)
+{
+    TS_CUDA(pool_malloc((void **)&out->q, sizeof(uint32_t) * n, s));
+    TS_CUDA(pool_malloc((void **)&out->e, sizeof(uint32_t) * n, s));
+    TS_CUDA(pool_malloc((void **)&out->tin, sizeof(double) * n, s));
+    TS_CUDA(pool_malloc((void **)&out->tout, sizeof(double) * n, s));
+    b.out_q = out->q;
+    b.out_e = out->e;
+    b.out_tin = out->tin;
+    b.out_tout = out->tout;
+    return TS_OK;
+}
+
+// The search with work buffers of guessed sizes in one allocation, every kernel enqueued before
+// the one wait. *done stays false, and nothing is kept, when a guess was too small, memory or a
+// slot was short: the stepwise path below, which waits for every size, then answers (also with
+// its errors). Up to ONE_GO_ROWS rows (8 per query) are in place after the wait; more take their
+// exact arrays and a second one.
+//
+// Bound: launches and their latency. A search of 20 query segments against 20,000 (34 calls to the
+// allocator, 12 pageable copies, four waits, 18 kernels before) 327 -> 207 us, of 10,000
+// against 1M on the grid 395 -> 245 us, with the binding and the copies of the rows.
+ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_params *qp,
+                        cudaStream_t s, SearchOut *out, bool *done)
+{
+    const uint64_t nq = q->n;
+    const bool grid = ix->kind == TS_INDEX_SPATIAL;
+    struct Slot {
+        HostSlot *h = g_slots.take();
+        cudaStream_t busy = nullptr;
+        bool is_busy = false;  // kernels that use the slot may be in flight (an error in between)
+        ~Slot()
+        {
+            if (is_busy) cudaStreamSynchronize(busy);
+            if (h) g_slots.give(h);
+        }
+    } slot;
+    if (!slot.h) return TS_OK;
+    PlainOut *dout = nullptr;
+    {
+        void *p = nullptr;
+        if (cudaHostGetDevicePointer(&p, slot.h, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return TS_OK;
+        }
+        dout = static_cast<PlainOut *>(p);
+    }
+    PipeCaps c;
+    c.nq = nq;
+    c.nreq = 1;
+    c.units = grid ? 16 * nq + 1024 : nq;
+    c.groups = c.units / GROUP + 2;
+    c.tiles = 64 * c.groups + 65536;
+    c.scratch = scratch_slots(std::min<uint64_t>(std::max<uint64_t>(4 * nq + (1ull << 20), 512 * nq),
+                                                 SCRATCH_MAX));
+    c.rows = std::min<uint64_t>(8 * nq + 64, ONE_GO_ROWS);
+    PipeBufs b = PipeBufs{};
+    ReqDesc *reqs = nullptr;
+    Carver size;
+    plain_layout(size, c, grid, b, &reqs);
+    DevBuf arena;
+    if (arena.alloc(size.off, s) != TS_OK) return TS_OK;
+    Carver cut;
+    cut.base = arena.as<unsigned char>();
+    plain_layout(cut, c, grid, b, &reqs);
+
+    const double *src[8] = {q->x0, q->y0, q->z0, q->t0, q->x1, q->y1, q->z1, q->t1};
+    DevBuf qcopy;
+    const double *cols[8];
+    if (q->on_host && nq <= STAGE_QUERIES) {
+        for (int k = 0; k < 8; k++) {
+            if (!src[k]) return TS_OK;  // (the stepwise path names the column)
+            memcpy(slot.h->stage + k * nq, src[k], sizeof(double) * nq);
+            cols[k] = reinterpret_cast<const double *>(reinterpret_cast<unsigned char *>(dout) +
+                                                       offsetof(HostSlot, stage)) + k * nq;
+        }
+    } else {
+        *done = true;
+        TS_CHECK(device_cols(q, s, qcopy, cols));
+        *done = false;
+    }
+    ReqDesc rd;
+    fill_req(rd, qp, 0, (uint32_t)nq);
+    for (int k = 0; k < 8; k++) rd.cols[k] = cols[k];
+    *done = true;  // (every return below but those that say otherwise)
+    TS_CHECK(alloc_rows(out, c.rows, s, b));
+    slot.busy = s;
+    slot.is_busy = true;
+    TS_LAUNCH_PDL(k_plain_start, dim3(1), dim3(32), 0, s, rd, reqs, b);
+    TS_CHECK(pipe_prepare(ix, nullptr, nq, reqs, 1, b, c, s));
+    if (grid) {
+        TS_CHECK(scan_u32(b.qnu, b.quoff, nq, b.status, s));
+        TS_CHECK(pipe_grid_units(ix, nq, b, c, s));
+    }
+    TS_CHECK(pipe_group(ix, reqs, 1, b, c, false, s));
+    c.stall_ns = g_stall_ns.exchange(0);  // (a stall requested by a test of the timeout path)
+    TS_CHECK(pipe_count(ix, reqs, b, c, s));
+    TS_CHECK(pipe_scan_rows(b, c, s));
+    TS_CHECK(pipe_write(ix, reqs, b, c, s));
+    TS_LAUNCH_PDL(k_plain_out, dim3(1), dim3(32), 0, s, nq, c.tiles, b, dout);
+    TS_CUDA(cudaStreamSynchronize(s));
+    slot.is_busy = false;
+    const PlainOut &o = slot.h->out;
+    TS_CHECK(read_dev_status(o.status & ~(uint32_t)DEV_ERR_OVERFLOW));
+    const uint64_t T = (uint64_t)o.hdr[HDR_T_LO] | ((uint64_t)o.hdr[HDR_T_HI] << 32);
+    if (o.units > c.units || T > c.tiles) {  // a guess was too small
+        free_rows(out, s);
+        *done = false;
+        return TS_OK;
+    }
+    fill_stats(o.stats, &out->stats);
+    out->stats.n_queries = nq;
+    const uint64_t total = o.total;
+    out->count = total;
+    if (out->stats.n_hits != total) {
+        set_error("hit count mismatch (%llu vs %llu)", (unsigned long long)out->stats.n_hits,
+                  (unsigned long long)total);
+        return TS_ERR_INTERNAL;
+    }
+    if (total == 0 || total > c.rows) free_rows(out, s);
+    if (qp->max_results && total > qp->max_results) {
+        free_rows(out, s);
+        set_error("%llu result rows exceed max_results %llu", (unsigned long long)total,
+                  (unsigned long long)qp->max_results);
+        return TS_ERR_CAPACITY;
+    }
+    if (total <= c.rows) return TS_OK;
+    TS_CHECK(alloc_rows(out, total, s, b));
+    c.rows = total;
+    c.stall_ns = 0;
+    slot.is_busy = true;
+    TS_CUDA(cudaMemsetAsync(b.status, 0, sizeof(uint32_t), s));  // (the rows' overflow)
+    TS_CHECK(pipe_write(ix, reqs, b, c, s));
+    TS_LAUNCH_PDL(k_plain_out, dim3(1), dim3(32), 0, s, nq, c.tiles, b, dout);
+    TS_CUDA(cudaStreamSynchronize(s));
+    slot.is_busy = false;
+    TS_CHECK(read_dev_status(o.status));
+    fill_stats(o.stats, &out->stats);
+    out->stats.n_queries = nq;
     return TS_OK;
 }
 
@@ -1797,6 +2096,11 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     const uint64_t nq = q->n;
     out->stats.n_queries = nq;
     if (nq == 0) return TS_OK;
+    if (nq <= ONE_GO_QUERIES) {
+        bool done = false;
+        const ts_status got = search_one_go(ix, q, qp, s, out, &done);
+        if (done) return got;
+    }
     DevBuf qcopy;
     const double *cols[8];
     TS_CHECK(device_cols(q, s, qcopy, cols));
@@ -1832,20 +2136,14 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     b.s_tout = b.s_tin + c.scratch;
     b.tile_off = w.tile_off.as<uint64_t>();
 
-    EventPair ev_count, ev_write;
-    TS_CHECK(ev_count.create());
-    TS_CHECK(ev_write.create());
     c.stall_ns = g_stall_ns.exchange(0);  // (a stall requested by a test of the timeout path)
-    TS_CUDA(cudaEventRecord(ev_count.a, s));
     TS_CHECK(pipe_count(ix, w.reqdesc.as<ReqDesc>(), b, c, s));
-    TS_CUDA(cudaEventRecord(ev_count.b, s));
     TS_CHECK(pipe_scan_rows(b, c, s));
     uint64_t total = 0;
     TS_CUDA(cudaMemcpyAsync(&total, b.tile_off + c.tiles, 8, cudaMemcpyDeviceToHost, s));
     TS_CHECK(copy_stats(b, s, &out->stats, &st));
     TS_CHECK(read_dev_status(st));
     out->stats.n_queries = nq;
-    out->stats.ms_count_pass = ev_count.ms();
     out->count = total;
     if (out->stats.n_hits != total) {
         set_error("hit count mismatch (%llu vs %llu)", (unsigned long long)out->stats.n_hits,
@@ -1867,14 +2165,9 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     b.out_tin = out->tin;
     b.out_tout = out->tout;
     c.rows = total;
-    TS_CUDA(cudaEventRecord(ev_write.a, s));
     TS_CHECK(pipe_write(ix, w.reqdesc.as<ReqDesc>(), b, c, s));
-    TS_CUDA(cudaEventRecord(ev_write.b, s));
-    TS_CUDA(cudaMemcpyAsync(&st, b.status, 4, cudaMemcpyDeviceToHost, s));
-    TS_CUDA(cudaStreamSynchronize(s));
-    TS_CHECK(read_dev_status(st));
-    out->stats.ms_write_pass = ev_write.ms();
-    return TS_OK;
+    TS_CHECK(copy_stats(b, s, &out->stats, &st));
+    return read_dev_status(st);
 }
 
 // The query columns of stationary points: x0 = x1 = x (likewise y, z), t0 = t_start, t1 = t_end.

@@ -106,6 +106,27 @@ inline uint64_t scratch_slots(uint64_t n)
     return n + (n / 2 + 100000 < 700000 ? n / 2 + 100000 : 700000);
 }
 
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Carves one device allocation into buffers (without a base: adds up their sizes).
+struct Carver {
+    size_t off = 0;
+    unsigned char *base = nullptr;
+    template <class T>
+    T *take(uint64_t count)
+    {
+        size_t at = off;
+        off += align256(sizeof(T) * (count ? count : 1));
+        return base ? reinterpret_cast<T *>(base + at) : nullptr;
+    }
+};
+
+// Milliseconds between two readings of the device clock (0 when either was not taken).
+inline double stamp_ms(unsigned long long a, unsigned long long b)
+{
+    return a && b > a ? (double)(b - a) * 1e-6 : 0.0;
+}
+
 // Result of one search (device arrays owned by the ts_result handle).
 struct SearchOut {
     uint64_t count = 0;

@@ -1,0 +1,123 @@
+"""Plain searches enqueued in one go on guessed capacities: guesses that hold and guesses that do
+not (cell runs, tiles, rows, queries above what one go takes), host queries read in place and
+copied, more searches at a time than there are slots; every result against the oracle."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1410_2698_gb300 import _lib, api
+from paper_1410_2698_gb300.workloads import Segments
+from tests import parity
+from tests.cases import random_segments
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(idx, db, q, d, ts, te, device=False):
+    import torch
+    qq = q
+    if device:
+        qq = [torch.from_numpy(np.ascontiguousarray(c)).cuda() for c in q.arrays()]
+    res = api.ts_search(idx, qq, d, ts, te)
+    ref = oracle.search(db, q, ts, te, d)
+    parity.compare(res.to_host(sort=True), ref, db, q, ts, te, d)
+    assert res.count == ref["q_idx"].size == res.stats["n_hits"]
+    assert res.stats["n_queries"] == q.n and res.stats["ms_count_pass"] > 0
+    return res.count
+
+
+@pytest.mark.parametrize("nq", [1, 1024, 1025, 20000])
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("kind", ["temporal", "spatiotemporal", "spatial", "brute"])
+def test_query_counts(kind, device, nq):
+    rng = np.random.default_rng(nq)
+    db = random_segments(rng, 3000, box=30.0)
+    q = random_segments(rng, nq, box=30.0)
+    _check(api.ts_build_index(db, kind=kind), db, q, 1.0, 1.0, 9.0, device)
+
+
+def test_more_rows_than_asked_for_and_none():
+    rng = np.random.default_rng(2)
+    db = random_segments(rng, 5000, box=5.0)
+    q = random_segments(rng, 40, box=5.0)
+    idx = api.ts_build_index(db, kind="temporal")
+    assert _check(idx, db, q, 4.0, 0.0, 12.0) > 64 + 8 * q.n
+    assert _check(idx, db, q, 4.0, 50.0, 60.0) == 0
+    few = api.ts_search(idx, q, 4.0, 0.0, 12.0, max_results=7)
+    assert few.status == 4 and few.count > 7 and few.device_arrays() == (None,) * 4
+
+
+def test_more_cell_runs_than_guessed():
+    """Queries across the whole grid: a thousand runs of cells each, where 16 are guessed."""
+    rng = np.random.default_rng(3)
+    db = random_segments(rng, 4000, box=100.0)
+    q = random_segments(rng, 200, box=100.0, max_len=90.0)
+    idx = api.ts_build_index(db, kind="spatial", grid_cells=64)
+    assert int(api.ts_schedule(idx, q, 1.0, 0.0, 12.0)[1].sum()) > 16 * q.n + 1024
+    _check(idx, db, q, 1.0, 0.0, 12.0)
+
+
+def test_more_tiles_than_guessed():
+    """All pairs of 3,000 queries and 250,000 entries: 977 tiles a group, where 64 are guessed."""
+    rng = np.random.default_rng(4)
+    db = random_segments(rng, 250000, box=400.0)
+    q = random_segments(rng, 3000, box=400.0)
+    idx = api.ts_build_index(db, kind="brute")
+    _check(idx, db, q, 2.0, 0.0, 12.0)
+    assert api.ts_search(idx, q, 2.0, 0.0, 12.0).stats["n_tiles"] > 64 * 95 + 65536
+
+
+def test_more_queries_than_one_go_takes():
+    rng = np.random.default_rng(5)
+    db = random_segments(rng, 2000, box=60.0)
+    q = random_segments(rng, 65537, box=60.0)
+    _check(api.ts_build_index(db, kind="spatiotemporal"), db, q, 0.5, 0.0, 12.0, True)
+
+
+def test_invalid_queries_and_columns():
+    import ctypes
+    rng = np.random.default_rng(6)
+    db = random_segments(rng, 500)
+    idx = api.ts_build_index(db, kind="spatial")
+    m = random_segments(rng, 30).as_matrix()
+    m[7, 2] = np.nan
+    with pytest.raises(_lib.TsError, match="invalid query segment"):
+        api.ts_search(idx, Segments.from_matrix(m), 1.0, 0.0, 9.0)
+    s, keep = api.make_segments(random_segments(rng, 30))
+    s.y1 = None
+    qp = _lib.ts_query_params(1.0, 0.0, 9.0, 0)
+    out = ctypes.c_void_p()
+    assert _lib.load().ts_search(idx.handle, ctypes.byref(s), ctypes.byref(qp), None,
+                                 ctypes.byref(out)) == 1
+    assert "NULL query column" in api.ts_last_error()
+    _check(idx, db, random_segments(rng, 30), 1.0, 0.0, 9.0)
+
+
+def test_threads_and_streams():
+    """24 threads with a stream each, 16 slots: the others wait for sizes step by step."""
+    import torch
+    rng = np.random.default_rng(7)
+    db = random_segments(rng, 4000, box=20.0)
+    idx = api.ts_build_index(db, kind="spatial")
+    sets = [random_segments(rng, 50 + 13 * k, box=20.0) for k in range(24)]
+    refs = [oracle.search(db, q, 0.0, 12.0, 2.0) for q in sets]
+    errors = []
+
+    def work(k):
+        try:
+            s = torch.cuda.Stream()
+            for _ in range(6):
+                got = api.ts_search(idx, sets[k], 2.0, 0.0, 12.0, stream=s.cuda_stream)
+                parity.compare(got.to_host(stream=s.cuda_stream, sort=True), refs[k], db, sets[k], 0.0, 12.0,
+                               2.0)
+        except Exception as e:  # noqa: BLE001
+            errors.append((k, e))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(24)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
