@@ -3,6 +3,7 @@
 // Steps (all device kernels; the host only picks parameters from exact reductions):
 //   ingest   : validate (finite, t1 > t0), order keys of t_start, exact extents   (Sec. 3.1)
 //   sort     : stable radix sort by t_start, ties by input index                     (Sec. 4.2)
+//   parts    : temporal bin and subbins or cell of every entry, in the input's order
 //   gather   : FP64 exact records (velocity precomputed) and FP32 outward-rounded
 //              prefilter records in sorted order
 //   bins     : m temporal bins, B_j^start, B_j^end, first/last offsets, prefix max   (Sec. 4.2)
@@ -32,17 +33,13 @@ inline unsigned nblocks(uint64_t n, int tpb = TPB)
 
 // reduction slots (order keys): 0 min t0, 1 max t1, 2 max duration, 3..5 min emin, 6..8 max
 // emax, 9..11 max extent
-enum { R_TMIN = 0, R_TMAX = 1, R_DUR = 2, R_EMIN = 3, R_EMAX = 6, R_LONG = 9, R_N = 12 };
+// 12 the bits in which some t0's key differs from the first's
+enum { R_TMIN = 0, R_TMAX = 1, R_DUR = 2, R_EMIN = 3, R_EMAX = 6, R_LONG = 9, R_VARY = 12, R_N = 13 };
 
-__device__ inline bool finite_d(double x) { return isfinite(x); }
-
-__device__ inline unsigned long long warp_min_u64(unsigned long long v)
+// (on the integer pipe)
+__device__ inline bool finite_d(double x)
 {
-    for (int o = 16; o; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w < v ? w : v;
-    }
-    return v;
+    return ((uint32_t)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
 }
 
 __device__ inline unsigned long long warp_max_u64(unsigned long long v)
@@ -66,58 +63,135 @@ __global__ void k_init_red(unsigned long long *red)
     red[i] = is_min ? ~0ull : 0ull;
 }
 
-__global__ void k_ingest(SegIn in, uint64_t n, uint64_t *keys, uint32_t *vals,
-                         unsigned long long *red, uint32_t *status)
+// Grid-stride, the extremes in registers and one atomic per block and extreme: an atomic per warp
+// and extreme on these 12 addresses took 230 of 244 us for 1M segments. Comparisons are made on
+// the order keys, integers; four FP64 subtractions are left. Bound: HBM (64 B read, 12 written).
+__global__ void __launch_bounds__(TPB) k_ingest(SegIn in, uint64_t n, uint64_t *keys, uint32_t *vals,
+                                                unsigned long long *red, uint32_t *status)
 {
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool ok = i < n;
-    double v[8];
-#pragma unroll
-    for (int k = 0; k < 8; k++) v[k] = ok ? in.f[k][i] : 0.0;
-    bool valid = true;
-#pragma unroll
-    for (int k = 0; k < 8; k++) valid = valid && finite_d(v[k]);
-    valid = valid && (v[7] > v[3]);
-    if (ok && !valid) atomicOr(status, DEV_ERR_INVALID);
-    if (ok) {
-        keys[i] = dkey(v[3]);
-        vals[i] = (uint32_t)i;
-    }
-    bool use = ok && valid;
     unsigned long long r[R_N];
-    r[R_TMIN] = use ? dkey(v[3]) : ~0ull;
-    r[R_TMAX] = use ? dkey(v[7]) : 0ull;
-    r[R_DUR] = use ? dkey(v[7] - v[3]) : 0ull;
 #pragma unroll
-    for (int d = 0; d < 3; d++) {
-        double lo = v[d] < v[4 + d] ? v[d] : v[4 + d];
-        double hi = v[d] < v[4 + d] ? v[4 + d] : v[d];
-        r[R_EMIN + d] = use ? dkey(lo) : ~0ull;
-        r[R_EMAX + d] = use ? dkey(hi) : 0ull;
-        r[R_LONG + d] = use ? dkey(hi - lo) : 0ull;
-    }
-    const int lane = threadIdx.x & 31;
+    for (int k = 0; k < R_N; k++) r[k] = (k == R_TMIN || (k >= R_EMIN && k < R_EMIN + 3)) ? ~0ull : 0ull;
+    const uint64_t first = dkey(in.f[3][0]);
+    bool bad = false;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        double v[8];
 #pragma unroll
-    for (int k = 0; k < R_N; k++) {
-        bool is_min = (k == R_TMIN) || (k >= R_EMIN && k < R_EMIN + 3);
-        unsigned long long w = is_min ? warp_min_u64(r[k]) : warp_max_u64(r[k]);
-        if (lane == 0) {
-            if (is_min) atomicMin(&red[k], w);
-            else atomicMax(&red[k], w);
+        for (int k = 0; k < 8; k++) v[k] = in.f[k][i];
+        bool valid = true;
+        unsigned long long key[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            valid = valid && finite_d(v[k]);
+            key[k] = dkey(v[k]);
+        }
+        valid = valid && key[7] > key[3];
+        bad = bad || !valid;
+        keys[i] = key[3];
+        vals[i] = (uint32_t)i;
+        r[R_VARY] |= key[3] ^ first;
+        if (!valid) continue;
+        r[R_TMIN] = min(r[R_TMIN], key[3]);
+        r[R_TMAX] = max(r[R_TMAX], key[7]);
+        r[R_DUR] = max(r[R_DUR], (unsigned long long)dkey(v[7] - v[3]));
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            r[R_EMIN + d] = min(r[R_EMIN + d], min(key[d], key[4 + d]));
+            r[R_EMAX + d] = max(r[R_EMAX + d], max(key[d], key[4 + d]));
+            r[R_LONG + d] = max(r[R_LONG + d], (unsigned long long)dkey(fabs(v[4 + d] - v[d])));
         }
     }
+    if (bad) atomicOr(status, DEV_ERR_INVALID);
+    __shared__ unsigned long long part[R_N][TPB / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < R_N; k++) {
+        const bool is_min = k == R_TMIN || (k >= R_EMIN && k < R_EMIN + 3);
+        unsigned long long w = r[k];
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long x = __shfl_xor_sync(0xffffffffu, w, o);
+            w = k == R_VARY ? (w | x) : (is_min ? min(w, x) : max(w, x));
+        }
+        if (lane == 0) part[k][wid] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x < R_N) {
+        const int k = threadIdx.x;
+        const bool is_min = k == R_TMIN || (k >= R_EMIN && k < R_EMIN + 3);
+        unsigned long long w = part[k][0];
+        for (int j = 1; j < TPB / 32; j++) {
+            const unsigned long long x = part[k][j];
+            w = k == R_VARY ? (w | x) : (is_min ? min(w, x) : max(w, x));
+        }
+        if (k == R_VARY) atomicOr(&red[k], w);
+        else if (is_min) atomicMin(&red[k], w);
+        else atomicMax(&red[k], w);
+    }
+}
+
+// A 1-D partition on the device: part_of from its boundary table (lo + j*w, j = 0..v).
+struct PartTab {
+    const double *bd;
+    double lo, w;
+    float iw;  // ~ 1/w, for the first guess; 0 where it has no FP32 value: part_of itself
+    int v;
+
+    // The same part as part_of: a guess in FP32 corrected by comparisons with the boundaries, made
+    // on the order keys (a division and the comparisons in FP64 took 90 us for a dimension of 1M
+    // entries, ten times what reading them takes).
+    __device__ __forceinline__ int of(double x) const
+    {
+        if (v <= 1 || iw == 0.0f) return part_of(x, lo, w, v);
+        const uint64_t kx = dkey(x);
+        if (kx < dkey(bd[0])) return -1;
+        const float f = floorf(((float)(x - lo)) * iw);
+        int j = !(f < (float)v) ? v - 1 : (f < 0.0f ? 0 : (int)f);
+        while (j + 1 < v && dkey(bd[j + 1]) <= kx) j++;
+        while (j > 0 && dkey(bd[j]) > kx) j--;
+        return j;
+    }
+};
+
+__global__ void k_bounds(double *bd, double lo, double w, uint32_t v)
+{
+    const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j <= v) bd[j] = part_bound(lo, w, (int)j);
+}
+
+// Temporal bin, and the parts of the MBB's corners in the three axes: first | last << 16 (subbins),
+// or the cell of the minimum corner (grid), of every entry in the input's order.
+__global__ void k_parts(SegIn in, uint64_t n, PartTab bins, PartTab px, PartTab py, PartTab pz,
+                        int kind, uint32_t *bin_in, uint32_t *part_in)
+{
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int j = bins.of(in.f[3][i]);
+    bin_in[i] = (uint32_t)(j < 0 ? 0 : j);  // (t0 >= tmin always)
+    if (kind != TS_INDEX_SPATIOTEMPORAL && kind != TS_INDEX_SPATIAL) return;
+    uint32_t cell = 0;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const PartTab &p = d == 0 ? px : (d == 1 ? py : pz);
+        const int a = p.of(in.f[d][i]), b = p.of(in.f[4 + d][i]);
+        const int lo = max(min(a, b), 0), hi = max(a, b);
+        if (kind == TS_INDEX_SPATIAL) cell = cell * (uint32_t)p.v + (uint32_t)lo;
+        else part_in[(uint64_t)d * n + i] = (uint32_t)lo | ((uint32_t)max(hi, 0) << 16);
+    }
+    if (kind == TS_INDEX_SPATIAL) part_in[i] = cell;
 }
 
 // Outward rounding of an FP64 interval to FP32 (conservative prefilter boxes).
 __device__ inline float f_dn(double x) { return __double2float_rd(x); }
 __device__ inline float f_up(double x) { return __double2float_ru(x); }
 
-__global__ void k_gather(SegIn in, uint64_t n, const uint32_t *perm, SegD *seg, RecF *rec,
-                         uint32_t *orig)
+__global__ void k_gather(SegIn in, uint64_t n, const uint32_t *perm, const uint32_t *bin_in,
+                         SegD *seg, RecF *rec, uint32_t *orig, uint32_t *bin_of,
+                         unsigned long long *end_key)
 {
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    uint32_t i = perm[s];
+    const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = s < n;
+    const uint32_t i = perm[on ? s : n - 1];
     double x0 = in.f[0][i], y0 = in.f[1][i], z0 = in.f[2][i], t0 = in.f[3][i];
     double x1 = in.f[4][i], y1 = in.f[5][i], z1 = in.f[6][i], t1 = in.f[7][i];
     double dt = t1 - t0;
@@ -126,14 +200,27 @@ __global__ void k_gather(SegIn in, uint64_t n, const uint32_t *perm, SegD *seg, 
     d.vx = (x1 - x0) / dt;
     d.vy = (y1 - y0) / dt;
     d.vz = (z1 - z0) / dt;
-    seg[s] = d;
     RecF r;
     r.xmin = f_dn(fmin(x0, x1)); r.xmax = f_up(fmax(x0, x1));
     r.ymin = f_dn(fmin(y0, y1)); r.ymax = f_up(fmax(y0, y1));
     r.zmin = f_dn(fmin(z0, z1)); r.zmax = f_up(fmax(z0, z1));
     r.t0 = f_dn(t0); r.t1 = f_up(t1);
-    rec[s] = r;
-    orig[s] = i;
+    const uint32_t j = bin_in[i];
+    if (on) {
+        seg[s] = d;
+        rec[s] = r;
+        orig[s] = i;
+        bin_of[s] = j;
+    }
+    // the bin's latest end: one atomic for a warp of one bin (the lanes are in start order)
+    const unsigned FULL = 0xffffffffu;
+    const unsigned long long k = dkey(t1);
+    if (__all_sync(FULL, j == __shfl_sync(FULL, j, 0))) {
+        const unsigned long long w = warp_max_u64(k);
+        if ((threadIdx.x & 31) == 0) atomicMax(&end_key[j], w);
+    } else {
+        atomicMax(&end_key[j], k);
+    }
 }
 
 // Key of an entry inside its bin: (bin, Morton code of its FP32 box centre, `bits` per axis). Any
@@ -201,17 +288,6 @@ __global__ void k_bins_init(uint32_t m, double tmin, double b, double *bin_start
     end_key[j] = dkey(part_bound(tmin, b, (int)j + 1));
 }
 
-__global__ void k_bin_of(const SegD *seg, uint64_t n, uint32_t m, double tmin, double b,
-                         uint32_t *bin_of, unsigned long long *end_key)
-{
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    int j = part_of(seg[s].t0, tmin, b, (int)m);
-    if (j < 0) j = 0;  // t0 >= tmin always
-    bin_of[s] = (uint32_t)j;
-    atomicMax(&end_key[j], dkey(seg[s].t1));
-}
-
 // off[j] = first sorted entry with bin >= j (bin_of is non-decreasing)
 __global__ void k_bin_bounds(const uint32_t *bin_of, uint64_t n, uint32_t m, uint32_t *off)
 {
@@ -224,79 +300,61 @@ __global__ void k_bin_bounds(const uint32_t *bin_of, uint64_t n, uint32_t m, uin
         for (uint32_t k = j + 1; k <= m; k++) off[k] = (uint32_t)n;
 }
 
-__global__ void k_bin_end_final(const unsigned long long *end_key, uint32_t m, double *bin_end)
+// The bins' ends and their prefix maximum (one block; maxima of the order keys).
+__global__ void k_bin_ends(const unsigned long long *end_key, uint32_t m, double *bin_end,
+                           double *pmax)
 {
-    uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < m) bin_end[j] = dkey_inv(end_key[j]);
-}
-
-// prefix maximum over the bins (one block)
-__global__ void k_prefix_max(const double *in, uint32_t m, double *out)
-{
-    __shared__ double tot[1024];
-    uint32_t per = (m + blockDim.x - 1) / blockDim.x;
-    uint32_t a = threadIdx.x * per, bnd = min(m, a + per);
-    double run = -INFINITY;
-    for (uint32_t j = a; j < bnd; j++) run = fmax(run, in[j]);
-    tot[threadIdx.x] = run;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = -INFINITY;
-        for (unsigned t = 0; t < blockDim.x; t++) {
-            double v = tot[t];
-            tot[t] = r;
-            r = fmax(r, v);
-        }
+    __shared__ unsigned long long tot[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t per = (m + blockDim.x - 1) / blockDim.x;
+    const uint32_t a = min(m, threadIdx.x * per), e = min(m, a + per);
+    unsigned long long run = 0;
+    for (uint32_t j = a; j < e; j++) run = max(run, end_key[j]);
+    unsigned long long incl = run;  // prefix maximum over the threads
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl = max(incl, v);
     }
+    if (lane == 31) tot[wid] = incl;
     __syncthreads();
-    run = tot[threadIdx.x];
-    for (uint32_t j = a; j < bnd; j++) {
-        run = fmax(run, in[j]);
-        out[j] = run;
+    run = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 0) run = 0;
+    for (int w = 0; w < wid; w++) run = max(run, tot[w]);
+    for (uint32_t j = a; j < e; j++) {
+        run = max(run, end_key[j]);
+        bin_end[j] = dkey_inv(end_key[j]);
+        pmax[j] = dkey_inv(run);
     }
 }
 
 // ---------------------------------------------------------------------------------------------
 // partitions (subbins / grid)
 // ---------------------------------------------------------------------------------------------
-// Per-dimension MBB of a sorted entry, taken from the caller's original endpoints (exact).
-__global__ void k_mbb(SegIn in, const uint32_t *orig, uint64_t n, int dim, double *lo, double *hi)
+// Subbins per entry and dimension, in the sweep order `tid` of the bins' entries.
+__global__ void k_part_count(const uint32_t *part_in, const uint32_t *orig, const uint32_t *tid,
+                             uint64_t n, uint32_t *cnt)
 {
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    uint32_t i = orig[s];
-    double a = in.f[dim][i], b = in.f[4 + dim][i];
-    lo[s] = a < b ? a : b;
-    hi[s] = a < b ? b : a;
+    const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t i = orig[tid[p]];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const uint32_t ab = part_in[(uint64_t)d * n + i];
+        cnt[(uint64_t)d * n + p] = (ab >> 16) - (ab & 0xffffu) + 1u;
+    }
 }
 
-// (in the sweep order `tid` of the bins' entries)
-__global__ void k_part_count(const double *lo, const double *hi, const uint32_t *tid, uint64_t n,
-                             double plo, double pw, int v, uint32_t *cnt)
+__global__ void k_part_emit(const uint32_t *part_in, const uint32_t *orig, const uint32_t *tid,
+                            uint64_t n, const uint32_t *pos, uint32_t *keys, uint32_t *vals)
 {
-    uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t s = tid[p];
-    int a = part_of(lo[s], plo, pw, v);
-    int b = part_of(hi[s], plo, pw, v);
-    if (a < 0) a = 0;
-    cnt[p] = b >= a ? (uint32_t)(b - a + 1) : 0u;
-}
-
-__global__ void k_part_emit(const double *lo, const double *hi, const uint32_t *tid, uint64_t n,
-                            double plo, double pw, int v, const uint32_t *pos, uint32_t *keys,
-                            uint32_t *vals)
-{
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t s = tid[i];
-    int a = part_of(lo[s], plo, pw, v);
-    int b = part_of(hi[s], plo, pw, v);
-    if (a < 0) a = 0;
-    uint32_t p = pos[i];
-    for (int j = a; j <= b; j++, p++) {
-        keys[p] = (uint32_t)j;
-        vals[p] = s;
+    const uint32_t ab = part_in[orig[s]];
+    uint32_t at = pos[p];
+    for (uint32_t j = ab & 0xffffu; j <= ab >> 16; j++, at++) {
+        keys[at] = j;
+        vals[at] = s;
     }
 }
 
@@ -318,18 +376,12 @@ __global__ void k_gather_rec(const uint32_t *ids, uint64_t len, const RecF *rec,
 }
 
 // grid: every sorted entry is keyed by the cell of its MBB's minimum corner (single assignment)
-__global__ void k_grid_key(const double *lo3, uint64_t n, double gx, double gy, double gz,
-                           double wx, double wy, double wz, int g, uint32_t *keys, uint32_t *vals)
+__global__ void k_grid_key(const uint32_t *cell_in, const uint32_t *orig, uint64_t n, uint32_t *keys,
+                           uint32_t *vals)
 {
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    const double plo[3] = {gx, gy, gz}, pw[3] = {wx, wy, wz};
-    uint32_t c[3];
-    for (int d = 0; d < 3; d++) {
-        int a = part_of(lo3[(uint64_t)d * n + s], plo[d], pw[d], g);
-        c[d] = (uint32_t)(a < 0 ? 0 : a);
-    }
-    keys[s] = (c[0] * (uint32_t)g + c[1]) * (uint32_t)g + c[2];
+    keys[s] = cell_in[orig[s]];
     vals[s] = (uint32_t)s;
 }
 
@@ -370,18 +422,6 @@ struct Ctx {
     }
 };
 
-// Scan counts into positions and return the total (synchronises; index building is offline).
-ts_status counts_to_pos(Ctx &c, const uint32_t *cnt, uint64_t n, DevBuf &pos, uint64_t *total)
-{
-    TS_CHECK(pos.alloc(sizeof(uint32_t) * (n + 1), c.s));
-    TS_CHECK(scan_u32(cnt, pos.as<uint32_t>(), n, c.status.as<uint32_t>(), c.s));
-    uint32_t t = 0;
-    TS_CUDA(cudaMemcpyAsync(&t, pos.as<uint32_t>() + n, 4, cudaMemcpyDeviceToHost, c.s));
-    TS_CHECK(c.read_status());
-    *total = t;
-    return TS_OK;
-}
-
 // Bounding records of an array's chunks.
 ts_status build_boxes(Ctx &c, Index *ix, const Chunk *rec, uint64_t n, RecF **box)
 {
@@ -398,24 +438,16 @@ ts_status build_boxes(Ctx &c, Index *ix, const Chunk *rec, uint64_t n, RecF **bo
 // One dimension of the spatiotemporal index. The ids are emitted in the bins' sweep order and
 // sorted stably by subbin, so a (subbin, bin) range keeps the Morton order inside and its chunks
 // are small boxes too.
-ts_status build_st_dim(Ctx &c, Index *ix, int dim, const double *lo, const double *hi,
-                       const uint32_t *bin_of)
+ts_status build_st_dim(Ctx &c, Index *ix, int dim, const uint32_t *part_in, const uint32_t *pos,
+                       uint64_t len, const uint32_t *bin_of)
 {
     const uint64_t n = ix->n;
     const int v = (int)ix->v[dim];
-    DevBuf cnt, pos;
-    TS_CHECK(cnt.alloc(sizeof(uint32_t) * n, c.s));
-    k_part_count<<<nblocks(n), TPB, 0, c.s>>>(lo, hi, ix->tid, n, ix->sub_lo[dim], ix->sub_w[dim],
-                                              v, cnt.as<uint32_t>());
-    TS_LAUNCHED();
-    uint64_t len = 0;
-    TS_CHECK(counts_to_pos(c, cnt.as<uint32_t>(), n, pos, &len));
     DevBuf keys;
     TS_CHECK(keys.alloc(sizeof(uint32_t) * len, c.s));
     TS_CHECK(ix->alloc(&ix->st_ids[dim], len));
-    k_part_emit<<<nblocks(n), TPB, 0, c.s>>>(lo, hi, ix->tid, n, ix->sub_lo[dim], ix->sub_w[dim], v,
-                                             pos.as<uint32_t>(), keys.as<uint32_t>(),
-                                             ix->st_ids[dim]);
+    k_part_emit<<<nblocks(n), TPB, 0, c.s>>>(part_in, ix->orig, ix->tid, n, pos,
+                                             keys.as<uint32_t>(), ix->st_ids[dim]);
     TS_LAUNCHED();
     TS_CHECK(radix_sort_u32(keys.as<uint32_t>(), ix->st_ids[dim], len, bits_for((uint64_t)v - 1),
                             c.s));
@@ -433,20 +465,17 @@ ts_status build_st_dim(Ctx &c, Index *ix, int dim, const double *lo, const doubl
     TS_LAUNCHED();
     TS_CHECK(build_boxes(c, ix, ix->st_rec[dim], len, &ix->st_box[dim]));
     ix->st_len[dim] = len;
-    return c.read_status();
+    return TS_OK;
 }
 
-ts_status build_grid(Ctx &c, Index *ix, const double *lo3, const double *hi3)
+ts_status build_grid(Ctx &c, Index *ix, const uint32_t *cell_in)
 {
-    (void)hi3;
     const uint64_t n = ix->n;
     const int g = (int)ix->g;
     DevBuf keys;
     TS_CHECK(keys.alloc(sizeof(uint32_t) * n, c.s));
     TS_CHECK(ix->alloc(&ix->ga, n));
-    k_grid_key<<<nblocks(n), TPB, 0, c.s>>>(lo3, n, ix->g_lo[0], ix->g_lo[1], ix->g_lo[2],
-                                            ix->g_w[0], ix->g_w[1], ix->g_w[2], g,
-                                            keys.as<uint32_t>(), ix->ga);
+    k_grid_key<<<nblocks(n), TPB, 0, c.s>>>(cell_in, ix->orig, n, keys.as<uint32_t>(), ix->ga);
     TS_LAUNCHED();
     const uint64_t ncell = (uint64_t)g * g * g;
     TS_CHECK(radix_sort_u32(keys.as<uint32_t>(), ix->ga, n, bits_for(ncell - 1), c.s));
@@ -464,29 +493,33 @@ ts_status build_grid(Ctx &c, Index *ix, const double *lo3, const double *hi3)
     // a cell spans a short stretch of time and a query's window skips most of a cell's chunks
     TS_CHECK(build_boxes(c, ix, ix->ga_rec, n, &ix->gbox));
     ix->g_len = n;
-    return c.read_status();
+    return TS_OK;
 }
 
 }  // namespace
+
+// An index larger than this leaves no more than this in the pool.
+constexpr size_t INDEX_KEEP = 512ull << 20;
 
 void destroy_index(Index *ix)
 {
     if (!ix) return;
     cudaDeviceSynchronize();
     for (void *p : ix->allocs) cudaFree(p);
+    if (ix->bytes > INDEX_KEEP) pool_trim(INDEX_KEEP);
     ix->magic = 0;
     delete ix;
 }
 
-// Boundary table lo + j*w (j = 0..v) of a partition, evaluated exactly as part_bound does.
-static ts_status upload_bounds(Index *ix, double **dst, double lo, double w, uint32_t v,
-                               cudaStream_t s)
+// The partition's boundary table lo + j*w (j = 0..v), evaluated exactly as part_bound does.
+static ts_status make_bounds(Index *ix, double **dst, double lo, double w, uint32_t v,
+                             cudaStream_t s, PartTab *tab)
 {
-    std::vector<double> h(v + 1);
-    for (uint32_t j = 0; j <= v; j++) h[j] = part_bound(lo, w, (int)j);
     TS_CHECK(ix->alloc(dst, v + 1));
-    TS_CUDA(cudaMemcpyAsync(*dst, h.data(), sizeof(double) * (v + 1), cudaMemcpyHostToDevice, s));
-    TS_CUDA(cudaStreamSynchronize(s));
+    k_bounds<<<nblocks((uint64_t)v + 1), TPB, 0, s>>>(*dst, lo, w, v);
+    TS_LAUNCHED();
+    const float iw = w > 0.0 ? (float)(1.0 / w) : 0.0f;
+    *tab = PartTab{*dst, lo, w, iw < 3.0e38f && w < 1.0e300 ? iw : 0.0f, (int)v};
     return TS_OK;
 }
 
@@ -540,6 +573,7 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     Index *ix = new Index();
     ix->kind = p->kind;
     ix->n = n;
+    ix->stream = s;
     cudaGetDevice(&ix->device);
     struct Guard {
         Index *&p;
@@ -553,7 +587,7 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     TS_CHECK(red.alloc(sizeof(unsigned long long) * R_N, s));
     k_init_red<<<1, 32, 0, s>>>(red.as<unsigned long long>());
     TS_LAUNCHED();
-    k_ingest<<<nblocks(n), TPB, 0, s>>>(in, n, keys.as<uint64_t>(), vals.as<uint32_t>(),
+    k_ingest<<<std::min(nblocks(n), 152u * 8u), TPB, 0, s>>>(in, n, keys.as<uint64_t>(), vals.as<uint32_t>(),
                                         red.as<unsigned long long>(), c.status.as<uint32_t>());
     TS_LAUNCHED();
     unsigned long long hred[R_N];
@@ -567,16 +601,6 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         ix->emax[d] = dkey_inv(hred[R_EMAX + d]);
         ix->longest[d] = dkey_inv(hred[R_LONG + d]);
     }
-
-    // sort by start time (stable: ties in input order)
-    TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, 64, s, nullptr, false));
-    TS_CHECK(ix->alloc(&ix->seg, n));
-    TS_CHECK(ix->alloc(&ix->rec, n));
-    TS_CHECK(ix->alloc(&ix->orig, n));
-    k_gather<<<nblocks(n), TPB, 0, s>>>(in, n, vals.as<uint32_t>(), ix->seg, ix->rec, ix->orig);
-    TS_LAUNCHED();
-    keys.release();
-    vals.release();
 
     // temporal bins (all kinds: the schedule of every index starts from the time range)
     {
@@ -597,7 +621,10 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         ix->m = (uint32_t)m;
         ix->b = span / (double)ix->m;
     }
-    DevBuf bin_of, end_key;
+    // temporal bins, subbins (Sec. 4.3) or grid (Sec. 4.1): boundary tables, and the parts of every
+    // entry
+    DevBuf bin_in, part_in, bin_of, end_key;
+    TS_CHECK(bin_in.alloc(sizeof(uint32_t) * n, s));
     TS_CHECK(bin_of.alloc(sizeof(uint32_t) * n, s));
     TS_CHECK(end_key.alloc(sizeof(unsigned long long) * ix->m, s));
     TS_CHECK(ix->alloc(&ix->bin_start, ix->m));
@@ -607,15 +634,60 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     k_bins_init<<<nblocks(ix->m), TPB, 0, s>>>(ix->m, ix->tmin, ix->b, ix->bin_start,
                                                end_key.as<unsigned long long>());
     TS_LAUNCHED();
-    k_bin_of<<<nblocks(n), TPB, 0, s>>>(ix->seg, n, ix->m, ix->tmin, ix->b, bin_of.as<uint32_t>(),
+    PartTab bins{ix->bin_start, ix->tmin, ix->b,
+                 ix->b > 0.0 && ix->b < 1.0e300 ? (float)(1.0 / ix->b) : 0.0f, (int)ix->m};
+    if (!(bins.iw < 3.0e38f)) bins.iw = 0.0f;
+    PartTab part[3] = {bins, bins, bins};
+    if (p->kind == TS_INDEX_SPATIOTEMPORAL) {
+        const uint32_t v_req = p->sub_bins ? p->sub_bins : 16u;
+        for (int d = 0; d < 3; d++) {
+            // v lowered so a subbin is at least as wide as the longest entry (Sec. 4.3)
+            double ext = ix->emax[d] - ix->emin[d];
+            double v = v_req < 1 ? 1.0 : (double)v_req;
+            if (ix->longest[d] > 0.0) {
+                double cap = floor(ext / ix->longest[d]);
+                if (cap < 1.0) cap = 1.0;
+                if (v > cap) v = cap;
+            }
+            if (!(ext > 0.0)) v = 1.0;
+            if (v > 4096.0) v = 4096.0;
+            ix->v[d] = (uint32_t)v;
+            ix->sub_lo[d] = ix->emin[d];
+            ix->sub_w[d] = ext / (double)ix->v[d];
+            TS_CHECK(make_bounds(ix, &ix->sub_bound[d], ix->sub_lo[d], ix->sub_w[d], ix->v[d], s,
+                                 &part[d]));
+        }
+        TS_CHECK(part_in.alloc(sizeof(uint32_t) * 3 * n, s));
+    } else if (p->kind == TS_INDEX_SPATIAL) {
+        const uint32_t g = p->grid_cells ? p->grid_cells : 50u;
+        ix->g = g;
+        for (int d = 0; d < 3; d++) {
+            ix->g_lo[d] = ix->emin[d];
+            ix->g_w[d] = (ix->emax[d] - ix->emin[d]) / (double)g;
+            TS_CHECK(make_bounds(ix, &ix->g_bound[d], ix->g_lo[d], ix->g_w[d], g, s, &part[d]));
+        }
+        TS_CHECK(part_in.alloc(sizeof(uint32_t) * n, s));
+    }
+    k_parts<<<nblocks(n), TPB, 0, s>>>(in, n, bins, part[0], part[1], part[2], p->kind,
+                                       bin_in.as<uint32_t>(), part_in.as<uint32_t>());
+    TS_LAUNCHED();
+
+    // sort by start time (stable: ties in input order), by the bits that vary
+    TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, 64, s, nullptr, false,
+                            hred[R_VARY]));
+    TS_CHECK(ix->alloc(&ix->seg, n));
+    TS_CHECK(ix->alloc(&ix->rec, n));
+    TS_CHECK(ix->alloc(&ix->orig, n));
+    k_gather<<<nblocks(n), TPB, 0, s>>>(in, n, vals.as<uint32_t>(), bin_in.as<uint32_t>(), ix->seg,
+                                        ix->rec, ix->orig, bin_of.as<uint32_t>(),
                                         end_key.as<unsigned long long>());
     TS_LAUNCHED();
+    keys.release();
+    vals.release();
     k_bin_bounds<<<nblocks(n), TPB, 0, s>>>(bin_of.as<uint32_t>(), n, ix->m, ix->bin_off);
     TS_LAUNCHED();
-    k_bin_end_final<<<nblocks(ix->m), TPB, 0, s>>>(end_key.as<unsigned long long>(), ix->m,
-                                                   ix->bin_end);
-    TS_LAUNCHED();
-    k_prefix_max<<<1, 1024, 0, s>>>(ix->bin_end, ix->m, ix->bin_pmax);
+    k_bin_ends<<<1, 1024, 0, s>>>(end_key.as<unsigned long long>(), ix->m, ix->bin_end,
+                                  ix->bin_pmax);
     TS_LAUNCHED();
 
     if (p->kind != TS_INDEX_SPATIAL) {
@@ -641,46 +713,27 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         TS_CHECK(build_boxes(c, ix, ix->trec, n, &ix->tbox));
     }
 
-    if (p->kind == TS_INDEX_SPATIOTEMPORAL || p->kind == TS_INDEX_SPATIAL) {
-        DevBuf lo3, hi3;
-        TS_CHECK(lo3.alloc(sizeof(double) * n * 3, s));
-        TS_CHECK(hi3.alloc(sizeof(double) * n * 3, s));
+    if (p->kind == TS_INDEX_SPATIOTEMPORAL) {
+        // positions of the entries' ids in the three arrays; their lengths in one wait
+        DevBuf cnt, pos;
+        TS_CHECK(cnt.alloc(sizeof(uint32_t) * 3 * n, s));
+        TS_CHECK(pos.alloc(sizeof(uint32_t) * 3 * (n + 1), s));
+        k_part_count<<<nblocks(n), TPB, 0, s>>>(part_in.as<uint32_t>(), ix->orig, ix->tid, n,
+                                                cnt.as<uint32_t>());
+        TS_LAUNCHED();
+        uint32_t len[3];
         for (int d = 0; d < 3; d++) {
-            k_mbb<<<nblocks(n), TPB, 0, s>>>(in, ix->orig, n, d, lo3.as<double>() + d * n,
-                                             hi3.as<double>() + d * n);
-            TS_LAUNCHED();
+            uint32_t *pd = pos.as<uint32_t>() + d * (n + 1);
+            TS_CHECK(scan_u32(cnt.as<uint32_t>() + d * n, pd, n, c.status.as<uint32_t>(), s));
+            TS_CUDA(cudaMemcpyAsync(&len[d], pd + n, 4, cudaMemcpyDeviceToHost, s));
         }
-        if (p->kind == TS_INDEX_SPATIOTEMPORAL) {
-            uint32_t v_req = p->sub_bins ? p->sub_bins : 16u;
-            for (int d = 0; d < 3; d++) {
-                // v lowered so a subbin is at least as wide as the longest entry (Sec. 4.3)
-                double ext = ix->emax[d] - ix->emin[d];
-                double v = v_req < 1 ? 1.0 : (double)v_req;
-                if (ix->longest[d] > 0.0) {
-                    double cap = floor(ext / ix->longest[d]);
-                    if (cap < 1.0) cap = 1.0;
-                    if (v > cap) v = cap;
-                }
-                if (!(ext > 0.0)) v = 1.0;
-                if (v > 4096.0) v = 4096.0;
-                ix->v[d] = (uint32_t)v;
-                ix->sub_lo[d] = ix->emin[d];
-                ix->sub_w[d] = ext / (double)ix->v[d];
-                TS_CHECK(upload_bounds(ix, &ix->sub_bound[d], ix->sub_lo[d], ix->sub_w[d],
-                                       ix->v[d], s));
-                TS_CHECK(build_st_dim(c, ix, d, lo3.as<double>() + d * n, hi3.as<double>() + d * n,
-                                      bin_of.as<uint32_t>()));
-            }
-        } else {
-            uint32_t g = p->grid_cells ? p->grid_cells : 50u;
-            ix->g = g;
-            for (int d = 0; d < 3; d++) {
-                ix->g_lo[d] = ix->emin[d];
-                ix->g_w[d] = (ix->emax[d] - ix->emin[d]) / (double)g;
-                TS_CHECK(upload_bounds(ix, &ix->g_bound[d], ix->g_lo[d], ix->g_w[d], g, s));
-            }
-            TS_CHECK(build_grid(c, ix, lo3.as<double>(), hi3.as<double>()));
-        }
+        TS_CHECK(c.read_status());
+        for (int d = 0; d < 3; d++)
+            TS_CHECK(build_st_dim(c, ix, d, part_in.as<uint32_t>() + d * n,
+                                  pos.as<uint32_t>() + d * (n + 1), len[d],
+                                  bin_of.as<uint32_t>()));
+    } else if (p->kind == TS_INDEX_SPATIAL) {
+        TS_CHECK(build_grid(c, ix, part_in.as<uint32_t>()));
     }
     TS_CHECK(c.read_status());
     *out = ix;

@@ -65,15 +65,19 @@ struct Index {
 
     size_t bytes = 0;
     std::vector<void *> allocs;
+    cudaStream_t stream = nullptr;  // of the build
 
     template <class T>
     ts_status alloc(T **p, size_t count)
     {
         size_t nb = sizeof(T) * (count ? count : 1);
-        cudaError_t e = cudaMalloc((void **)p, nb);
+        // from the library's pool: 22 cudaMalloc and cudaFree took 1.6 of the 3.5 ms in which an
+        // index of 1M segments was built, searched once and freed (destroy_index hands the memory
+        // of a large one back to the device)
+        cudaError_t e = pool_malloc((void **)p, nb, stream);
         if (e != cudaSuccess) {
             *p = nullptr;
-            return cuda_status(e, "cudaMalloc(index)");
+            return cuda_status(e, "pool_malloc(index)");
         }
         allocs.push_back((void *)*p);
         bytes += nb;

@@ -93,13 +93,13 @@ enum : int {
 // ---------------------------------------------------------------------------------------------
 __host__ __device__ inline uint64_t dkey(double x)
 {
-    x = x + 0.0;  // -0.0 -> +0.0
 #ifdef __CUDA_ARCH__
     uint64_t u = (uint64_t)__double_as_longlong(x);
 #else
     uint64_t u;
     memcpy(&u, &x, 8);
 #endif
+    if ((u << 1) == 0) u = 0;  // -0.0 -> +0.0 (not by an FP64 addition: its pipe is slow)
     return (u & 0x8000000000000000ull) ? ~u : (u | 0x8000000000000000ull);
 }
 
@@ -207,8 +207,9 @@ inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t
 // Stream-ordered allocation from the library's pool (freed blocks stay pooled); inside a stream
 // capture a graph memory node. Release with cudaFreeAsync.
 cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream);
-// Return the pool's unused memory of the current device to the device (synchronises it).
-void pool_trim();
+// Return the pool's unused memory of the current device, but for `keep` bytes, to the device
+// (synchronises it).
+void pool_trim(size_t keep = 0);
 
 struct DevBuf {
     void *p = nullptr;
@@ -246,9 +247,10 @@ ts_status scan_u32_to_u64(const uint32_t *in, uint64_t *out, uint64_t n, cudaStr
 ts_status scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *status,
                    cudaStream_t s, const uint32_t *n_dev = nullptr);
 // stable LSD radix sort of (key, value) pairs by the low `bits` bits of the key; without keys_out
-// the keys are left in no particular order
+// the keys are left in no particular order; bits outside `vary` are the same in all keys
 ts_status radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                         const uint32_t *n_dev = nullptr, bool keys_out = true);
+                         const uint32_t *n_dev = nullptr, bool keys_out = true,
+                         uint64_t vary = ~0ull);
 ts_status radix_sort_u32(uint32_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
                          const uint32_t *n_dev = nullptr, bool keys_out = true);
 

@@ -80,10 +80,10 @@ static cudaMemPool_t work_pool()
     return pools[dev];
 }
 
-void pool_trim()
+void pool_trim(size_t keep)
 {
     cudaMemPool_t pool = work_pool();
-    if (pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+    if (pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(pool, keep);
     cudaGetLastError();
 }
 
@@ -517,7 +517,7 @@ __global__ void k_copy_kv(const K *ks, const uint32_t *vs, K *kd, uint32_t *vd, 
 
 template <class K>
 static ts_status radix_sort_impl(K *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                                 const uint32_t *n_dev, bool keys_out)
+                                 const uint32_t *n_dev, bool keys_out, uint64_t vary = ~0ull)
 {
     if (n <= 1 || bits <= 0) return TS_OK;
     if (n <= RS_SMALL) {
@@ -535,9 +535,11 @@ static ts_status radix_sort_impl(K *keys, uint32_t *vals, uint64_t n, int bits, 
     if (!fused) TS_CHECK(off.alloc(sizeof(uint64_t) * (nh + 1), s));
     K *ka = keys, *kbp = kb.as<K>();
     uint32_t *va = vals, *vbp = vb.as<uint32_t>();
-    int passes = (bits + 7) / 8;
-    for (int p = 0; p < passes; p++) {
-        int shift = 8 * p;
+    // digits of the bits that vary, from the lowest of them on
+    if (bits < 64) vary &= (1ull << bits) - 1;
+    for (int shift = 0; shift < bits; shift += 8) {
+        if (!(vary >> shift)) break;
+        while (!((vary >> shift) & 1)) shift++;
         if (fused) {
             TS_LAUNCH_PDL((k_rs_hist<K, true>), dim3(ntiles), dim3(RS_THREADS), 0, s, ka, n, n_dev,
                           shift, hist.as<uint32_t>(), ntiles);
@@ -562,9 +564,9 @@ static ts_status radix_sort_impl(K *keys, uint32_t *vals, uint64_t n, int bits, 
 }
 
 ts_status radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
-                         const uint32_t *n_dev, bool keys_out)
+                         const uint32_t *n_dev, bool keys_out, uint64_t vary)
 {
-    return radix_sort_impl<uint64_t>(keys, vals, n, bits, s, n_dev, keys_out);
+    return radix_sort_impl<uint64_t>(keys, vals, n, bits, s, n_dev, keys_out, vary);
 }
 
 ts_status radix_sort_u32(uint32_t *keys, uint32_t *vals, uint64_t n, int bits, cudaStream_t s,
