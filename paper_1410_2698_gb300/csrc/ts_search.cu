@@ -645,14 +645,18 @@ __global__ void k_hdr(uint64_t gcap, uint64_t tcap, PipeBufs b)
 // The tiles that some member may meet, listed for the pair kernel (in no fixed order: a tile's rows
 // are placed by its index) with the mask of their chunks whose bounding records meet the bounds
 // of the group's members. Tiles and chunks that no member can meet cost a test here instead of a
-// turn of a pair-kernel warp. `split` warps share a group's tiles, 32 tiles at a time.
+// turn of a pair-kernel warp, and where tiles are many an entry holds a run of up to 32 chunks'
+// tiles, so that a warp fetches the group's members once for all of them. `split` warps share a
+// group's tiles, 32 tiles at a time. (1.13 G exact tests among 34M tiles of the grid: pair kernel
+// 75.8 -> 68.0 ms with runs; where a warp gets fewer than 256 tiles, runs leave the last warps
+// alone with long ones: 0.27 -> 0.31 ms on 180,000 tiles.)
 //
 // Listing tiles, ordering the temporal bins' entries and the queries along the Morton curve: the
 // pair kernel on 100,000 merger query segments against 20M (temporal, d = 1) 2.42 -> 1.02 ms, on
 // 50,000 dense ones against 2M (temporal, d = 2) 0.354 -> 0.23 ms. This kernel took 0.05 and
 // 0.01 ms of it; it is bound by L2 latency (0.9 ms for 34M tiles of the grid).
-__global__ void k_tile_desc(uint64_t gcap, uint64_t tcap, uint32_t tile, ArrayPtrs<const RecF> box,
-                            PipeBufs b)
+__global__ void k_tile_desc(uint64_t gcap, uint64_t tcap, uint32_t tile, uint32_t pair_warps,
+                            ArrayPtrs<const RecF> box, PipeBufs b)
 {
     pdl_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0) b.stats[ST_CNT0] = globaltimer_ns();
@@ -672,6 +676,9 @@ __global__ void k_tile_desc(uint64_t gcap, uint64_t tcap, uint32_t tile, ArrayPt
     const uint64_t ngrp = min((uint64_t)G, gcap);
     const uint64_t split = max((uint64_t)1, warps / max((uint64_t)1, ngrp));
     const uint32_t tch = tile / PK_CH;
+    // tiles per entry: as many as the 32 bits of its mask hold, but 256 tiles for every warp of
+    // the pair kernel
+    const uint32_t per = (uint32_t)max(1ull, min(32ull / tch, (unsigned long long)T / (256ull * pair_warps)));
     for (uint64_t k = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < ngrp * split;
          k += warps) {
         const uint64_t g = k / split;
@@ -720,11 +727,21 @@ __global__ void k_tile_desc(uint64_t gcap, uint64_t tcap, uint32_t tile, ArrayPt
                 if (at > -32 && at < 32) mask |= at >= 0 ? m >> at : m << -at;
             }
             if (tch < 32) mask &= (1u << tch) - 1u;
-            const unsigned any = __ballot_sync(FULL, mask != 0u);
+            const uint32_t tmask = t < ntile ? mask : 0u;
+            // one entry for a run of up to `per` tiles: its first tile's lane gathers their masks
+            const uint32_t block = (uint32_t)j << 26 | (t - f) / per;  // (32 * 2^26 tiles)
+            const uint32_t before = __shfl_up_sync(FULL, block, 1);
+            const bool head = t < ntile && (lane == 0 || before != block);
+            for (uint32_t k = 1; k < per; k++) {
+                const uint32_t m = __shfl_down_sync(FULL, tmask, k);
+                const uint32_t o = __shfl_down_sync(FULL, block, k);
+                if (lane + k < 32 && o == block) mask |= m << (k * tch);
+            }
+            const unsigned any = __ballot_sync(FULL, head && mask != 0u);
             uint32_t at = 0;
             if (lane == 0 && any) at = atomicAdd(&b.counters[2], (uint32_t)__popc(any));
             at = __shfl_sync(FULL, at, 0);
-            if (mask)
+            if (head && mask)
                 b.tdesc[at + __popc(any & ((1u << lane) - 1u))] =
                     make_uint4((uint32_t)(base + t) | (sel << 29), mask, (uint32_t)g, s0);
         }
@@ -776,6 +793,7 @@ struct PairParams {
     uint64_t rows_cap;  // write pass: rows beyond this capacity are not written (flagged)
     uint64_t scap;      // hits the count pass keeps for placement (0: none)
     uint32_t tile;      // records per tile
+    uint32_t tile_inv;  // ceil(2^16 / chunks per tile): c * it >> 16 is chunk c's tile (c < 32)
     // > 0 (tests only): the first warp of block 0 waits this long on a barrier phase that never
     // completes before taking any tile, so the kernel's timeout path runs (status, return)
     uint64_t stall_ns;
@@ -935,8 +953,8 @@ __device__ __noinline__ uint32_t pair_flush(uint32_t qn, bool all)
 }
 
 // Persistent pair kernel. Warps take listed tiles (a group of up to 32 query units and up to
-// `tile` consecutive entries of one sorted array): the first by their index in the grid, the rest
-// from a device counter. Entry records stream through a ring of PK_STAGES shared-memory buffers
+// `tile` consecutive entries of one sorted array, or a run of such tiles): the first by their
+// index in the grid, the rest from a device counter. Entry records stream through a ring of PK_STAGES shared-memory buffers
 // filled by 1-D bulk copies. The conservative FP32 filters pick the candidates of the exact test;
 // those wait in a per-warp queue that is carried across tiles and drained 32 at a time, so that
 // the exact tests run on full warps.
@@ -1012,15 +1030,22 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
         uint32_t t_next = 0;
         if (lane == 0) t_next = nwarps + atomicAdd(&B.counters[PASS], 1u);
         if (PASS == PASS_WRITE) {
-            const uint32_t th = B.tile_hits[D.x & PK_MAX_TILES];
-            if ((th & ~TILE_REDO) == 0 || (P.scap && !(th & TILE_REDO))) {
-                // no rows in this tile, or every one of them was kept by the count pass
+            // the chunks of the entry's tiles that have rows the count pass did not keep
+            const uint32_t tch = P.tile / PK_CH, c = (uint32_t)lane * tch;
+            bool redo = false;
+            if (c < 32 && (D.y >> c) != 0u) {  // (a tile of the entry, or before its last one)
+                const uint32_t th = B.tile_hits[(D.x & PK_MAX_TILES) + lane];
+                redo = (th & ~TILE_REDO) != 0 && (!P.scap || (th & TILE_REDO));
+            }
+            const uint32_t bits = tch < 32 ? (1u << tch) - 1u : FULL;
+            D.y &= __reduce_or_sync(FULL, redo ? bits << c : 0u);
+            if (!D.y) {
                 t = __shfl_sync(FULL, t_next, 0);
                 D = t < ntiles ? B.tdesc[t] : make_uint4(0u, 0u, 0u, 0u);
                 continue;
             }
         }
-        const uint32_t tile = D.x & PK_MAX_TILES, sel = D.x >> 29, cand = D.y, s0 = D.w;
+        const uint32_t tile0 = D.x & PK_MAX_TILES, sel = D.x >> 29, cand = D.y, s0 = D.w;
         // the chunk at s0 + c * PK_CH, whole (slots past the array's end or a member's range are
         // masked by the range)
         auto copy_chunk = [&](uint32_t c, uint32_t st) {
@@ -1078,6 +1103,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
 
         // a candidate that passed the filters joins the exact-test queue; its exact record, a
         // gather from HBM, is on its way to L2 while it waits there
+        uint32_t tile = tile0;  // (of the chunk being swept)
         auto enqueue = [&](bool p, uint32_t qi, uint32_t e) {
             const unsigned bm = __ballot_sync(FULL, p);
             if (bm) {
@@ -1110,6 +1136,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
             pending &= ~(1u << st);
             if (PASS == PASS_COUNT && lane == 0) W.count[0]++;
             const Chunk &C = W.stage[st];
+            tile = tile0 + ((c * P.tile_inv) >> 16);
             const unsigned act = __ballot_sync(FULL, (mc >> c) & 1u);
             // what is left of the chunk: members of the per-member pass, listed pairs [b, npl),
             // survivors of the bitmask pass (none of them when no member meets a chunk that was
@@ -1299,20 +1326,21 @@ __global__ void k_place(PipeBufs b, uint64_t scap, uint64_t tcap, uint64_t rows_
     }
     // four hits per thread at a time, their loads independent: a hit's tile offset waits for its
     // tile, and one such chain per thread left HBM idle (978 M hits, 56 B each at least: 23.3 ms
-    // with one, 16.6 ms with four and a grid of several waves, 3.3 TB/s)
-    const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * nth) {
+    // with one, 16.6 ms with four and a grid of several waves, 13.4 ms with a block's four
+    // next to each other, 4.1 TB/s)
+    for (uint64_t i0 = (uint64_t)blockIdx.x * 4 * TPB + threadIdx.x; i0 < n;
+         i0 += (uint64_t)gridDim.x * 4 * TPB) {
         uint32_t t[4], rank[4], q[4], e[4];
         double tin[4], tout[4];
         uint64_t o[4], end[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const uint64_t i = i0 + k * nth;
+            const uint64_t i = i0 + k * TPB;
             t[k] = i < n ? __ldcs(b.s_tile + i) : 0xffffffffu;  // (a slot without a hit)
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const uint64_t i = i0 + k * nth;
+            const uint64_t i = i0 + k * TPB;
             const bool on = t[k] != 0xffffffffu;
             const uint32_t tk = on && t[k] < T ? t[k] : 0u;
             rank[k] = on ? __ldcs(b.s_rank + i) : 0u;
@@ -1385,6 +1413,7 @@ void fill_pair_params(PairParams &P, const Index *ix, const ReqDesc *reqs, const
     P.rows_cap = c.rows;
     P.scap = c.scratch;
     P.tile = c.tile;
+    P.tile_inv = (65536u + c.tile / PK_CH - 1) / (c.tile / PK_CH);
     P.stall_ns = 0;
 }
 
@@ -1567,7 +1596,7 @@ ts_status pipe_count(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, co
         const unsigned dblk = (unsigned)std::min<uint64_t>(
             std::max<uint64_t>((c.groups * 32 + TPB - 1) / TPB, (c.tiles + TPB - 1) / TPB), 152 * 8);
         TS_LAUNCH_PDL(k_tile_desc, dim3(dblk), dim3(TPB), 0, s,
-                      c.groups, c.tiles, c.tile, box, b);
+                      c.groups, c.tiles, c.tile, (uint32_t)(blocks * PK_WARPS), box, b);
         TS_LAUNCH_PDL(k_pair<PASS_COUNT>, dim3(blocks), dim3(PK_THREADS),
                       PAIR_SMEM, s, P);
     }

@@ -74,7 +74,7 @@ struct PipeBufs {
     uint32_t *ntiles;
     uint64_t *tile_base;  // groups + 1
     // tiles and rows
-    uint4 *tdesc;         // per listed tile: {tile | sel << 29, chunk mask, group, first record}
+    uint4 *tdesc;  // per listed run of tiles: {first tile | sel << 29, chunk mask, group, record}
     uint32_t *tile_hits;  // per tile: hits, and TILE_REDO
     uint64_t *tile_off;   // tiles + 1
     uint32_t *out_q, *out_e;

@@ -51,3 +51,26 @@ def test_far_queries_and_many_requests(kind):
     reqs = [(q.take(np.arange(r % 7, 300, 7)), 2.0, 0.0, 20.0 - r % 3) for r in range(70)]
     for (qr, d, ts, te), res in zip(reqs, api.ts_search_batch(idx, reqs)):
         parity.compare(res.to_host(sort=True), oracle.search(db, qr, ts, te, d), db, qr, ts, te, d)
+
+
+@pytest.mark.parametrize("tile", [64, 192, 512])
+@pytest.mark.parametrize("scratch", [0, 3000])
+def test_runs_of_tiles(tile, scratch):
+    """So many tiles that a listed entry holds a run of them (16,000 queries against all of 400,000
+    entries in tiles of 64 are 3.1M), with all hits kept for placement and with the flagged tiles
+    of the runs swept again: the rows and their order are the plain search's."""
+    rng = np.random.default_rng(9)
+    db = random_segments(rng, 400000, box=300.0)
+    q = random_segments(rng, 16000, box=300.0)
+    idx = api.ts_build_index(db, kind="brute")
+    ref = api.ts_search(idx, q, 1.0, 0.0, 12.0)
+    want = ref.to_host()
+    plan = api.BatchPlan(idx, max_requests=1, max_queries=q.n, max_rows=ref.count + 10,
+                         tile_records=tile, max_tiles=4 << 20, scratch_rows=scratch)
+    plan.run([(q, 1.0, 0.0, 12.0)])
+    st = plan.wait()
+    assert not st["overflow"] and st["rows"] == ref.count > 3000
+    got = plan.request_to_host(0)
+    for k in ("q_idx", "e_idx", "t_in", "t_out"):
+        assert np.array_equal(got[k], want[k]), k
+    plan.free()
