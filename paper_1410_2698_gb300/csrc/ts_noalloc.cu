@@ -33,8 +33,11 @@ constexpr uint64_t NA_COUNTS = NA_CTRL;
 constexpr uint64_t NA_OFFS = (NA_COUNTS + 4 * NA_MAX_TILES + 255) / 256 * 256;
 constexpr uint64_t NA_PARTS = (NA_OFFS + 8 * (NA_MAX_TILES + 1) + 255) / 256 * 256;
 constexpr uint64_t NA_MAX_PARTS = (NA_MAX_TILES + NA_SCAN - 1) / NA_SCAN;
-// bounding records of the runs, in what the counts and offsets leave of the scratch (110,000)
-constexpr uint64_t NA_BOXES = (NA_PARTS + 8 * (NA_MAX_PARTS + 1) + 255) / 256 * 256;
+// bounding records of the runs, in what the counts and offsets leave of the scratch (106,000), and
+// of the tiles' whole widths
+constexpr uint64_t NA_MAX_WIDE = 4096;
+constexpr uint64_t NA_WIDE = (NA_PARTS + 8 * (NA_MAX_PARTS + 1) + 255) / 256 * 256;
+constexpr uint64_t NA_BOXES = NA_WIDE + NA_MAX_WIDE * sizeof(RecF);
 constexpr uint64_t NA_MAX_BOXES = (NA_SCRATCH_BYTES - NA_BOXES) / sizeof(RecF);
 static_assert(NA_PARTS + 8 * (NA_MAX_PARTS + 1) <= NA_SCRATCH_BYTES, "scratch layout");
 static_assert(NA_MAX_PARTS <= 2048, "one block scans the partial sums");
@@ -56,7 +59,9 @@ struct NaParams {
     double d, dd, Ts, Te;
     float d_up, d_dn, d2u;
     uint32_t run;            // database segments per bounding record (32 to NA_EB); 0: none kept
-    uint32_t seg;            // consecutive tiles a warp takes at a time
+    uint32_t seg;            // consecutive tiles a warp takes at a time (at most 32)
+    uint32_t wide;           // bounding records of the tiles' widths are kept
+    uint64_t capacity;       // rows the output arrays hold (0 when one of them is missing)
     uint32_t *q_out, *e_out;
     double *tin_out, *tout_out;
     unsigned char *scratch;  // device address of g_na_scratch
@@ -144,17 +149,41 @@ __global__ void __launch_bounds__(256) k_na_boxes(NaParams P)
     }
 }
 
-// A warp per tile, P.seg consecutive tiles at a time so that its query segments, one per lane, are
-// prepared once for several tiles. A tile is 32 blocks of 32 database segments: every lane tests
+// Bounding record of every 1024 consecutive segments, from those of their runs, a warp per record.
+__global__ void __launch_bounds__(256) k_na_wide(NaParams P)
+{
+    const float4 *box = reinterpret_cast<const float4 *>(P.scratch + NA_BOXES);
+    RecF *wide = reinterpret_cast<RecF *>(P.scratch + NA_WIDE);
+    const int lane = threadIdx.x & 31;
+    const uint64_t ch = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (ch >= P.nchunk) return;
+    // (the lanes past the last segment repeat the last run's)
+    const uint64_t i = min(ch * NA_EB + (uint64_t)lane * 32, P.n - 1);
+    const float4 u = box[2 * (i / P.run)], w = box[2 * (i / P.run) + 1];
+    float lo[4] = {u.x, u.z, w.x, w.z}, hi[4] = {u.y, u.w, w.y, w.w};
+    na_warp_bounds(lo, hi);
+    if (lane == 0) {
+        RecF b;
+        b.xmin = lo[0]; b.xmax = hi[0];
+        b.ymin = lo[1]; b.ymax = hi[1];
+        b.zmin = lo[2]; b.zmax = hi[2];
+        b.t0 = lo[3]; b.t1 = hi[3];
+        wide[ch] = b;
+    }
+}
+
+// A warp takes P.seg consecutive tiles of one block of 32 query segments, which are prepared once,
+// one per lane. First a lane per tile: does its whole width meet the bounds of the queries (pass 0),
+// has it rows (pass 1)? A tile that passes is 32 blocks of 32 database segments: every lane tests
 // one block's bounding record against the bounds of all 32 queries, then the blocks that pass are
 // tested against each query, and only a block that some query meets is read (a lane per segment)
 // and filtered, member by member; the survivors are listed in (member, lane) order and go through
 // the exact test 32 at a time. Rows of a tile are in (block, member, lane) order.
 //
-// Bound: latency and issue on sparse data (a tile that no query meets costs one load and one test
-// of 32 records), the FP32 filters where every block is met. A call on 10,000 x 200,000 segments of
-// random walks, its 10,000 rows then sorted, took 15.2 ms when every tile converted and tested all
-// its segments and prepared its queries (6.51 + 7.73 ms in the two passes), 0.42 ms now.
+// Bound: latency and issue on sparse data (a tile that no query meets costs a lane one load and one
+// test), the FP32 filters where every block is met. The two passes on 10,000 x 200,000 segments of
+// random walks took 6.51 + 7.73 ms when every tile converted and tested all its segments and
+// prepared its queries, 0.083 + 0.031 ms when a warp looked at every tile, 0.066 + 0.028 ms now.
 template <int PASS>
 __global__ void __launch_bounds__(NA_WARPS * 32) k_na_tiles(NaParams P)
 {
@@ -167,19 +196,29 @@ __global__ void __launch_bounds__(NA_WARPS * 32) k_na_tiles(NaParams P)
     uint32_t *counts = reinterpret_cast<uint32_t *>(P.scratch + NA_COUNTS);
     const unsigned long long *offs = reinterpret_cast<const unsigned long long *>(P.scratch + NA_OFFS);
     const float4 *box = reinterpret_cast<const float4 *>(P.scratch + NA_BOXES);
-    const uint64_t stride = (uint64_t)gridDim.x * NA_WARPS * P.seg;
+    const float4 *wide = reinterpret_cast<const float4 *>(P.scratch + NA_WIDE);
+    const uint64_t nwin = (P.nchunk + P.seg - 1) / P.seg;
+    const uint64_t units = P.ntiles / P.nchunk * nwin;
     uint64_t qb = ~0ull;              // query block in the lanes
     bool live = false, have_q = false;
     float4 ea = make_float4(0.f, 0.f, 0.f, 0.f), eb = ea, ga = ea, gb = ea;
-    for (uint64_t t0 = ((uint64_t)blockIdx.x * NA_WARPS + wid) * P.seg; t0 < P.ntiles; t0 += stride)
-    for (uint64_t t = t0; t < t0 + P.seg && t < P.ntiles; t++) {
-        const unsigned long long wbase = PASS == 1 ? offs[t] : 0ull;
-        const unsigned long long wend = PASS == 1 ? offs[t + 1] : 0ull;
-        if (PASS == 1 && wbase == wend) continue;
-        const uint64_t ch = t % P.nchunk, e0 = ch * NA_EB;
-        const uint64_t qi = t / P.nchunk * NA_QB + lane;
-        if (t / P.nchunk != qb) {  // the next 32 query segments, one per lane
-            qb = t / P.nchunk;
+    if (PASS == 1 && (ctrl->total > P.capacity || ctrl->status)) return;  // (no rows)
+    for (uint64_t u = (uint64_t)blockIdx.x * NA_WARPS + wid; u < units;
+         u += (uint64_t)gridDim.x * NA_WARPS) {
+        // a lane per tile
+        const uint64_t ch0 = u % nwin * P.seg, tl = u / nwin * P.nchunk + ch0 + lane;
+        const bool in = (uint32_t)lane < P.seg && ch0 + lane < P.nchunk;
+        unsigned long long wb = 0, we = 0;
+        if (PASS == 1) {
+            if (in) {
+                wb = offs[tl];
+                we = offs[tl + 1];
+            }
+            if (!__ballot_sync(FULL, wb != we)) continue;
+        }
+        const uint64_t qi = u / nwin * NA_QB + lane;
+        if (u / nwin != qb) {  // the next 32 query segments, one per lane
+            qb = u / nwin;
             have_q = live = false;
             if (qi < P.nq) {
                 double v[8];
@@ -206,106 +245,122 @@ __global__ void __launch_bounds__(NA_WARPS * 32) k_na_tiles(NaParams P)
             gb = make_float4(hi[0], hi[1], hi[2], hi[3]);
             __syncwarp();
         }
-        // blocks of the tile that meet the bounds of the queries, a lane per block
-        const uint32_t nent = (uint32_t)((P.n - e0) < NA_EB ? (P.n - e0) : NA_EB);
-        const bool inblk = (uint32_t)lane * 32 < nent;
-        RecF bx;
-        bx.xmin = bx.ymin = bx.zmin = bx.t0 = -INFINITY;
-        bx.xmax = bx.ymax = bx.zmax = bx.t1 = INFINITY;
-        if (P.run && inblk) {
-            const uint64_t c = (e0 + (uint32_t)lane * 32) / P.run;
-            const float4 u = box[2 * c], w = box[2 * c + 1];
-            bx.xmin = u.x; bx.xmax = u.y; bx.ymin = u.z; bx.ymax = u.w;
-            bx.zmin = w.x; bx.zmax = w.y; bx.t0 = w.z; bx.t1 = w.w;
+        bool meet = PASS == 1 ? wb != we : in;
+        if (PASS == 0 && in) {
+            if (P.wide) {
+                const float4 x = wide[2 * (ch0 + lane)], y = wide[2 * (ch0 + lane) + 1];
+                RecF b;
+                b.xmin = x.x; b.xmax = x.y; b.ymin = x.z; b.ymax = x.w;
+                b.zmin = y.x; b.zmax = y.y; b.t0 = y.z; b.t1 = y.w;
+                meet = filter_box(b, ga, gb);
+            }
+            if (!meet) counts[tl] = 0;
         }
-        unsigned todo = __ballot_sync(FULL, inblk && filter_box(bx, ga, gb));
-        unsigned long long hits = 0;
-        for (; todo; todo &= todo - 1u) {
-            const int c = __ffs(todo) - 1;
-            RecF cb;  // block c's record, for every lane's own query
-            cb.xmin = __shfl_sync(FULL, bx.xmin, c); cb.xmax = __shfl_sync(FULL, bx.xmax, c);
-            cb.ymin = __shfl_sync(FULL, bx.ymin, c); cb.ymax = __shfl_sync(FULL, bx.ymax, c);
-            cb.zmin = __shfl_sync(FULL, bx.zmin, c); cb.zmax = __shfl_sync(FULL, bx.zmax, c);
-            cb.t0 = __shfl_sync(FULL, bx.t0, c); cb.t1 = __shfl_sync(FULL, bx.t1, c);
-            unsigned act = __ballot_sync(FULL, live && filter_box(cb, ea, eb));
-            if (!act) continue;
-            const uint32_t j = (uint32_t)c * 32 + lane;
-            const bool inb = j < nent;
-            const uint64_t ei = e0 + (inb ? j : 0);
-            double v[8];
-#pragma unroll
-            for (int k = 0; k < 8; k++) v[k] = P.e[k][ei];
-            const bool use = inb && na_valid(v);
-            const RecF r = na_rec(v);
-            uint32_t np = 0;  // listed pairs (warp-uniform)
-            for (; act; act &= act - 1u) {
-                const int m = __ffs(act) - 1;
-                const float4 mea = W.ea[m], meb = W.eb[m];
-                const bool p = use && filter_box(r, mea, meb) &&
-                               filter_gap_e(r, mea, meb, P.d_dn, P.d2u);
-                const unsigned pm = __ballot_sync(FULL, p);
-                if (p) W.pair[np + __popc(pm & lt_mask)] = (uint16_t)(m << 5 | lane);
-                np += __popc(pm);
+        for (unsigned tiles = __ballot_sync(FULL, meet); tiles; tiles &= tiles - 1u) {
+            const int l = __ffs(tiles) - 1;
+            const uint64_t t = __shfl_sync(FULL, (unsigned long long)tl, l), e0 = (ch0 + l) * NA_EB;
+            const unsigned long long wbase = __shfl_sync(FULL, wb, l), wend = __shfl_sync(FULL, we, l);
+            // blocks of the tile that meet the bounds of the queries, a lane per block
+            const uint32_t nent = (uint32_t)((P.n - e0) < NA_EB ? (P.n - e0) : NA_EB);
+            const bool inblk = (uint32_t)lane * 32 < nent;
+            RecF bx;
+            bx.xmin = bx.ymin = bx.zmin = bx.t0 = -INFINITY;
+            bx.xmax = bx.ymax = bx.zmax = bx.t1 = INFINITY;
+            if (P.run && inblk) {
+                const uint64_t c = (e0 + (uint32_t)lane * 32) / P.run;
+                const float4 u = box[2 * c], w = box[2 * c + 1];
+                bx.xmin = u.x; bx.xmax = u.y; bx.ymin = u.z; bx.ymax = u.w;
+                bx.zmin = w.x; bx.zmax = w.y; bx.t0 = w.z; bx.t1 = w.w;
             }
-            if (!np) continue;
-            {
-                const double dt = v[7] - v[3];
-                SegD e;
-                e.x0 = v[0]; e.y0 = v[1]; e.z0 = v[2]; e.t0 = v[3]; e.t1 = v[7];
-                e.vx = (v[4] - v[0]) / dt;
-                e.vy = (v[5] - v[1]) / dt;
-                e.vz = (v[6] - v[2]) / dt;
-                W.e[lane] = e;
-            }
-            if (!have_q) {
-                have_q = true;
-                if (qi < P.nq) {
+            unsigned todo = __ballot_sync(FULL, inblk && filter_box(bx, ga, gb));
+            unsigned long long hits = 0;
+            for (; todo; todo &= todo - 1u) {
+                const int c = __ffs(todo) - 1;
+                RecF cb;  // block c's record, for every lane's own query
+                cb.xmin = __shfl_sync(FULL, bx.xmin, c); cb.xmax = __shfl_sync(FULL, bx.xmax, c);
+                cb.ymin = __shfl_sync(FULL, bx.ymin, c); cb.ymax = __shfl_sync(FULL, bx.ymax, c);
+                cb.zmin = __shfl_sync(FULL, bx.zmin, c); cb.zmax = __shfl_sync(FULL, bx.zmax, c);
+                cb.t0 = __shfl_sync(FULL, bx.t0, c); cb.t1 = __shfl_sync(FULL, bx.t1, c);
+                unsigned act = __ballot_sync(FULL, live && filter_box(cb, ea, eb));
+                if (!act) continue;
+                const uint32_t j = (uint32_t)c * 32 + lane;
+                const bool inb = j < nent;
+                const uint64_t ei = e0 + (inb ? j : 0);
+                double v[8];
 #pragma unroll
-                    for (int k = 0; k < 8; k++) v[k] = P.q[k][qi];
+                for (int k = 0; k < 8; k++) v[k] = P.e[k][ei];
+                const bool use = inb && na_valid(v);
+                const RecF r = na_rec(v);
+                uint32_t np = 0;  // listed pairs (warp-uniform)
+                for (; act; act &= act - 1u) {
+                    const int m = __ffs(act) - 1;
+                    const float4 mea = W.ea[m], meb = W.eb[m];
+                    const bool p = use && filter_box(r, mea, meb) &&
+                                   filter_gap_e(r, mea, meb, P.d_dn, P.d2u);
+                    const unsigned pm = __ballot_sync(FULL, p);
+                    if (p) W.pair[np + __popc(pm & lt_mask)] = (uint16_t)(m << 5 | lane);
+                    np += __popc(pm);
+                }
+                if (!np) continue;
+                {
                     const double dt = v[7] - v[3];
-                    QueryD q;
-                    q.vx = (v[4] - v[0]) / dt;
-                    q.vy = (v[5] - v[1]) / dt;
-                    q.vz = (v[6] - v[2]) / dt;
-                    q.w0 = dmx(v[3], P.Ts);
-                    q.w1 = dmn(v[7], P.Te);
-                    const double dw = q.w0 - v[3];  // 0 unless the interval clips the start
-                    q.xw = fma(q.vx, dw, v[0]);
-                    q.yw = fma(q.vy, dw, v[1]);
-                    q.zw = fma(q.vz, dw, v[2]);
-                    q.ndd = -P.dd;
-                    W.q[lane] = q;
+                    SegD e;
+                    e.x0 = v[0]; e.y0 = v[1]; e.z0 = v[2]; e.t0 = v[3]; e.t1 = v[7];
+                    e.vx = (v[4] - v[0]) / dt;
+                    e.vy = (v[5] - v[1]) / dt;
+                    e.vz = (v[6] - v[2]) / dt;
+                    W.e[lane] = e;
                 }
-            }
-            __syncwarp();
-            for (uint32_t b = 0; b < np; b += 32) {
-                bool h = false;
-                double tin = 0.0, tout = 0.0;
-                uint32_t pr = 0;
-                if (b + lane < np) {
-                    pr = W.pair[b + lane];
-                    h = pair_test(W.q[pr >> 5], W.e[pr & 31u], PASS == 1, &tin, &tout);
-                }
-                const unsigned hm = __ballot_sync(FULL, h);
-                if (PASS == 1 && h) {
-                    const unsigned long long o = wbase + hits + __popc(hm & lt_mask);
-                    if (o < wend) {
-                        P.q_out[o] = (uint32_t)(qb * NA_QB + (pr >> 5));
-                        P.e_out[o] = (uint32_t)(e0 + (uint32_t)c * 32 + (pr & 31u));
-                        P.tin_out[o] = tin;
-                        P.tout_out[o] = tout;
+                if (!have_q) {
+                    have_q = true;
+                    if (qi < P.nq) {
+#pragma unroll
+                        for (int k = 0; k < 8; k++) v[k] = P.q[k][qi];
+                        const double dt = v[7] - v[3];
+                        QueryD q;
+                        q.vx = (v[4] - v[0]) / dt;
+                        q.vy = (v[5] - v[1]) / dt;
+                        q.vz = (v[6] - v[2]) / dt;
+                        q.w0 = dmx(v[3], P.Ts);
+                        q.w1 = dmn(v[7], P.Te);
+                        const double dw = q.w0 - v[3];  // 0 unless the interval clips the start
+                        q.xw = fma(q.vx, dw, v[0]);
+                        q.yw = fma(q.vy, dw, v[1]);
+                        q.zw = fma(q.vz, dw, v[2]);
+                        q.ndd = -P.dd;
+                        W.q[lane] = q;
                     }
                 }
-                hits += __popc(hm);
+                __syncwarp();
+                for (uint32_t b = 0; b < np; b += 32) {
+                    bool h = false;
+                    double tin = 0.0, tout = 0.0;
+                    uint32_t pr = 0;
+                    if (b + lane < np) {
+                        pr = W.pair[b + lane];
+                        h = pair_test(W.q[pr >> 5], W.e[pr & 31u], PASS == 1, &tin, &tout);
+                    }
+                    const unsigned hm = __ballot_sync(FULL, h);
+                    if (PASS == 1 && h) {
+                        const unsigned long long o = wbase + hits + __popc(hm & lt_mask);
+                        if (o < wend) {
+                            P.q_out[o] = (uint32_t)(qb * NA_QB + (pr >> 5));
+                            P.e_out[o] = (uint32_t)(e0 + (uint32_t)c * 32 + (pr & 31u));
+                            P.tin_out[o] = tin;
+                            P.tout_out[o] = tout;
+                        }
+                    }
+                    hits += __popc(hm);
+                }
+                __syncwarp();
+            }
+            if (PASS == 0) {
+                if (lane == 0) counts[t] = (uint32_t)hits;  // (at most 32 x 1024)
+            } else {
+                if (lane == 0 && wbase + hits != wend) atomicOr(&ctrl->status, DEV_ERR_INTERNAL);
             }
             __syncwarp();
         }
-        if (PASS == 0) {
-            if (lane == 0) counts[t] = (uint32_t)hits;  // (at most 32 x 1024)
-        } else {
-            if (lane == 0 && wbase + hits != wend) atomicOr(&ctrl->status, DEV_ERR_INTERNAL);
-        }
-        __syncwarp();
     }
 }
 
@@ -511,10 +566,12 @@ ts_status search_brute_noalloc(const ts_segments *db, const ts_segments *q,
     TS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const uint64_t want = (ntiles + NA_WARPS - 1) / NA_WARPS;
     const unsigned grid = (unsigned)(want < (uint64_t)sms * 6 ? want : (uint64_t)sms * 6);
-    // consecutive tiles per warp: as many as leave every warp several turns (uneven tiles), few
-    // enough that the warp's queries change seldom
-    const uint64_t seg = ntiles / ((uint64_t)grid * NA_WARPS * 4);
-    P.seg = (uint32_t)(seg < 1 ? 1 : (seg > 16 ? 16 : seg));
+    // consecutive tiles per warp: as many as leave every warp a turn
+    const uint64_t seg = ntiles / ((uint64_t)grid * NA_WARPS);
+    P.seg = (uint32_t)(seg < 1 ? 1 : (seg > 32 ? 32 : seg));
+    P.wide = P.run && nchunk <= NA_MAX_WIDE;
+    const bool out_ok = q_idx && e_idx && t_in && t_out;
+    P.capacity = out_ok ? capacity : 0;
     const uint64_t runs = (db->n + 31) / 32;
     const unsigned bgrid = (unsigned)std::min<uint64_t>((runs + 7) / 8, (uint64_t)sms * 16);
     const uint64_t nparts = (ntiles + NA_SCAN - 1) / NA_SCAN;
@@ -523,6 +580,10 @@ ts_status search_brute_noalloc(const ts_segments *db, const ts_segments *q,
     TS_CUDA(cudaMemsetAsync(scratch, 0, NA_CTRL, s));
     k_na_boxes<<<bgrid, 256, 0, s>>>(P);
     TS_LAUNCHED();
+    if (P.wide) {
+        k_na_wide<<<(unsigned)((nchunk + 7) / 8), 256, 0, s>>>(P);
+        TS_LAUNCHED();
+    }
     k_na_tiles<0><<<grid, NA_WARPS * 32, 0, s>>>(P);
     TS_LAUNCHED();
     k_na_scan_parts<<<(unsigned)nparts, 1024, 0, s>>>(scratch, ntiles);
@@ -530,6 +591,9 @@ ts_status search_brute_noalloc(const ts_segments *db, const ts_segments *q,
     k_na_scan_top<<<1, 1024, 0, s>>>(scratch, nparts);
     TS_LAUNCHED();
     k_na_scan_final<<<(unsigned)nparts, 1024, 0, s>>>(scratch, ntiles);
+    TS_LAUNCHED();
+    // (the device sees whether the rows fit: one wait, for the outcome of both passes)
+    k_na_tiles<1><<<grid, NA_WARPS * 32, 0, s>>>(P);
     TS_LAUNCHED();
     NaCtrl h;
     TS_CUDA(cudaMemcpyAsync(&h, scratch, sizeof(NaCtrl), cudaMemcpyDeviceToHost, s));
@@ -541,16 +605,11 @@ ts_status search_brute_noalloc(const ts_segments *db, const ts_segments *q,
                   (unsigned long long)h.total, (unsigned long long)capacity);
         return TS_ERR_CAPACITY;
     }
-    if (h.total == 0) return TS_OK;
-    if (!q_idx || !e_idx || !t_in || !t_out) {
+    if (h.total && !out_ok) {
         set_error("ts_search_brute_noalloc: NULL output array");
         return TS_ERR_INVALID_ARG;
     }
-    k_na_tiles<1><<<grid, NA_WARPS * 32, 0, s>>>(P);
-    TS_LAUNCHED();
-    TS_CUDA(cudaMemcpyAsync(&h, scratch, sizeof(NaCtrl), cudaMemcpyDeviceToHost, s));
-    TS_CUDA(cudaStreamSynchronize(s));
-    return na_status(h.status);
+    return TS_OK;
 }
 
 }  // namespace ts
