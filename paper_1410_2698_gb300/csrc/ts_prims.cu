@@ -169,107 +169,112 @@ __device__ __forceinline__ void put_off(uint32_t *out, uint64_t v, uint32_t *sta
     *out = (uint32_t)v;
 }
 
-template <class Tin>
-__global__ void k_tile_sums(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
+// Tiles of one block of a scan over n values: as many blocks as SCAN_BLOCKS at most, each with a run
+// of consecutive tiles, so that a capacity far above the count costs empty blocks only up to that
+// number (a plan of 33M tiles launched 16,000 blocks for 2,000 tiles) and two kernels always do.
+constexpr uint64_t SCAN_BLOCKS = 152 * 8;
+
+struct ScanPart {
+    uint64_t n, first, last;  // values, tiles [first, last)
+};
+__device__ __forceinline__ ScanPart scan_part(uint64_t ncap, const uint32_t *n_dev)
+{
+    ScanPart p;
+    p.n = dev_count(ncap, n_dev);
+    const uint64_t tiles = p.n / SCAN_TILE + 1;  // (one of them holds index n)
+    const uint64_t per = (tiles + gridDim.x - 1) / gridDim.x;
+    p.first = min(tiles, per * blockIdx.x);
+    p.last = min(tiles, p.first + per);
+    return p;
+}
+
+__global__ void k_tile_sums(const uint32_t *in, uint64_t ncap, const uint32_t *n_dev, uint32_t mask,
                             uint64_t *sums)
 {
     pdl_enter();
-    const uint64_t n = dev_count(ncap, n_dev);
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
-    if (base >= n) {
-        if (threadIdx.x == 0) sums[blockIdx.x] = 0;
-        return;
-    }
+    const ScanPart p = scan_part(ncap, n_dev);
     uint64_t acc = 0;
+    for (uint64_t t = p.first; t < p.last; t++) {
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; k++) {
-        uint64_t i = base + (uint64_t)k * SCAN_THREADS + threadIdx.x;
-        if (i < n) acc += (uint64_t)(in[i] & mask);
+        for (int k = 0; k < SCAN_ITEMS; k++) {
+            const uint64_t i = t * SCAN_TILE + (uint64_t)k * SCAN_THREADS + threadIdx.x;
+            if (i < p.n) acc += in[i] & mask;
+        }
     }
     uint64_t total;
     block_excl_scan<uint64_t>(acc, &total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// Scan of one tile per block, out[i] = exclusive prefix; the block whose tile holds index n writes
-// out[n] = total. The tiles before: `tile_off` holds their scanned sums, or `sums` the sums
-// themselves, which every block adds up (at most SCAN_LOOKBACK of them), or neither (one tile).
-constexpr uint64_t SCAN_LOOKBACK = 4096;
-
-template <class Tin, class Tout>
-__global__ void k_tile_scan(const Tin *in, uint64_t ncap, const uint32_t *n_dev, Tin mask,
-                            const uint64_t *tile_off, const uint64_t *sums, Tout *out,
-                            uint32_t *status)
+// out[i] = exclusive prefix, and out[n] = total by the block whose tile holds index n. Every block
+// first adds up the sums of the blocks before it.
+template <class Tout>
+__global__ void k_tile_scan(const uint32_t *in, uint64_t ncap, const uint32_t *n_dev, uint32_t mask,
+                            const uint64_t *sums, Tout *out, uint32_t *status)
 {
     pdl_enter();
-    const uint64_t n = dev_count(ncap, n_dev);
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
-    if (base > n) return;
-    // thread-contiguous items for a stable sequential order within a thread
-    uint64_t v[SCAN_ITEMS], acc = 0;
-    const uint64_t tbase = base + (uint64_t)threadIdx.x * SCAN_ITEMS;
-#pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; k++) {
-        const uint64_t i = tbase + k;
-        v[k] = i < n ? (uint64_t)(in[i] & mask) : 0ull;
-        acc += v[k];
-    }
-    uint64_t before = tile_off ? tile_off[blockIdx.x] : 0ull;
-    if (sums) {
+    const ScanPart p = scan_part(ncap, n_dev);
+    if (p.first >= p.last) return;
+    uint64_t before = 0;
+    if (blockIdx.x) {
         uint64_t pre = 0;
         for (uint32_t j = threadIdx.x; j < blockIdx.x; j += SCAN_THREADS) pre += sums[j];
         block_excl_scan<uint64_t>(pre, &before);
     }
-    uint64_t total;
-    uint64_t off = before + block_excl_scan<uint64_t>(acc, &total);
+    for (uint64_t t = p.first; t < p.last; t++) {
+        // thread-contiguous items for a stable sequential order within a thread
+        uint32_t v[SCAN_ITEMS];
+        uint64_t acc = 0;
+        const uint64_t tbase = t * SCAN_TILE + (uint64_t)threadIdx.x * SCAN_ITEMS;
 #pragma unroll
-    for (int k = 0; k < SCAN_ITEMS; k++) {
-        const uint64_t i = tbase + k;
-        if (i < n) put_off(out + i, off, status);
-        off += v[k];
+        for (int k = 0; k < SCAN_ITEMS; k++) {
+            v[k] = tbase + k < p.n ? in[tbase + k] & mask : 0u;
+            acc += v[k];
+        }
+        uint64_t total;
+        uint64_t off = before + block_excl_scan<uint64_t>(acc, &total);
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; k++) {
+            if (tbase + k < p.n) put_off(out + tbase + k, off, status);
+            off += v[k];
+        }
+        before += total;
+        if (threadIdx.x == 0 && p.n < (t + 1) * SCAN_TILE) put_off(out + p.n, before, status);
     }
-    if (threadIdx.x == 0 && n < base + SCAN_TILE) put_off(out + n, before + total, status);
 }
 
-// Exclusive scan of n (or *n_dev <= n) values: out[0..n] with out[n] = total. One block per tile
-// of SCAN_TILE values plus one, so that the tile holding index n always exists. 32-bit offsets are
-// written by the scan itself: the 64-bit array and the kernel that narrowed it are gone.
-template <class Tin, class Tout>
-static ts_status scan_impl(const Tin *in, Tout *out, uint64_t n, const uint32_t *n_dev,
-                           cudaStream_t s, Tin mask, uint32_t *status)
+// Exclusive scan of n (or *n_dev <= n) values: out[0..n] with out[n] = total. 32-bit offsets are
+// checked and written by the scan itself.
+template <class Tout>
+static ts_status scan_impl(const uint32_t *in, Tout *out, uint64_t n, const uint32_t *n_dev,
+                           cudaStream_t s, uint32_t mask, uint32_t *status)
 {
     if (n == 0) {
         TS_CUDA(cudaMemsetAsync(out, 0, sizeof(Tout), s));
         return TS_OK;
     }
-    const uint64_t nt = n / SCAN_TILE + 1;
-    DevBuf sums, offs;
-    if (nt > 1) {
-        TS_CHECK(sums.alloc(sizeof(uint64_t) * nt, s));
-        TS_LAUNCH_PDL(k_tile_sums<Tin>, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
+    const unsigned nb = (unsigned)std::min<uint64_t>(n / SCAN_TILE + 1, SCAN_BLOCKS);
+    DevBuf sums;
+    if (nb > 1) {
+        TS_CHECK(sums.alloc(sizeof(uint64_t) * nb, s));
+        TS_LAUNCH_PDL(k_tile_sums, dim3(nb), dim3(SCAN_THREADS), 0, s,
                       in, n, n_dev, mask, sums.as<uint64_t>());
     }
-    if (nt > SCAN_LOOKBACK) {
-        TS_CHECK(offs.alloc(sizeof(uint64_t) * (nt + 1), s));
-        TS_CHECK((scan_impl<uint64_t, uint64_t>(sums.as<uint64_t>(), offs.as<uint64_t>(), nt,
-                                                nullptr, s, ~0ull, nullptr)));
-    }
-    TS_LAUNCH_PDL((k_tile_scan<Tin, Tout>), dim3((unsigned)nt), dim3(SCAN_THREADS), 0, s,
-                  in, n, n_dev, mask, nt > SCAN_LOOKBACK ? offs.as<uint64_t>() : nullptr,
-                  nt > 1 && nt <= SCAN_LOOKBACK ? sums.as<uint64_t>() : nullptr, out, status);
+    TS_LAUNCH_PDL(k_tile_scan<Tout>, dim3(nb), dim3(SCAN_THREADS), 0, s,
+                  in, n, n_dev, mask, sums.as<uint64_t>(), out, status);
     return TS_OK;
 }
 
 ts_status scan_u32_to_u64(const uint32_t *in, uint64_t *out, uint64_t n, cudaStream_t s,
                           const uint32_t *n_dev, uint32_t mask)
 {
-    return scan_impl<uint32_t, uint64_t>(in, out, n, n_dev, s, mask, nullptr);
+    return scan_impl<uint64_t>(in, out, n, n_dev, s, mask, nullptr);
 }
 
 ts_status scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *status,
                    cudaStream_t s, const uint32_t *n_dev)
 {
-    return scan_impl<uint32_t, uint32_t>(in, out, n, n_dev, s, ~0u, status);
+    return scan_impl<uint32_t>(in, out, n, n_dev, s, ~0u, status);
 }
 
 // ---------------------------------------------------------------------------------------------
