@@ -540,6 +540,9 @@ ts_status ts_result_copy_to_host(const ts_result *r, uint32_t *q_idx, uint32_t *
     }
     const uint64_t n = r->out.count;
     cudaStream_t s = (cudaStream_t)stream;
+    ts_status few = TS_OK;
+    if (copy_few_rows(r->out, q_idx, e_idx, t_in, t_out, s, &few))
+        return few == TS_OK ? clear_error(few) : few;
     if (n && r->out.q) {
         if (q_idx) TS_CUDA(cudaMemcpyAsync(q_idx, r->out.q, 4 * n, cudaMemcpyDeviceToHost, s));
         if (e_idx) TS_CUDA(cudaMemcpyAsync(e_idx, r->out.e, 4 * n, cudaMemcpyDeviceToHost, s));

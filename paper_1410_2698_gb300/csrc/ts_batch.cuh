@@ -69,7 +69,6 @@ struct RowBlock {
     ts_status alloc(uint64_t n, cudaStream_t s);
     ~RowBlock();
 };
-constexpr uint64_t ROW_BYTES = 2 * sizeof(uint32_t) + 2 * sizeof(double);
 
 void note_launches(unsigned long long n);
 

@@ -2199,6 +2199,66 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     return read_dev_status(st);
 }
 
+// Rows into a slot's pinned memory: t_in, t_out, q_idx, e_idx.
+__global__ void k_rows_out(uint64_t n, const uint32_t *q, const uint32_t *e, const double *tin,
+                           const double *tout, double *to)
+{
+    pdl_enter();
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint32_t *w = reinterpret_cast<uint32_t *>(to + 2 * n);
+    to[i] = tin[i];
+    to[n + i] = tout[i];
+    w[i] = q[i];
+    w[n + i] = e[i];
+}
+
+// Few rows reach pageable host memory through a slot, in one kernel and one wait (four pageable
+// copies take 10 us each). False when the four copies have to do it: more rows than a slot holds,
+// no slot free, rows of another device than the current one, or a destination that is not host
+// memory.
+bool copy_few_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
+                   cudaStream_t s, ts_status *st)
+{
+    const uint64_t n = o.count;
+    if (n == 0 || !o.q || n * ROW_BYTES > sizeof(HostSlot::stage)) return false;
+    int dev = -1;
+    cudaPointerAttributes pa;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&pa, o.q) != cudaSuccess ||
+        pa.device != dev) {
+        cudaGetLastError();
+        return false;
+    }
+    for (const void *p : {(const void *)q, (const void *)e, (const void *)tin, (const void *)tout})
+        if (p && (cudaPointerGetAttributes(&pa, p) != cudaSuccess ||
+                  pa.type == cudaMemoryTypeDevice)) {
+            cudaGetLastError();
+            return false;
+        }
+    struct Slot {
+        HostSlot *h = g_slots.take();
+        ~Slot() { if (h) g_slots.give(h); }
+    } slot;
+    void *d = nullptr;
+    if (!slot.h || cudaHostGetDevicePointer(&d, slot.h->stage, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    *st = [&]() -> ts_status {
+        TS_LAUNCH_PDL(k_rows_out, dim3(nblk(n)), dim3(TPB), 0, s, n, o.q, o.e, o.tin, o.tout,
+                      static_cast<double *>(d));
+        TS_CUDA(cudaStreamSynchronize(s));
+        const double *h = slot.h->stage;
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(h + 2 * n);
+        if (tin) memcpy(tin, h, 8 * n);
+        if (tout) memcpy(tout, h + n, 8 * n);
+        if (q) memcpy(q, w, 4 * n);
+        if (e) memcpy(e, w + n, 4 * n);
+        return TS_OK;
+    }();
+    return true;
+}
+
 // The query columns of stationary points: x0 = x1 = x (likewise y, z), t0 = t_start, t1 = t_end.
 __global__ void k_point_cols(const double *x, const double *y, const double *z, uint64_t n,
                              double ts, double te, double *cols)

@@ -135,6 +135,10 @@ struct SearchOut {
     ts_search_stats stats{};
 };
 
+constexpr uint64_t ROW_BYTES = 24;  // q_idx, e_idx, t_in, t_out
+bool copy_few_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
+                   cudaStream_t s, ts_status *st);
+
 const char *last_error();
 unsigned long long launch_count();
 

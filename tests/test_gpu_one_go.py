@@ -121,3 +121,20 @@ def test_threads_and_streams():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+@pytest.mark.parametrize("n", [1, 2729, 2730, 2731, 9000])
+def test_rows_to_host(n):
+    """Rows through a slot (up to 2,730) and by four copies are the device's rows."""
+    m = np.zeros((n, 8))
+    m[:, 7] = 1.0 + np.arange(n) / n
+    idx = api.ts_build_index(Segments.from_matrix(m), kind="temporal")
+    res = api.ts_search(idx, Segments.from_matrix(m[:1]), 1.0, 0.0, 5.0)
+    assert res.count == n
+    host = res.to_host()
+    assert np.array_equal(np.sort(host["e_idx"]), np.arange(n))
+    assert np.all(host["q_idx"] == 0) and np.all(host["t_in"] == 0) and np.all(host["t_out"] == 1)
+    lib = _lib.load()
+    only = np.empty(n, np.uint32)  # a destination of its own, the others left out
+    _lib.check(lib.ts_result_copy_to_host(res.handle, None, only.ctypes.data, None, None, None))
+    assert np.array_equal(only, host["e_idx"])
