@@ -97,12 +97,12 @@ typedef struct ts_search_stats {
     uint64_t n_tiles;     /* work tiles (query group x candidate range) */
     uint64_t n_groups;    /* query groups (up to 32 queries sharing a candidate range) */
     uint64_t n_subbin;    /* queries served from a subbin range (spatiotemporal index) */
-    double ms_count_pass; /* device time of the pair kernel's count pass (CUDA events) */
-    double ms_write_pass; /* device time of the pair kernel's write pass (CUDA events) */
+    double ms_count_pass; /* device time of the pair kernel's count pass (device clock) */
+    double ms_write_pass; /* device time of the pair kernel's write pass (device clock) */
     /* how the pair kernel's count pass swept the candidates (diagnostics): */
     uint64_t n_chunks;    /* (tile, chunk of 64 entries) pairs swept */
-    uint64_t n_dense;     /* chunks swept by the two-axis bitmask (more than 8 members meet them) */
-    uint64_t n_sparse;    /* (member, chunk) visits of the per-member path (few members meet) */
+    uint64_t n_dense;     /* grid chunks swept by the two-axis bitmask (more than 8 members meet) */
+    uint64_t n_sparse;    /* (member, chunk) visits of the per-member path */
     uint64_t n_stage2;    /* bitmask survivors given the full FP32 box and gap filters */
 } ts_search_stats;
 

@@ -239,6 +239,47 @@ __global__ void k_tm_key(const RecF *rec, const uint32_t *bin_of, uint64_t n, Mo
     vals[s] = (uint32_t)s;
 }
 
+// Entries (every stride-th) by their place along each axis.
+__global__ void __launch_bounds__(TPB) k_axis_hist(const RecF *rec, uint64_t n, uint64_t stride,
+                                                   MortonMap mm, uint32_t *hist)
+{
+    __shared__ uint32_t h[3 * AXIS_BINS];
+    for (int i = threadIdx.x; i < 3 * AXIS_BINS; i += TPB) h[i] = 0;
+    __syncthreads();
+    for (uint64_t i = ((uint64_t)blockIdx.x * TPB + threadIdx.x) * stride; i < n;
+         i += (uint64_t)gridDim.x * TPB * stride) {
+        const RecF r = rec[i];
+        atomicAdd(&h[(int)mm.place(0.5f * r.xmin + 0.5f * r.xmax, 0)], 1u);
+        atomicAdd(&h[AXIS_BINS + (int)mm.place(0.5f * r.ymin + 0.5f * r.ymax, 1)], 1u);
+        atomicAdd(&h[2 * AXIS_BINS + (int)mm.place(0.5f * r.zmin + 0.5f * r.zmax, 2)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * AXIS_BINS; i += TPB)
+        if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
+// The share of the entries before every place (a warp per axis).
+__global__ void k_axis_rank(const uint32_t *hist, float *rank)
+{
+    const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
+    constexpr int PER = AXIS_BINS / 32;
+    uint32_t sum = 0;
+    for (int k = 0; k < PER; k++) sum += hist[d * AXIS_BINS + lane * PER + k];
+    uint32_t incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const float total = (float)max(1u, __shfl_sync(0xffffffffu, incl, 31));
+    uint32_t run = incl - sum;
+    float *r = rank + d * (AXIS_BINS + 1);
+    for (int k = 0; k < PER; k++) {
+        r[lane * PER + k] = (float)run / total;
+        run += hist[d * AXIS_BINS + lane * PER + k];
+    }
+    if (lane == 31) r[AXIS_BINS] = 1.0f;
+}
+
 // Bounding record of every aligned chunk of 64 records, a warp per chunk.
 __global__ void k_chunk_box(const Chunk *rec, uint64_t n, uint64_t nchunks, RecF *box)
 {
@@ -694,20 +735,25 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         // bins ordered along the Morton curve inside (ranges over the start-time order cover
         // whole bins): 4 bits an axis more than it takes to tell the entries of a mean bin apart
         const int per_bin = bits_for(n / ix->m);
+        DevBuf tkeys, hist;
+        TS_CHECK(hist.alloc(sizeof(uint32_t) * 3 * AXIS_BINS, s));
+        TS_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(uint32_t) * 3 * AXIS_BINS, s));
+        TS_CHECK(ix->alloc(&ix->axis_rank, 3 * (AXIS_BINS + 1)));
+        TS_CHECK(ix->alloc(&ix->tid, n));
         const MortonMap mm =
             morton_map(ix, std::min(10, std::max(4, (per_bin + 2) / 3 + 4)));
-        DevBuf tkeys, tvals;
-        TS_CHECK(tkeys.alloc(sizeof(uint64_t) * n, s));
-        TS_CHECK(tvals.alloc(sizeof(uint32_t) * n, s));
-        k_tm_key<<<nblocks(n), TPB, 0, s>>>(ix->rec, bin_of.as<uint32_t>(), n, mm,
-                                            tkeys.as<uint64_t>(), tvals.as<uint32_t>());
+        k_axis_hist<<<64, TPB, 0, s>>>(ix->rec, n, std::max<uint64_t>(1, n >> 17), mm,
+                                       hist.as<uint32_t>());
         TS_LAUNCHED();
-        TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), tvals.as<uint32_t>(), n,
+        k_axis_rank<<<1, 96, 0, s>>>(hist.as<uint32_t>(), ix->axis_rank);
+        TS_LAUNCHED();
+        TS_CHECK(tkeys.alloc(sizeof(uint64_t) * n, s));
+        k_tm_key<<<nblocks(n), TPB, 0, s>>>(ix->rec, bin_of.as<uint32_t>(), n, mm,
+                                            tkeys.as<uint64_t>(), ix->tid);
+        TS_LAUNCHED();
+        TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), ix->tid, n,
                                 3 * mm.bits + bits_for((uint64_t)ix->m - 1), s, nullptr, false));
         TS_CHECK(ix->alloc(&ix->trec, (n + CHUNK - 1) / CHUNK));
-        TS_CHECK(ix->alloc(&ix->tid, n));
-        TS_CUDA(cudaMemcpyAsync(ix->tid, tvals.p, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice,
-                                s));
         k_gather_rec<<<nblocks(n), TPB, 0, s>>>(ix->tid, n, ix->rec, ix->trec);
         TS_LAUNCHED();
         TS_CHECK(build_boxes(c, ix, ix->trec, n, &ix->tbox));

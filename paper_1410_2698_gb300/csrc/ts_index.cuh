@@ -31,6 +31,7 @@ struct Index {
     Chunk *trec = nullptr;
     uint32_t *tid = nullptr;
     RecF *tbox = nullptr;
+    float *axis_rank = nullptr;  // share of the entries before each of 256 places of each axis
 
     // temporal bins (Sec. 4.2)
     uint32_t m = 0;
@@ -85,10 +86,19 @@ struct Index {
     }
 };
 
-// Morton code of a point of the database's extents: `bits` per axis, interleaved. Points outside
-// (queries) take the nearest cell; the code only orders, so its FP32 rounding never matters.
+// Morton code of a point among the database's entries: its rank along each axis (the share of the
+// entries before it, from a table over the extents), `bits` bits of it, interleaved. Ranks rather
+// than coordinates: entries crowd, and so do the queries, and a few bits of the coordinate leave a
+// crowd in one cell (merger, 100,000 query segments of the cores: 1.20M chunks swept with 3 bits of
+// the coordinates, 0.93M with 4 of the ranks; pair kernel 0.84 -> 0.69 ms, with the per-member pass
+// that small chunks call for).
+// Points outside (queries) take the nearest cell; the code only orders, so its FP32 rounding never
+// matters.
+constexpr int AXIS_BINS = 256;
+
 struct MortonMap {
     float lo[3], inv[3];
+    const float *rank;  // 3 x (AXIS_BINS + 1)
     int bits;
 
     __device__ static __forceinline__ uint32_t spread(uint32_t v)  // bit k -> bit 3k, 10 bits
@@ -98,10 +108,18 @@ struct MortonMap {
         v = (v | (v << 4)) & 0x030c30c3u;
         return (v | (v << 2)) & 0x09249249u;
     }
+    // place among the axis's bins, [0, AXIS_BINS) (NaN: 0)
+    __device__ __forceinline__ float place(float x, int d) const
+    {
+        return fminf(fmaxf((x - lo[d]) * inv[d], 0.0f), (float)AXIS_BINS - 0.01f);
+    }
     __device__ __forceinline__ uint32_t cell(float x, int d) const
     {
-        const float top = (float)((1 << bits) - 1);
-        return (uint32_t)fminf(fmaxf((x - lo[d]) * inv[d], 0.0f), top);  // (NaN: 0)
+        const float p = place(x, d);
+        const int k = (int)p;
+        const float a = rank[d * (AXIS_BINS + 1) + k], b = rank[d * (AXIS_BINS + 1) + k + 1];
+        const float r = a + (p - (float)k) * (b - a);
+        return min((uint32_t)(r * (float)(1 << bits)), (1u << bits) - 1u);
     }
     __device__ __forceinline__ uint32_t code(float x, float y, float z) const
     {
@@ -113,10 +131,11 @@ inline MortonMap morton_map(const Index *ix, int bits)
 {
     MortonMap m;
     m.bits = bits;
+    m.rank = ix->axis_rank;
     for (int d = 0; d < 3; d++) {
         const double ext = ix->emax[d] - ix->emin[d];
         m.lo[d] = (float)ix->emin[d];
-        const float inv = ext > 0.0 ? (float)((double)(1 << bits) / ext) : 0.0f;
+        const float inv = ext > 0.0 ? (float)((double)AXIS_BINS / ext) : 0.0f;
         m.inv[d] = inv < 3.0e38f ? inv : 0.0f;
     }
     return m;

@@ -23,7 +23,7 @@ constexpr int PK_STAGES = 2;   // chunk stages per warp (copies in flight while 
 constexpr int PK_QUEUE = 128;  // exact-test queue per warp (drained at a chunk's end)
 constexpr uint32_t PK_PLIST = 128;  // box-test survivors of a chunk awaiting the gap bound
 constexpr uint32_t PK_MAX_TILES = (1u << 29) - 1;  // tile index bits of a queued candidate
-constexpr int PK_SPARSE = 8;  // chunks met by at most this many members: per-member sweep
+constexpr int PK_SPARSE = 8;  // grid chunks met by at most this many members: per-member sweep
 constexpr int PK_TILE = 256;   // records per tile (multiple of PK_CH)
 constexpr int GROUP = 32;      // units per group
 constexpr int PK_MIN_BLOCKS = 2;  // resident pair-kernel blocks per SM the register budget targets
