@@ -1830,7 +1830,34 @@ namespace {
 
 constexpr uint64_t ONE_GO_QUERIES = 1ull << 16;  // above, the kernels dwarf the waits
 constexpr uint64_t ONE_GO_ROWS = 1ull << 16;     // rows a result may have room for unasked
+constexpr uint64_t ONE_GO_UNITS = 1ull << 22;    // (2 KB of work buffers each 32)
+constexpr uint64_t ONE_GO_TILES = 1ull << 24;    // (28 B of work buffers each)
 constexpr uint64_t STAGE_QUERIES = 1024;         // host queries read in place from pinned memory
+
+// Runs of cells of a query no longer than the longest entry: its extents in x and y, d more on
+// both sides and the longest entry's more below, in cells. (A first guess of 16 was too small for
+// d of several cells, and a dense search on the grid ran twice: 403 -> 503 us.)
+uint64_t grid_runs(const Index *ix, double d)
+{
+    uint64_t runs = 1;
+    for (int k = 0; k < 2; k++) {
+        const double cells = ix->g_w[k] > 0.0 ? ceil((2.0 * d + 2.0 * ix->longest[k]) / ix->g_w[k]) + 1.0
+                                              : 1.0;
+        runs *= cells < (double)ix->g ? (uint64_t)cells : (uint64_t)ix->g;
+    }
+    return runs;
+}
+
+// About the most tiles of a group: all entries without bins, those of the bins that a window as
+// long as the longest entry meets, twice over, with bins; a few runs of cells on the grid.
+uint64_t group_tiles(const Index *ix)
+{
+    if (ix->kind == TS_INDEX_SPATIAL) return 64;
+    double n = (double)ix->n;
+    if (ix->kind != TS_INDEX_BRUTE && ix->b > 0.0)
+        n = std::min(n, 2.0 * (ceil(ix->max_dur / ix->b) + 4.0) * (n / ix->m));
+    return (uint64_t)(n / PK_TILE) + GROUP + 2;
+}
 
 // What the host reads after the wait.
 struct PlainOut {
@@ -2016,9 +2043,10 @@ ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_pa
     PipeCaps c;
     c.nq = nq;
     c.nreq = 1;
-    c.units = grid ? 16 * nq + 1024 : nq;
+    c.units = grid ? nq * grid_runs(ix, qp->d) + 1024 : nq;
     c.groups = c.units / GROUP + 2;
-    c.tiles = 64 * c.groups + 65536;
+    c.tiles = group_tiles(ix) * c.groups + 65536;
+    if (c.units > ONE_GO_UNITS || c.tiles > ONE_GO_TILES) return TS_OK;
     c.scratch = scratch_slots(std::min<uint64_t>(std::max<uint64_t>(4 * nq + (1ull << 20), 512 * nq),
                                                  SCRATCH_MAX));
     c.rows = std::min<uint64_t>(8 * nq + 64, ONE_GO_ROWS);

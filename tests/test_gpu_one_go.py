@@ -50,23 +50,35 @@ def test_more_rows_than_asked_for_and_none():
 
 
 def test_more_cell_runs_than_guessed():
-    """Queries across the whole grid: a thousand runs of cells each, where 16 are guessed."""
+    """Queries across the whole grid, far longer than any entry: hundreds of runs of cells each,
+    where a handful is guessed."""
     rng = np.random.default_rng(3)
     db = random_segments(rng, 4000, box=100.0)
     q = random_segments(rng, 200, box=100.0, max_len=90.0)
     idx = api.ts_build_index(db, kind="spatial", grid_cells=64)
-    assert int(api.ts_schedule(idx, q, 1.0, 0.0, 12.0)[1].sum()) > 16 * q.n + 1024
+    assert int(api.ts_schedule(idx, q, 1.0, 0.0, 12.0)[1].sum()) > 49 * q.n + 1024
     _check(idx, db, q, 1.0, 0.0, 12.0)
 
 
+@pytest.mark.parametrize("d", [0.2, 5.0, 60.0])
+def test_distances_of_a_part_of_a_cell_to_all_cells(d):
+    rng = np.random.default_rng(8)
+    db = random_segments(rng, 3000, box=50.0)
+    q = random_segments(rng, 70, box=50.0)
+    _check(api.ts_build_index(db, kind="spatial"), db, q, d, 0.0, 12.0)
+
+
 def test_more_tiles_than_guessed():
-    """All pairs of 3,000 queries and 250,000 entries: 977 tiles a group, where 64 are guessed."""
+    """3,000 query segments as long as 500 entries, one after another in a group's 32 bins' worth of
+    entries: their ranges take all 977 tiles where a few bins' are guessed."""
     rng = np.random.default_rng(4)
-    db = random_segments(rng, 250000, box=400.0)
-    q = random_segments(rng, 3000, box=400.0)
-    idx = api.ts_build_index(db, kind="brute")
-    _check(idx, db, q, 2.0, 0.0, 12.0)
-    assert api.ts_search(idx, q, 2.0, 0.0, 12.0).stats["n_tiles"] > 64 * 95 + 65536
+    db = random_segments(rng, 250000, box=400.0, t_range=(0.0, 500.0), max_dur=1.0)
+    m = random_segments(rng, 3000, box=400.0).as_matrix()
+    m[:, 3], m[:, 7] = 0.0, 501.0
+    q = Segments.from_matrix(m)
+    idx = api.ts_build_index(db, kind="temporal")
+    _check(idx, db, q, 2.0, 0.0, 501.0)
+    assert api.ts_search(idx, q, 2.0, 0.0, 501.0).stats["n_tiles"] > 50 * 95 + 65536
 
 
 def test_more_queries_than_one_go_takes():
