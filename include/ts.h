@@ -206,6 +206,10 @@ ts_status ts_result_stats(const ts_result *r, ts_search_stats *stats);
 ts_status ts_result_copy_to_host(const ts_result *r, uint32_t *q_idx, uint32_t *e_idx,
                                  double *t_in, double *t_out, void *stream);
 
+/* The same rows ordered by (q_idx, e_idx), sorted on the device. */
+ts_status ts_result_copy_sorted_to_host(const ts_result *r, uint32_t *q_idx, uint32_t *e_idx,
+                                        double *t_in, double *t_out, void *stream);
+
 /* ---------------------------------------------------------------------------------------------
  * Batched search. Many requests (each a query set with its own d and interval) run through one
  * pipeline: one query preparation launch, one sort of all candidate ranges, one persistent pair

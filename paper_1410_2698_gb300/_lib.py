@@ -126,6 +126,7 @@ SIGNATURES = {
                               ctypes.POINTER(_P)]),
     "ts_result_stats": (_S, [_P, ctypes.POINTER(ts_search_stats)]),
     "ts_result_copy_to_host": (_S, [_P, _P, _P, _P, _P, _P]),
+    "ts_result_copy_sorted_to_host": (_S, [_P, _P, _P, _P, _P, _P]),
     "ts_free": (None, [_P]),
     "ts_last_error": (ctypes.c_char_p, []),
     "ts_version": (ctypes.c_char_p, []),

@@ -257,12 +257,13 @@ def ts_result_copy_to_host(result: Result, stream=None, sort=False) -> dict:
     e = np.empty(n, dtype=np.uint32)
     tin = np.empty(n, dtype=np.float64)
     tout = np.empty(n, dtype=np.float64)
+    on_device = sort and n > 256  # (fewer are sorted sooner by the host)
     if n:
-        check(lib.ts_result_copy_to_host(result.handle, q.ctypes.data, e.ctypes.data,
-                                         tin.ctypes.data, tout.ctypes.data,
-                                         _current_stream(stream)))
+        copy = lib.ts_result_copy_sorted_to_host if on_device else lib.ts_result_copy_to_host
+        check(copy(result.handle, q.ctypes.data, e.ctypes.data, tin.ctypes.data, tout.ctypes.data,
+                   _current_stream(stream)))
     out = {"q_idx": q, "e_idx": e, "t_in": tin, "t_out": tout}
-    if sort and n:
+    if sort and n and not on_device:
         order = np.lexsort((e, q))
         out = {k: v[order] for k, v in out.items()}
     return out

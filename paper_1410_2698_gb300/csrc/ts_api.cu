@@ -541,7 +541,7 @@ ts_status ts_result_copy_to_host(const ts_result *r, uint32_t *q_idx, uint32_t *
     const uint64_t n = r->out.count;
     cudaStream_t s = (cudaStream_t)stream;
     ts_status few = TS_OK;
-    if (copy_few_rows(r->out, q_idx, e_idx, t_in, t_out, s, &few))
+    if (copy_few_rows(r->out, nullptr, q_idx, e_idx, t_in, t_out, s, &few))
         return few == TS_OK ? clear_error(few) : few;
     if (n && r->out.q) {
         if (q_idx) TS_CUDA(cudaMemcpyAsync(q_idx, r->out.q, 4 * n, cudaMemcpyDeviceToHost, s));
@@ -551,6 +551,20 @@ ts_status ts_result_copy_to_host(const ts_result *r, uint32_t *q_idx, uint32_t *
     }
     TS_CUDA(cudaStreamSynchronize(s));
     return clear_error(TS_OK);
+}
+
+ts_status ts_result_copy_sorted_to_host(const ts_result *r, uint32_t *q_idx, uint32_t *e_idx,
+                                        double *t_in, double *t_out, void *stream)
+{
+    if (!r || r->magic != MAGIC_RESULT) {
+        set_error("ts_result_copy_sorted_to_host: invalid handle");
+        return TS_ERR_INVALID_ARG;
+    }
+    return guarded([&]() -> ts_status {
+        const ts_status st =
+            copy_sorted_rows(r->out, q_idx, e_idx, t_in, t_out, (cudaStream_t)stream);
+        return st == TS_OK ? clear_error(st) : st;
+    });
 }
 
 void ts_free(void *handle)

@@ -458,6 +458,7 @@ ts_status search_batch(const Index *ix, uint32_t nreq, const ts_segments *qs,
     for (uint32_t r = 0; r < nreq; r++) {
         outs[r].count = p->h_row0[r + 1] - p->h_row0[r];
         outs[r].stats.n_queries = qs[r].n;
+        outs[r].n_entries = ix->n;
         outs[r].stats.n_hits = outs[r].count;
         if (qps[r].max_results && outs[r].count > qps[r].max_results) over = true;
     }

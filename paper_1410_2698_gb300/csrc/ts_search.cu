@@ -1447,8 +1447,9 @@ int bits_for(uint64_t v)
 // ---------------------------------------------------------------------------------------------
 // pipeline stages
 // ---------------------------------------------------------------------------------------------
-KeyFmt key_fmt(const Index *ix, uint32_t nreq)
+KeyFmt key_fmt(const Index *ix, const PipeCaps &c)
 {
+    const uint32_t nreq = c.nreq;
     uint64_t maxlen = ix->n;
     for (int d = 0; d < 3; d++) maxlen = std::max<uint64_t>(maxlen, ix->st_len[d]);
     maxlen = std::max<uint64_t>(maxlen, ix->g_len);
@@ -1504,7 +1505,7 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
     P.kind = ix->kind;
     P.reqs = reqs;
     P.nreq = nreq;
-    P.kf = key_fmt(ix, c.nreq);
+    P.kf = key_fmt(ix, c);
     P.mm = morton_map(ix, P.kf.morton);
     P.n = ix->n;
     P.m = ix->m;
@@ -1554,7 +1555,7 @@ ts_status pipe_grid_units(const Index *ix, uint64_t nq, const PipeBufs &b, const
     if (!nq) return TS_OK;
     const unsigned ublk = (unsigned)std::min<uint64_t>((nq + TPB - 1) / TPB, 152 * 16);
     TS_LAUNCH_PDL(k_grid_units, dim3(ublk), dim3(TPB), 0, s,
-                  nq, c.units, key_fmt(ix, c.nreq), ix->g, ix->g_off, b);
+                  nq, c.units, key_fmt(ix, c), ix->g, ix->g_off, b);
     return TS_OK;
 }
 
@@ -1563,7 +1564,7 @@ ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const 
                      cudaStream_t s)
 {
     // one bit above the key fields: a unit without candidates has key ~0 and sorts last
-    const KeyFmt f = key_fmt(ix, c.nreq);
+    const KeyFmt f = key_fmt(ix, c);
     const int bits =
         3 * f.morton + f.lo_bits + f.sel_bits + bits_for(c.nreq > 1 ? c.nreq - 1 : 0) + 1;
     TS_CHECK(radix_sort_u64(b.keys, b.vals, c.units, bits, s, b.hdr + HDR_NU, false));
@@ -2153,6 +2154,7 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     *out = SearchOut{};
     const uint64_t nq = q->n;
     out->stats.n_queries = nq;
+    out->n_entries = ix->n;
     if (nq == 0) return TS_OK;
     if (nq <= ONE_GO_QUERIES) {
         bool done = false;
@@ -2228,36 +2230,56 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     return read_dev_status(st);
 }
 
-// Rows into a slot's pinned memory: t_in, t_out, q_idx, e_idx.
-__global__ void k_rows_out(uint64_t n, const uint32_t *q, const uint32_t *e, const double *tin,
-                           const double *tout, double *to)
+// Rows, in their order or in `order`, into one block of memory (a slot's pinned one, or the device's):
+// t_in, t_out, q_idx, e_idx.
+__global__ void k_rows_out(uint64_t n, const uint32_t *order, const uint32_t *q, const uint32_t *e,
+                           const double *tin, const double *tout, double *to)
 {
     pdl_enter();
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
     uint32_t *w = reinterpret_cast<uint32_t *>(to + 2 * n);
-    to[i] = tin[i];
-    to[n + i] = tout[i];
-    w[i] = q[i];
-    w[n + i] = e[i];
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t r = order ? order[i] : i;
+        to[i] = tin[r];
+        to[n + i] = tout[r];
+        w[i] = q[r];
+        w[n + i] = e[r];
+    }
+}
+
+__global__ void k_row_keys(uint64_t n, const uint32_t *q, const uint32_t *e, int ebits,
+                           uint64_t *keys, uint32_t *vals)
+{
+    pdl_enter();
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        keys[i] = ((uint64_t)q[i] << ebits) | e[i];
+        vals[i] = (uint32_t)i;
+    }
+}
+
+// Whether kernels of the current device may read the rows.
+bool rows_here(const SearchOut &o)
+{
+    int dev = -1;
+    cudaPointerAttributes pa;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&pa, o.q) == cudaSuccess &&
+        pa.device == dev)
+        return true;
+    cudaGetLastError();
+    return false;
 }
 
 // Few rows reach pageable host memory through a slot, in one kernel and one wait (four pageable
 // copies take 10 us each). False when the four copies have to do it: more rows than a slot holds,
 // no slot free, rows of another device than the current one, or a destination that is not host
 // memory.
-bool copy_few_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
-                   cudaStream_t s, ts_status *st)
+bool copy_few_rows(const SearchOut &o, const uint32_t *order, uint32_t *q, uint32_t *e, double *tin,
+                   double *tout, cudaStream_t s, ts_status *st)
 {
     const uint64_t n = o.count;
-    if (n == 0 || !o.q || n * ROW_BYTES > sizeof(HostSlot::stage)) return false;
-    int dev = -1;
+    if (n == 0 || !o.q || n * ROW_BYTES > sizeof(HostSlot::stage) || !rows_here(o)) return false;
     cudaPointerAttributes pa;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&pa, o.q) != cudaSuccess ||
-        pa.device != dev) {
-        cudaGetLastError();
-        return false;
-    }
     for (const void *p : {(const void *)q, (const void *)e, (const void *)tin, (const void *)tout})
         if (p && (cudaPointerGetAttributes(&pa, p) != cudaSuccess ||
                   pa.type == cudaMemoryTypeDevice)) {
@@ -2274,8 +2296,8 @@ bool copy_few_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, do
         return false;
     }
     *st = [&]() -> ts_status {
-        TS_LAUNCH_PDL(k_rows_out, dim3(nblk(n)), dim3(TPB), 0, s, n, o.q, o.e, o.tin, o.tout,
-                      static_cast<double *>(d));
+        TS_LAUNCH_PDL(k_rows_out, dim3(nblk(n)), dim3(TPB), 0, s, n, order, o.q, o.e, o.tin,
+                      o.tout, static_cast<double *>(d));
         TS_CUDA(cudaStreamSynchronize(s));
         const double *h = slot.h->stage;
         const uint32_t *w = reinterpret_cast<const uint32_t *>(h + 2 * n);
@@ -2286,6 +2308,61 @@ bool copy_few_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, do
         return TS_OK;
     }();
     return true;
+}
+
+// Rows to the host by (query, entry): sorted on the device (the two indices are one key of as many
+// bits as queries and entries take; no two rows have the same) and copied from one block. Rows of
+// another device, or more than the device's memory can sort, are sorted here. 15,000 rows, sorted
+// by numpy from the host's copy before: 1147 -> 433 us with their search.
+ts_status copy_sorted_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
+                           cudaStream_t s)
+{
+    const uint64_t n = o.count;
+    if (n == 0 || !o.q) {
+        TS_CUDA(cudaStreamSynchronize(s));
+        return TS_OK;
+    }
+    DevBuf keys, vals, rows;
+    if (n <= 0xffffffffull && rows_here(o) && keys.alloc(8 * n, s) == TS_OK &&
+        vals.alloc(4 * n, s) == TS_OK && rows.alloc(ROW_BYTES * n, s) == TS_OK) {
+        const int eb = o.n_entries ? bits_for(o.n_entries - 1) : 32;
+        const int qb = o.stats.n_queries ? bits_for(o.stats.n_queries - 1) : 32;
+        TS_LAUNCH_PDL(k_row_keys, dim3(nblk(n)), dim3(TPB), 0, s, n, o.q, o.e, eb,
+                      keys.as<uint64_t>(), vals.as<uint32_t>());
+        TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, eb + qb, s, nullptr,
+                                false));
+        ts_status few = TS_OK;
+        if (copy_few_rows(o, vals.as<uint32_t>(), q, e, tin, tout, s, &few)) return few;
+        double *d = rows.as<double>();
+        uint32_t *w = reinterpret_cast<uint32_t *>(d + 2 * n);
+        TS_LAUNCH_PDL(k_rows_out, dim3(nblk(n)), dim3(TPB), 0, s, n, vals.as<uint32_t>(), o.q, o.e,
+                      o.tin, o.tout, d);
+        if (tin) TS_CUDA(cudaMemcpyAsync(tin, d, 8 * n, cudaMemcpyDeviceToHost, s));
+        if (tout) TS_CUDA(cudaMemcpyAsync(tout, d + n, 8 * n, cudaMemcpyDeviceToHost, s));
+        if (q) TS_CUDA(cudaMemcpyAsync(q, w, 4 * n, cudaMemcpyDeviceToHost, s));
+        if (e) TS_CUDA(cudaMemcpyAsync(e, w + n, 4 * n, cudaMemcpyDeviceToHost, s));
+        TS_CUDA(cudaStreamSynchronize(s));
+        return TS_OK;
+    }
+    std::vector<uint32_t> hq(n), he(n);
+    std::vector<double> ha(n), hb(n);
+    TS_CUDA(cudaMemcpyAsync(hq.data(), o.q, 4 * n, cudaMemcpyDeviceToHost, s));
+    TS_CUDA(cudaMemcpyAsync(he.data(), o.e, 4 * n, cudaMemcpyDeviceToHost, s));
+    TS_CUDA(cudaMemcpyAsync(ha.data(), o.tin, 8 * n, cudaMemcpyDeviceToHost, s));
+    TS_CUDA(cudaMemcpyAsync(hb.data(), o.tout, 8 * n, cudaMemcpyDeviceToHost, s));
+    TS_CUDA(cudaStreamSynchronize(s));
+    std::vector<uint64_t> at(n);
+    for (uint64_t i = 0; i < n; i++) at[i] = i;
+    std::sort(at.begin(), at.end(), [&](uint64_t a, uint64_t b) {
+        return hq[a] != hq[b] ? hq[a] < hq[b] : he[a] < he[b];
+    });
+    for (uint64_t i = 0; i < n; i++) {
+        if (q) q[i] = hq[at[i]];
+        if (e) e[i] = he[at[i]];
+        if (tin) tin[i] = ha[at[i]];
+        if (tout) tout[i] = hb[at[i]];
+    }
+    return TS_OK;
 }
 
 // The query columns of stationary points: x0 = x1 = x (likewise y, z), t0 = t_start, t1 = t_end.

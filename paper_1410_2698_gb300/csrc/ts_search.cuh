@@ -132,12 +132,15 @@ struct SearchOut {
     uint64_t count = 0;
     uint32_t *q = nullptr, *e = nullptr;
     double *tin = nullptr, *tout = nullptr;
+    uint64_t n_entries = 0;  // entry indices are below this (0: not known)
     ts_search_stats stats{};
 };
 
 constexpr uint64_t ROW_BYTES = 24;  // q_idx, e_idx, t_in, t_out
-bool copy_few_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
-                   cudaStream_t s, ts_status *st);
+bool copy_few_rows(const SearchOut &o, const uint32_t *order, uint32_t *q, uint32_t *e, double *tin,
+                   double *tout, cudaStream_t s, ts_status *st);
+ts_status copy_sorted_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
+                           cudaStream_t s);
 
 const char *last_error();
 unsigned long long launch_count();
@@ -183,7 +186,7 @@ struct ArrayPtrs {
 };
 constexpr int KEY_LO_BITS = 13;
 constexpr int KEY_LO_MIN = 11;
-KeyFmt key_fmt(const Index *ix, uint32_t nreq);
+KeyFmt key_fmt(const Index *ix, const PipeCaps &c);
 ts_status search_brute_noalloc(const ts_segments *db, const ts_segments *q,
                                const ts_query_params *qp, uint32_t *q_idx, uint32_t *e_idx,
                                double *t_in, double *t_out, uint64_t capacity, uint64_t *count,

@@ -278,6 +278,7 @@ void write_done(Server *s, Slot &sl)
             q->out.count = n;
             q->out.stats.n_queries = q->n;
             q->out.stats.n_hits = n;
+            q->out.n_entries = s->ix->n;
             if (n) {
                 q->out.q = sl.block->q + a;
                 q->out.e = sl.block->e + a;

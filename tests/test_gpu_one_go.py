@@ -150,3 +150,27 @@ def test_rows_to_host(n):
     only = np.empty(n, np.uint32)  # a destination of its own, the others left out
     _lib.check(lib.ts_result_copy_to_host(res.handle, None, only.ctypes.data, None, None, None))
     assert np.array_equal(only, host["e_idx"])
+
+
+@pytest.mark.parametrize("nq,box", [(1, 4.0), (3, 8.0), (40, 12.0), (300, 20.0), (2000, 12.0)])
+@pytest.mark.parametrize("kind", ["spatiotemporal", "spatial"])
+def test_rows_sorted_on_the_device(nq, box, kind):
+    """Rows by (query, entry) as numpy sorts them: few (sorted by the host, or through a slot) and
+    many, of a search and of a batch, also one field alone."""
+    rng = np.random.default_rng(nq)
+    db = random_segments(rng, 3000, box=box)
+    q = random_segments(rng, nq, box=box)
+    idx = api.ts_build_index(db, kind=kind)
+    lib = _lib.load()
+    for res in (api.ts_search(idx, q, 2.0, 0.0, 12.0),
+                api.ts_search_batch(idx, [(q, 1.0, 0.0, 12.0), (q, 2.0, 0.0, 12.0)])[1]):
+        rows = res.to_host()
+        order = np.lexsort((rows["e_idx"], rows["q_idx"]))
+        got = res.to_host(sort=True)
+        assert rows["q_idx"].size == res.count > 0
+        for k, v in rows.items():
+            assert np.array_equal(got[k], v[order]), k
+        only = np.empty(res.count)
+        _lib.check(lib.ts_result_copy_sorted_to_host(res.handle, None, None, None,
+                                                     only.ctypes.data, None))
+        assert np.array_equal(only, rows["t_out"][order])
