@@ -1463,10 +1463,13 @@ KeyFmt key_fmt(const Index *ix, const PipeCaps &c)
         f.lo_bits = std::min(full, std::max(KEY_LO_MIN, std::min(KEY_LO_BITS, 16 - head)));
     } else {
         // three radix passes: as many of the start's top bits as tell the bins (or a subbin's bins)
-        // apart, and the query's place
+        // apart, and the query's place; two passes where the pair kernel has too little to do for
+        // the place to pay for the third (10,764 walk queries: it took 28 us either way)
+        const int all = c.nq > 16384 ? 24 : 16;
         const int tell = bits_for(ix->m - 1) + 1 + (f.sel_bits ? 4 : 0);
-        f.lo_bits = std::min(full, std::min(KEY_LO_BITS, tell));
-        f.morton = std::max(2, std::min(6, (24 - head - f.lo_bits) / 3));
+        f.lo_bits = std::min(full, std::min(KEY_LO_BITS, std::max(1, std::min(tell, all - head))));
+        if (all == 16 && nreq > 32) f.lo_bits = std::min(full, std::max(f.lo_bits, 8));
+        f.morton = std::max(all == 16 ? 0 : 2, std::min(6, (all - head - f.lo_bits) / 3));
     }
     f.lo_shift = full - f.lo_bits;
     return f;
