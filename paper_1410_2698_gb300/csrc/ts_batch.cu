@@ -218,7 +218,12 @@ ts_status create_plan(const Index *ix, const ts_batch_params *prm, cudaStream_t 
         TS_CUDA(cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking));
         p->own_stream = true;
     }
-    TS_CUDA(cudaMemsetAsync(p->dmem, 0, p->dbytes, p->stream));
+    // zeros where something is read that no run wrote: the caller's view of the rows and the control
+    // words, the end of the memory (a run writes all else that it reads)
+    unsigned char *rest = reinterpret_cast<unsigned char *>(
+        own_rows ? static_cast<void *>(p->b.out_q) : static_cast<void *>(p->b.hdr));
+    TS_CUDA(cudaMemsetAsync(rest, 0, static_cast<unsigned char *>(p->dmem) + p->dbytes - rest,
+                            p->stream));
     TS_CUDA(cudaStreamSynchronize(p->stream));
     TS_CUDA(cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming));
     *out = p.release();
