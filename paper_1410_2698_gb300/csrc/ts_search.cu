@@ -21,9 +21,8 @@
 //   2. FP32 gap test: squared MBB distance accumulated rounding down against an upper bound of
 //      d^2 (run only when some lane passed stage 1); a pair is dropped only when a lower bound
 //      of its separation exceeds d, so no pair the FP64 test could accept is ever dropped;
-//   3. the exact FP64 test on the survivors (the closed form of the interaction with explicit
-//      fused multiply-adds; a hit's square root and quotients from refined hardware estimates),
-//      run 32 at a time on survivors compacted with ballot/popc so the FP64 pipe runs full warps.
+//   3. the exact test on the survivors (the closed form of the interaction, in FP64 and in pairs of
+//      FP32 values; ts_device.cuh), run 32 at a time on survivors compacted with ballot/popc.
 #include <math.h>
 
 #include <algorithm>
@@ -62,28 +61,50 @@ __device__ __forceinline__ uint32_t req_of(const ReqDesc *reqs, uint32_t nreq, u
     return lo;
 }
 
-__device__ __forceinline__ uint32_t first_pmax_above(const double *pmax, uint32_t m, double w0)
+// Query preparation compares FP64 values by their order keys and rounds them to FP32 on the integer
+// pipe; what is left to the FP64 pipe (2 lanes a clock and SM) are the velocities' divisions and the
+// expanded extents. 800,000 query segments on the grid 194 -> 162 us, 100,000 on subbins 38 -> 31.
+__device__ __forceinline__ bool finite_bits(double x)
+{
+    return ((uint32_t)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
+// x rounded to FP32 toward -inf (up = false) or +inf: truncated, and one step away from 0 when
+// something was cut off on that side. Zero and what lies outside FP32's normal range: converted.
+__device__ __forceinline__ float round_f32(double x, bool up)
+{
+    const long long u = dbits(x);
+    const uint32_t hi = (uint32_t)((unsigned long long)u >> 32), lo = (uint32_t)u;
+    if (((hi >> 20) & 0x7ffu) - 897u > 253u) return up ? __double2float_ru(x) : __double2float_rd(x);
+    const uint32_t f = ((__funnelshift_l(lo, hi, 3) & 0x7fffffffu) ^ 0x40000000u) |
+                       (hi & 0x80000000u);
+    const bool away = (lo & 0x1fffffffu) != 0 && (u < 0) != up;
+    return __uint_as_float(f + (away ? 1u : 0u));
+}
+
+__device__ __forceinline__ uint32_t first_pmax_above(const double *pmax, uint32_t m, uint64_t w0)
 {
     uint32_t lo = 0, hi = m;
     while (lo < hi) {
         uint32_t mid = lo + (hi - lo) / 2;
-        if (pmax[mid] > w0) hi = mid; else lo = mid + 1;
+        if (dkey(pmax[mid]) > w0) hi = mid; else lo = mid + 1;
     }
     return lo;
 }
 
 // The part of x (as part_of) from the partition's boundary table bd[j] = lo + j*w: a first guess
-// in FP32 (iwf ~ 1/w; 0 when w = 0), corrected by the exact FP64 boundary comparisons, so the
+// in FP32 (iwf ~ 1/w; 0 when w = 0), corrected by exact comparisons with the boundaries, so the
 // result equals part_of's.
 __device__ __forceinline__ int part_of_t(double x, const double *bd, float iwf, int v)
 {
     const double lo = bd[0];
-    if (!(x >= lo)) return -1;
+    const uint64_t kx = dkey(x);
+    if (kx < dkey(lo)) return -1;
     if (v <= 1 || iwf == 0.0f) return v - 1;
     const float f = floorf((float)(x - lo) * iwf);
     int j = !(f < (float)v) ? v - 1 : (f < 0.0f ? 0 : (int)f);
-    while (j + 1 < v && bd[j + 1] <= x) j++;
-    while (j > 0 && bd[j] > x) j--;
+    while (j + 1 < v && dkey(bd[j + 1]) <= kx) j++;
+    while (j > 0 && dkey(bd[j]) > kx) j--;
     return j;
 }
 
@@ -96,15 +117,16 @@ __device__ __forceinline__ uint32_t first_pmax_above_b(const double *pmax, const
                                                        double w0)
 {
     const int jw = part_of_t(w0, bs, iwf, (int)m);
-    if (jw < 0) return first_pmax_above(pmax, 1, w0);  // before every bin: 0 or (m = 1) 1
+    const uint64_t k0 = dkey(w0);
+    if (jw < 0) return first_pmax_above(pmax, 1, k0);  // before every bin: 0 or (m = 1) 1
     uint32_t hi = (uint32_t)jw + 1 < m ? (uint32_t)jw + 1 : m;
     uint32_t lo = (uint32_t)jw > back ? (uint32_t)jw - back : 0u;
-    if (lo > 0 && pmax[lo - 1] > w0) lo = 0;
+    if (lo > 0 && dkey(pmax[lo - 1]) > k0) lo = 0;
     // the answer lies in [lo, hi]; hi = m means no bin
-    if (hi == m && !(pmax[m - 1] > w0)) return m;
+    if (hi == m && !(dkey(pmax[m - 1]) > k0)) return m;
     while (lo < hi) {
         const uint32_t mid = lo + (hi - lo) / 2;
-        if (pmax[mid] > w0) hi = mid; else lo = mid + 1;
+        if (dkey(pmax[mid]) > k0) hi = mid; else lo = mid + 1;
     }
     return lo;
 }
@@ -114,7 +136,8 @@ __device__ __forceinline__ int last_start_below_t(const double *bs, uint32_t m, 
                                                   double w1)
 {
     int j = part_of_t(w1, bs, iwf, (int)m);
-    while (j >= 0 && !(bs[j] < w1)) j--;
+    const uint64_t k1 = dkey(w1);
+    while (j >= 0 && !(dkey(bs[j]) < k1)) j--;
     return j;
 }
 
@@ -218,38 +241,40 @@ __global__ void k_qprep(PrepParams P)
 #pragma unroll
         for (int k = 0; k < 8; k++) {
             v[k] = P.f[0] ? P.f[k][i] : R.cols[k][li];
-            fin = fin && isfinite(v[k]);
+            fin = fin && finite_bits(v[k]);
         }
-        if (!fin || !(v[7] > v[3])) atomicOr(P.b.status, DEV_ERR_INVALID);
+        const bool ok = fin && dkey(v[7]) > dkey(v[3]);
+        if (!ok) atomicOr(P.b.status, DEV_ERR_INVALID);
         const double dt = v[7] - v[3];
         QueryD q;
         q.vx = (v[4] - v[0]) / dt;
         q.vy = (v[5] - v[1]) / dt;
         q.vz = (v[6] - v[2]) / dt;
-        q.w0 = dmx(v[3], R.t_start);
-        q.w1 = dmn(v[7], R.t_end);
+        q.w0 = dkey(v[3]) > dkey(R.t_start) ? v[3] : R.t_start;
+        q.w1 = dkey(v[7]) < dkey(R.t_end) ? v[7] : R.t_end;
         const double dw = q.w0 - v[3];  // 0 unless the request interval clips the start
         q.xw = fma(q.vx, dw, v[0]);
         q.yw = fma(q.vy, dw, v[1]);
         q.zw = fma(q.vz, dw, v[2]);
         q.ndd = -R.dd;
         q.pad[0] = q.pad[1] = q.pad[2] = 0.0;
-        const bool valid = fin && (v[7] > v[3]) && (q.w0 < q.w1);
+        const bool valid = ok && dkey(q.w0) < dkey(q.w1);
         P.b.qd[i] = q;
         P.b.qreq[i] = r;
         double mn[3], mx[3];
         float fmn[3], fmx[3];
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            mn[d] = v[d] < v[4 + d] ? v[d] : v[4 + d];
-            mx[d] = v[d] < v[4 + d] ? v[4 + d] : v[d];
-            fmn[d] = __double2float_rd(mn[d]);
-            fmx[d] = __double2float_ru(mx[d]);
+            const bool up = dkey(v[d]) < dkey(v[4 + d]);
+            mn[d] = up ? v[d] : v[4 + d];
+            mx[d] = up ? v[4 + d] : v[d];
+            fmn[d] = round_f32(mn[d], false);
+            fmx[d] = round_f32(mx[d], true);
         }
         P.b.qf[2 * i + 0] = make_float4(__fsub_rd(fmn[0], R.d_up), __fsub_rd(fmn[1], R.d_up),
-                                        __fsub_rd(fmn[2], R.d_up), __double2float_rd(q.w0));
+                                        __fsub_rd(fmn[2], R.d_up), round_f32(q.w0, false));
         P.b.qf[2 * i + 1] = make_float4(__fadd_ru(fmx[0], R.d_up), __fadd_ru(fmx[1], R.d_up),
-                                        __fadd_ru(fmx[2], R.d_up), __double2float_ru(q.w1));
+                                        __fadd_ru(fmx[2], R.d_up), round_f32(q.w1, true));
 
         uint32_t sel = SEL_T, lo = 0, hi = 0;
         bool subbin = false, unit = false;
