@@ -41,16 +41,16 @@ INTERVAL_FLOPS = 10  # FP64 flops per hit for the roots (sqrt, 2 div, clamps; sq
 # dram__bytes_write.sum; the gathered FP64 records and the kept hits). The merger-like workload at
 # a tenth of the particles (merger-like-2m) stands in for the full one, whose launches are too
 # large to capture: the per-unit counts are those of the same kernel at the same hit ratio.
-_MERGER_PROFILE = {"fp64_inst_per_exact": 33.84, "warp_inst_per_test": 0.4961,
-                   "dram_bytes_per_exact": 62.02, "hit_ratio": 0.8697,
+_MERGER_PROFILE = {"fp64_inst_per_exact": 15.74, "warp_inst_per_test": 0.4728,
+                   "dram_bytes_per_exact": 64.63, "hit_ratio": 0.8697,
                    "capture": "profiles/k_pair_merger-like-2m_count-pass.md",
-                   "sources": "2cf662d8c6ac49b1"}
+                   "sources": "e452e00c9567bcdf"}
 # the Random-walk 1M workload (filter-bound: the issue slots bind); its DRAM bytes are mostly the
 # records the sweep streams, scaled here by the exact tests of the same workload
-_RW1M_PROFILE = {"fp64_inst_per_exact": 8.80, "warp_inst_per_test": 0.5090,
-                 "dram_bytes_per_exact": 438.6, "hit_ratio": 0.348,
+_RW1M_PROFILE = {"fp64_inst_per_exact": 5.67, "warp_inst_per_test": 0.6133,
+                 "dram_bytes_per_exact": 478.4, "hit_ratio": 0.348,
                  "capture": "profiles/k_pair_random-walk-1m_count-pass.md",
-                 "sources": "2cf662d8c6ac49b1"}
+                 "sources": "e452e00c9567bcdf"}
 PAIR_PROFILE = {"merger-like-20m": _MERGER_PROFILE, "merger-like-2m": _MERGER_PROFILE,
                 "random-walk-1m": _RW1M_PROFILE}
 PAIR_SOURCES = ("ts_search.cuh", "ts_internal.cuh", "ts_device.cuh")
@@ -224,8 +224,8 @@ def device_info(dev):
 
 
 def roofline(tot, pair_ms, peaks, workload, dev_info):
-    """Roofline of the pair kernel (its count and write passes, timed by the CUDA events its plans
-    record around them inside the timed step). The kernel's work runs on two pipes: the FP64 pipe
+    """Roofline of the pair kernel (its count and write passes, timed by the device clock that its
+    plans read around them inside the timed step). The kernel's work runs on two pipes: the FP64 pipe
     (the exact tests; the FP32 filters decide every other candidate) and the issue slots of the SM
     sub-partitions (the FP32 filters' sweep). For each, achieved = the instructions the kernel
     issued for this step's work (per-unit counts from the ncu capture of the same sources, times
@@ -461,7 +461,7 @@ def run_gpu(args):
         l2 = api.ts_kernel_launches()
 
         # the pair kernel timed alone: the same plans, one at a time on the bench stream (in
-        # the overlapped step the events of one plan also see the other plans' kernels)
+        # the overlapped step the clock of one plan also sees the other plans' kernels)
         def alone_step():
             for k in kinds:
                 plans[k].run(preq)
@@ -548,15 +548,15 @@ def run_gpu(args):
         for key in e:
             e[key] = e[key] / n_alone
     # roofline of the dominant kernel: the batched pair kernel (count + write passes), timed by
-    # the CUDA events each plan records around its passes on its stream. With the plans run one
-    # at a time these are the timed headline step's own events; with overlapped plans (where a
-    # plan's events also span the other plans' kernels) a loop of the same plans one at a time.
+    # the device clock that each plan reads around its passes. With the plans run one at a time
+    # these are the timed headline step's own; with overlapped plans (where a plan's passes also
+    # span the other plans' kernels) a loop of the same plans one at a time.
     step_tot = {k: v / n_alone for k, v in atot.items()}  # per step
     step_tot["launches"] = len(kinds)  # count passes (one per plan)
     roof = roofline(step_tot, apair_ms / n_alone, peaks, w.name, dinfo)
     if serial:
         roof["timed_form"] = ("batched, the timed headline step itself (plans one at a time; "
-                              "CUDA events of each plan around its pair-kernel passes)")
+                              "device clock of each plan around its pair-kernel passes)")
     else:
         roof["timed_form"] = "batched, one plan at a time (a loop of the headline step's plans)"
     roof["pair_kernel_share"] = apair_ms / sum(alone_ms) if alone_ms else None
