@@ -290,10 +290,13 @@ static __device__ __forceinline__ bool quad_solve(const Quad &k, bool interval, 
 // range where no product of the test leaves FP32 go through the FP64 code above instead (a few
 // pairs in 100,000), so the decisions are those of FP64.
 //
-// Of 2,000,000 random pairs at each of ten settings of d, step and window, no decision differs from
-// 113-bit arithmetic's, and the intervals are nearer to it than the FP64 code's, whose quotients
-// carry 40 bits: rms 1e-15 to 1.5e-14 of the window against 2.6e-14 to 2.6e-13, largest 5e-14 to
-// 3.7e-13 against 8e-13 to 2.1e-12.
+// Against 113-bit arithmetic no decision differs, and the intervals are as near to it as the FP64
+// code's, whose quotients carry 40 bits, or nearer (errors as shares of the window, 1,000,000
+// random pairs each on the host, FP64 in brackets): at ten settings of d, step and window rms 1e-15
+// to 1.1e-14 (1.6e-15 to 2.6e-13), largest 6e-14 to 1.1e-12 (7e-13 to 2.1e-12); roots within two
+// FP32 ulps of the window's end rms 3.4e-14 (3.9e-13), largest 1.0e-12 (2.2e-12). Where the pair
+// hardly moves (a hundredth of d in a window and less), both are as far off as the rounding of c
+// puts them: 5e-11 at a hundredth, 4e-10 at a thousandth.
 // 16 FP64 instructions a hit instead of 34; 1.13 G exact tests (merger, 20M segments, d = 1 and 5):
 // pair kernel 106.7 -> 100.5 ms.
 struct Ff {
@@ -454,11 +457,16 @@ static __device__ __forceinline__ int rel_test(const Rel &k, double ndd, bool in
         const Ff s = ff_add(b, bneg ? ff_neg(sq) : sq);  // minus the stable root's numerator
         const Ff r1 = ff_div(ff_neg(s), a), r2 = ff_div(ff_neg(c), s);
         const Ff lo = bneg ? r2 : r1, hi = bneg ? r1 : r2;
-        const bool clip = hi.h > T.h || (hi.h == T.h && hi.l >= T.l);
         const bool from = lo.h > 0.0f;
         if ((from && lo.h < 8.5e-22f) || !(hi.h >= 8.5e-22f)) return -1;  // (2^-70)
         if (from) lower = ff_double(lo);
-        if (!clip) upper = ff_double(hi);
+        // the root against the window's end as FP64 values: the pair T is cut off (l up to an ulp
+        // of h) where a root's is rounded (l up to half of one), so high parts of two neighbouring
+        // values may stand in the other order than the values (2 T: ff_double's range)
+        if (hi.h < 2.0f * T.h) {
+            const double end = ff_double(hi);
+            if (dbits(end) < dbits(upper)) upper = end;
+        }
         if (dbits(upper) < dbits(lower)) upper = lower;  // (within rounding only)
     }
     *tin = k.t_lo + lower;

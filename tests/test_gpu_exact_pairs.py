@@ -76,3 +76,27 @@ def test_windows(window):
     q = random_segments(rng, 150, box=8.0, t_range=(4.0, 5.0), max_len=6.0)
     ref, _ = _both(db, q, 1.5, 5.5, 5.5 + window)
     assert ref["q_idx"].size > 0
+
+
+@pytest.mark.parametrize("end", ["in", "out"])
+@pytest.mark.parametrize("near", ["start", "end"])
+def test_roots_at_the_ends_of_the_window(end, near):
+    """Entries that come within d (in) or leave (out) within two FP32 ulps of the ends of windows whose
+    lengths have 53 random bits, on both sides of them: the pairs' high parts alone do not order a
+    root and the window's end. One pair per place of a lattice, so a query meets one entry."""
+    rng = np.random.default_rng(29)
+    n, d = 15 ** 3, 1.0
+    place = 16.0 * np.stack(np.meshgrid(*[np.arange(15.0)] * 3), axis=-1).reshape(n, 3)
+    T = rng.uniform(0.1, 2.0, n)
+    root = rng.uniform(-2, 2, n) * np.spacing(T.astype(np.float32)).astype(float)
+    if near == "end":
+        root += T
+    u, v = rng.normal(size=(2, n, 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    # the separation grows at the root (out) or shrinks (in)
+    v *= np.where((np.sum(u * v, axis=1) > 0) == (end == "out"), 1.0, -1.0)[:, None]
+    p0 = place + d * u - v * (root + 1.0)[:, None]  # at time -1
+    q = Segments.from_matrix(np.column_stack([place, np.zeros(n), place, T]))
+    db = Segments.from_matrix(np.column_stack([p0, np.full(n, -1.0), p0 + 4.0 * v, np.full(n, 3.0)]))
+    ref, out = _both(db, q, d, -1.0, 3.0)
+    assert n // 4 < ref["q_idx"].size <= n and out["worst_out"] < 1e-9
