@@ -322,6 +322,30 @@ def _max_over_ranks(x, world, dev):
     return float(t.item())
 
 
+def plan_tiles(plain_tiles, tile_records):
+    """Tiles a plan makes room for where plain searches of its requests, in tiles of 256 records,
+    took `plain_tiles`: a range of so many tiles takes at most ceil(256 / tile_records) times as
+    many of tile_records, and 10 % more for groups of other queries (a plan sorts all its requests
+    at once)."""
+    t = plain_tiles * -(-256 // (tile_records or 256))
+    return t + t // 10 + 65536
+
+
+def fitting_plan(make, run, tiles, tries=3):
+    """make(max_tiles), grown until run(plan), a run's outcome, reports no overflow."""
+    for _ in range(tries):
+        plan = make(tiles)
+        st = run(plan)
+        if not st["overflow"]:
+            return plan
+        plan.free()
+        need = st["stats"]["n_tiles"]
+        if need <= tiles:
+            raise RuntimeError(f"batch plan overflow: {st['rows']} rows in {need} tiles")
+        tiles = need + need // 10
+    raise RuntimeError(f"batch plan overflow: {tiles} tiles")
+
+
 def run_gpu(args):
     import torch
     import torch.distributed as dist
@@ -412,12 +436,20 @@ def run_gpu(args):
             max(1 << 20, 2 * rows_per_batch[k])
         if pair_blocks is None:  # an explicit --pair-blocks overrides the tuned grid
             pair_blocks = args.pair_blocks or (tuned[k]["pair_blocks"] if k in tuned else 0)
-        return api.BatchPlan(indexes[k], max_requests=len(reqs),
-                             max_queries=w.queries.n * len(reqs), max_rows=rows, use_graph=True,
-                             stream=0 if own_stream else None,
-                             tile_records=tuned[k]["tile_records"] if k in tuned else args.tile,
-                             pair_blocks=pair_blocks, max_units=units[k],
-                             max_tiles=tiles_per_batch[k] + tiles_per_batch[k] // 10 + 65536)
+        tile = tuned[k]["tile_records"] if k in tuned else args.tile
+
+        def make(tiles):
+            return api.BatchPlan(indexes[k], max_requests=len(reqs),
+                                 max_queries=w.queries.n * len(reqs), max_rows=rows,
+                                 use_graph=True, stream=0 if own_stream else None,
+                                 tile_records=tile, pair_blocks=pair_blocks, max_units=units[k],
+                                 max_tiles=tiles)
+
+        def run(plan):
+            plan.run(preq, stream=0 if own_stream else None)
+            return plan.wait()
+
+        return fitting_plan(make, run, plan_tiles(tiles_per_batch[k], tile))
 
     batch_stats = []
     alone = []
@@ -476,16 +508,15 @@ def run_gpu(args):
         for k in kinds:
             plan = make_plan(k, False)
 
-            def one(plan=plan, k=k):
+            def one(plan=plan, k=k, collect=batch_stats):
                 plan.run(preq)
                 st = plan.wait()
                 if st["overflow"]:
                     raise RuntimeError(f"batch plan overflow for {k}")
-                batch_stats.append((k, st))
+                collect.append((k, st))
 
             for _ in range(max(args.warmup, 0)):
-                plan.run(preq)
-                plan.wait()
+                one(collect=[])
             n0 = len(batch_stats)
             a = api.ts_kernel_launches()
             for i, v in enumerate(_timed(args, stream, flush, one)):
