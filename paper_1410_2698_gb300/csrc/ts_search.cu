@@ -186,6 +186,11 @@ __device__ __forceinline__ uint64_t unit_key(uint32_t r, uint32_t sel, uint32_t 
     return (k << (3 * f.morton)) | code;
 }
 
+// Lookup tables that k_qprep copies into shared memory: what the 48 KB a launch may ask for without
+// an opt-in leave beside the kernel's own static arrays (the limit is on both together).
+constexpr int QP_COUNTS = 2;
+constexpr uint64_t QP_TABLE_BYTES = 48 * 1024 - QP_COUNTS * 32 * sizeof(uint32_t);
+
 __global__ void k_qprep(PrepParams P)
 {
     // the bin, subbin and cell boundary tables the lookups read, copied into shared memory (one
@@ -375,7 +380,7 @@ __global__ void k_qprep(PrepParams P)
         }
     }
     // the block's counts: one atomic per counter and block
-    __shared__ uint32_t red[2][32];
+    __shared__ uint32_t red[QP_COUNTS][32];
     const int warp = threadIdx.x >> 5, lane0 = threadIdx.x & 31;
     for (int o = 16; o; o >>= 1) {
         n_valid += __shfl_xor_sync(0xffffffffu, n_valid, o);
@@ -386,7 +391,7 @@ __global__ void k_qprep(PrepParams P)
         red[1][warp] = n_subbin;
     }
     __syncthreads();
-    if (threadIdx.x < 2) {
+    if (threadIdx.x < QP_COUNTS) {
         unsigned long long v = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) v += red[threadIdx.x][w];
         if (v) atomicAdd(&P.b.stats[threadIdx.x == 0 ? ST_QSEGS : ST_SUBBIN], v);
@@ -1560,7 +1565,7 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
     }
     P.g = ix->g;
     P.b = b;
-    // lookup tables in shared memory when they fit the default 48 KB
+    // lookup tables in shared memory when they fit
     uint64_t tb = 0;
     if (ix->kind == TS_INDEX_SPATIAL) {
         tb = 3ull * 8 * ((uint64_t)ix->g + 1);
@@ -1569,7 +1574,7 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
         if (ix->kind == TS_INDEX_SPATIOTEMPORAL)
             for (int d = 0; d < 3; d++) tb += 8ull * ((uint64_t)ix->v[d] + 1);
     }
-    P.smem_bytes = tb <= 48 * 1024 ? (uint32_t)tb : 0u;
+    P.smem_bytes = tb <= QP_TABLE_BYTES ? (uint32_t)tb : 0u;
     if (nq) {
         TS_LAUNCH_PDL(k_qprep, dim3(nblk(nq)), dim3(TPB), P.smem_bytes, s,
                       P);
