@@ -417,6 +417,11 @@ ts_status ts_eval_refined_estimates(const double *x, uint64_t n, double *rcp_est
  * search returns TS_ERR_TIMEOUT. Batch plans and the served loop are not affected. */
 ts_status ts_debug_inject_stall(uint64_t limit_ns);
 
+/* Test hook of what calls do when device memory is short (the paper has no counterpart): of the
+ * calling thread's allocations from the library's pool, `count` fail as if out of memory after the
+ * next `after` have been made (count = 0: none). No allocation is attempted for those. */
+ts_status ts_debug_fail_allocs(uint64_t after, uint64_t count);
+
 /* Library version string. */
 const char *ts_version(void);
 

@@ -323,6 +323,11 @@ def ts_debug_inject_stall(limit_ns: int) -> None:
     check(_lib.load().ts_debug_inject_stall(int(limit_ns)))
 
 
+def ts_debug_fail_allocs(after: int, count: int) -> None:
+    """Test hook: `count` of this thread's device allocations fail after the next `after`."""
+    check(_lib.load().ts_debug_fail_allocs(int(after), int(count)))
+
+
 def ts_kernel_launches() -> int:
     return int(_lib.load().ts_kernel_launches())
 

@@ -108,6 +108,12 @@ ts_status ts_debug_inject_stall(uint64_t limit_ns)
     return clear_error(TS_OK);
 }
 
+ts_status ts_debug_fail_allocs(uint64_t after, uint64_t count)
+{
+    fail_allocs(after, count);
+    return clear_error(TS_OK);
+}
+
 uint64_t ts_kernel_launches(void) { return (uint64_t)ts::launch_count(); }
 
 ts_status ts_search_brute_noalloc(const ts_segments *db, const ts_segments *q,

@@ -207,6 +207,9 @@ inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t
 // Stream-ordered allocation from the library's pool (freed blocks stay pooled); inside a stream
 // capture a graph memory node. Release with cudaFreeAsync.
 cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream);
+// Tests of what a search does short of memory: of this thread's calls of pool_malloc, `count` fail
+// after the next `after`.
+void fail_allocs(uint64_t after, uint64_t count);
 // Return the pool's unused memory of the current device, but for `keep` bytes, to the device
 // (synchronises it).
 void pool_trim(size_t keep = 0);

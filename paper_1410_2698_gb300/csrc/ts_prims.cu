@@ -87,8 +87,26 @@ void pool_trim(size_t keep)
     cudaGetLastError();
 }
 
+// Allocations of this thread until the ones that a test lets fail, and how many those are.
+static thread_local uint64_t g_fail_after = 0, g_fail_count = 0;
+
+void fail_allocs(uint64_t after, uint64_t count)
+{
+    g_fail_after = after;
+    g_fail_count = count;
+}
+
 cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream)
 {
+    if (g_fail_count) {
+        if (g_fail_after) {
+            g_fail_after--;
+        } else {
+            g_fail_count--;
+            *p = nullptr;
+            return cudaErrorMemoryAllocation;
+        }
+    }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(stream, &cs);
     cudaMemPool_t pool = cs == cudaStreamCaptureStatusNone ? work_pool() : nullptr;

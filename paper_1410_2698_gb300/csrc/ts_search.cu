@@ -2343,10 +2343,43 @@ bool copy_few_rows(const SearchOut &o, const uint32_t *order, uint32_t *q, uint3
     return true;
 }
 
+// copy_sorted_rows on the device; *done stays false where its memory does not reach for that.
+static ts_status sort_rows_here(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin,
+                                double *tout, cudaStream_t s, bool *done)
+{
+    const uint64_t n = o.count;
+    const int eb = o.n_entries ? bits_for(o.n_entries - 1) : 32;
+    const int qb = o.stats.n_queries ? bits_for(o.stats.n_queries - 1) : 32;
+    DevBuf keys, vals, rows;
+    TS_CHECK(keys.alloc(8 * n, s));
+    TS_CHECK(vals.alloc(4 * n, s));
+    TS_LAUNCH_PDL(k_row_keys, dim3(nblk(n)), dim3(TPB), 0, s, n, o.q, o.e, eb,
+                  keys.as<uint64_t>(), vals.as<uint32_t>());
+    TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, eb + qb, s, nullptr,
+                            false));
+    keys.release();
+    ts_status few = TS_OK;
+    *done = copy_few_rows(o, vals.as<uint32_t>(), q, e, tin, tout, s, &few);
+    if (*done) return few;
+    TS_CHECK(rows.alloc(ROW_BYTES * n, s));
+    double *d = rows.as<double>();
+    uint32_t *w = reinterpret_cast<uint32_t *>(d + 2 * n);
+    TS_LAUNCH_PDL(k_rows_out, dim3(nblk(n)), dim3(TPB), 0, s, n, vals.as<uint32_t>(), o.q, o.e,
+                  o.tin, o.tout, d);
+    if (tin) TS_CUDA(cudaMemcpyAsync(tin, d, 8 * n, cudaMemcpyDeviceToHost, s));
+    if (tout) TS_CUDA(cudaMemcpyAsync(tout, d + n, 8 * n, cudaMemcpyDeviceToHost, s));
+    if (q) TS_CUDA(cudaMemcpyAsync(q, w, 4 * n, cudaMemcpyDeviceToHost, s));
+    if (e) TS_CUDA(cudaMemcpyAsync(e, w + n, 4 * n, cudaMemcpyDeviceToHost, s));
+    TS_CUDA(cudaStreamSynchronize(s));
+    *done = true;
+    return TS_OK;
+}
+
 // Rows to the host by (query, entry): sorted on the device (the two indices are one key of as many
 // bits as queries and entries take; no two rows have the same) and copied from one block. Rows of
-// another device, or more than the device's memory can sort, are sorted here. 15,000 rows, sorted
-// by numpy from the host's copy before: 1147 -> 433 us with their search.
+// another device, or more than the device's memory can sort (25 B a row, then 28 with the block of
+// sorted rows), are sorted here. 15,000 rows, sorted by numpy from the host's copy before: 1147
+// -> 433 us with their search.
 ts_status copy_sorted_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double *tin, double *tout,
                            cudaStream_t s)
 {
@@ -2355,27 +2388,10 @@ ts_status copy_sorted_rows(const SearchOut &o, uint32_t *q, uint32_t *e, double 
         TS_CUDA(cudaStreamSynchronize(s));
         return TS_OK;
     }
-    DevBuf keys, vals, rows;
-    if (n <= 0xffffffffull && rows_here(o) && keys.alloc(8 * n, s) == TS_OK &&
-        vals.alloc(4 * n, s) == TS_OK && rows.alloc(ROW_BYTES * n, s) == TS_OK) {
-        const int eb = o.n_entries ? bits_for(o.n_entries - 1) : 32;
-        const int qb = o.stats.n_queries ? bits_for(o.stats.n_queries - 1) : 32;
-        TS_LAUNCH_PDL(k_row_keys, dim3(nblk(n)), dim3(TPB), 0, s, n, o.q, o.e, eb,
-                      keys.as<uint64_t>(), vals.as<uint32_t>());
-        TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, eb + qb, s, nullptr,
-                                false));
-        ts_status few = TS_OK;
-        if (copy_few_rows(o, vals.as<uint32_t>(), q, e, tin, tout, s, &few)) return few;
-        double *d = rows.as<double>();
-        uint32_t *w = reinterpret_cast<uint32_t *>(d + 2 * n);
-        TS_LAUNCH_PDL(k_rows_out, dim3(nblk(n)), dim3(TPB), 0, s, n, vals.as<uint32_t>(), o.q, o.e,
-                      o.tin, o.tout, d);
-        if (tin) TS_CUDA(cudaMemcpyAsync(tin, d, 8 * n, cudaMemcpyDeviceToHost, s));
-        if (tout) TS_CUDA(cudaMemcpyAsync(tout, d + n, 8 * n, cudaMemcpyDeviceToHost, s));
-        if (q) TS_CUDA(cudaMemcpyAsync(q, w, 4 * n, cudaMemcpyDeviceToHost, s));
-        if (e) TS_CUDA(cudaMemcpyAsync(e, w + n, 4 * n, cudaMemcpyDeviceToHost, s));
-        TS_CUDA(cudaStreamSynchronize(s));
-        return TS_OK;
+    if (n <= 0xffffffffull && rows_here(o)) {
+        bool done = false;
+        const ts_status st = sort_rows_here(o, q, e, tin, tout, s, &done);
+        if (done || (st != TS_OK && st != TS_ERR_OOM)) return st;
     }
     std::vector<uint32_t> hq(n), he(n);
     std::vector<double> ha(n), hb(n);
