@@ -2049,8 +2049,8 @@ ts_status alloc_rows(SearchOut *out, uint64_t n, cudaStream_t s, PipeBufs &b)
 // Bound: launches and their latency. A search of 20 query segments against 20,000 (34 calls to the
 // allocator, 12 pageable copies, four waits, 18 kernels before) 327 -> 207 us, of 10,000
 // against 1M on the grid 395 -> 245 us, with the binding and the copies of the rows.
-ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_params *qp,
-                        cudaStream_t s, SearchOut *out, bool *done)
+ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_params *qp,
+                       cudaStream_t s, SearchOut *out, bool *done)
 {
     const uint64_t nq = q->n;
     const bool grid = ix->kind == TS_INDEX_SPATIAL;
@@ -2167,6 +2167,21 @@ ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_pa
     TS_CHECK(read_dev_status(o.status));
     fill_stats(o.stats, &out->stats);
     out->stats.n_queries = nq;
+    return TS_OK;
+}
+
+// (memory may also run short after the arena: for the query copy, a sort's or a scan's buffers, the
+// rows. What was enqueued has ended by then, and the arena is back in the pool.)
+ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_params *qp,
+                        cudaStream_t s, SearchOut *out, bool *done)
+{
+    const ts_status st = one_go_steps(ix, q, qp, s, out, done);
+    if (st != TS_ERR_OOM) return st;
+    free_rows(out, s);
+    out->count = 0;
+    out->stats = ts_search_stats{};
+    out->stats.n_queries = q->n;
+    *done = false;
     return TS_OK;
 }
 
