@@ -545,9 +545,15 @@ constexpr size_t INDEX_KEEP = 512ull << 20;
 void destroy_index(Index *ix)
 {
     if (!ix) return;
+    // On the index's own device, whichever the caller's is: freeing memory of a pool waits for
+    // nothing, so whatever still reads the arrays has to have ended.
+    int dev = -1;
+    cudaGetDevice(&dev);
+    if (dev != ix->device) cudaSetDevice(ix->device);
     cudaDeviceSynchronize();
     for (void *p : ix->allocs) cudaFree(p);
     if (ix->bytes > INDEX_KEEP) pool_trim(INDEX_KEEP);
+    if (dev >= 0 && dev != ix->device) cudaSetDevice(dev);
     ix->magic = 0;
     delete ix;
 }
