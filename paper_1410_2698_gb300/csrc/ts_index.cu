@@ -539,7 +539,9 @@ ts_status build_grid(Ctx &c, Index *ix, const uint32_t *cell_in)
 
 }  // namespace
 
-// An index larger than this leaves no more than this in the pool.
+// What the freed indexes of a device may leave in the pool, all together: an index built in place of
+// another of up to this size finds its memory mapped (1M segments, built, searched once and freed:
+// 22 cudaMalloc and cudaFree took 1.6 of 3.5 ms).
 constexpr size_t INDEX_KEEP = 512ull << 20;
 
 void destroy_index(Index *ix)
@@ -551,8 +553,7 @@ void destroy_index(Index *ix)
     cudaGetDevice(&dev);
     if (dev != ix->device) cudaSetDevice(ix->device);
     cudaDeviceSynchronize();
-    for (void *p : ix->allocs) cudaFree(p);
-    if (ix->bytes > INDEX_KEEP) pool_trim(INDEX_KEEP);
+    index_free(ix->allocs.data(), ix->allocs.size(), ix->bytes, INDEX_KEEP, ix->device);
     if (dev >= 0 && dev != ix->device) cudaSetDevice(dev);
     ix->magic = 0;
     delete ix;

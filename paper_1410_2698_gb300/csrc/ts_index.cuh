@@ -72,13 +72,10 @@ struct Index {
     ts_status alloc(T **p, size_t count)
     {
         size_t nb = sizeof(T) * (count ? count : 1);
-        // from the library's pool: 22 cudaMalloc and cudaFree took 1.6 of the 3.5 ms in which an
-        // index of 1M segments was built, searched once and freed (destroy_index hands the memory
-        // of a large one back to the device)
-        cudaError_t e = pool_malloc((void **)p, nb, stream);
+        cudaError_t e = index_malloc((void **)p, nb, stream, device);
         if (e != cudaSuccess) {
             *p = nullptr;
-            return cuda_status(e, "pool_malloc(index)");
+            return cuda_status(e, "index_malloc");
         }
         allocs.push_back((void *)*p);
         bytes += nb;

@@ -204,15 +204,19 @@ inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t
     } while (0)
 
 // Stream-ordered device buffer (cudaMallocAsync / cudaFreeAsync).
-// Stream-ordered allocation from the library's pool (freed blocks stay pooled); inside a stream
-// capture a graph memory node. Release with cudaFreeAsync.
-cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream);
+// Stream-ordered allocation from the library's pool of work buffers, or of the indexes' arrays
+// (freed blocks stay pooled); inside a stream capture a graph memory node. Release with
+// cudaFreeAsync.
+cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream, bool index = false);
 // Tests of what a search does short of memory: of this thread's calls of pool_malloc, `count` fail
 // after the next `after`.
 void fail_allocs(uint64_t after, uint64_t count);
-// Return the pool's unused memory of the current device, but for `keep` bytes, to the device
-// (synchronises it).
-void pool_trim(size_t keep = 0);
+// Return the pools' unused memory of the current device to the device (synchronises it).
+void pool_trim();
+// An index's arrays, on `device`, the current one: allocated one by one, freed together (`bytes` in
+// all) once nothing reads them. Freed indexes leave at most `keep` bytes in their pool.
+cudaError_t index_malloc(void **p, size_t nbytes, cudaStream_t stream, int device);
+void index_free(void *const *p, size_t n, size_t bytes, size_t keep, int device);
 
 struct DevBuf {
     void *p = nullptr;

@@ -53,37 +53,42 @@ void DevBuf::release()
     bytes = 0;
 }
 
-// The library's stream-ordered pool of a device: freed blocks stay in the pool (no release
-// threshold), so the work buffers of repeated searches are not mapped and unmapped every call.
-static cudaMemPool_t work_pool()
+// The library's stream-ordered pools of a device, one for work buffers and rows and one for the
+// indexes' arrays: freed blocks stay in the pool (no release threshold), so the work buffers of
+// repeated searches, and the arrays of indexes built one after another, are not mapped and
+// unmapped every call. (Two, so that what freed indexes leave can be bounded by itself.)
+static cudaMemPool_t device_pool(bool index)
 {
     static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
+    static cudaMemPool_t pools[64][2] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
     std::lock_guard<std::mutex> lk(mu);
-    if (!pools[dev]) {
+    cudaMemPool_t &pool = pools[dev][index ? 1 : 0];
+    if (!pool) {
         cudaMemPoolProps props;
         memset(&props, 0, sizeof(props));
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
         if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
             cudaGetLastError();
+            pool = nullptr;
             return nullptr;
         }
         uint64_t keep = ~0ull;
         cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        pools[dev] = pool;
     }
-    return pools[dev];
+    return pool;
 }
 
-void pool_trim(size_t keep)
+void pool_trim()
 {
-    cudaMemPool_t pool = work_pool();
-    if (pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(pool, keep);
+    cudaMemPool_t work = device_pool(false), index = device_pool(true);
+    if (cudaDeviceSynchronize() == cudaSuccess) {
+        if (work) cudaMemPoolTrimTo(work, 0);
+        if (index) cudaMemPoolTrimTo(index, 0);
+    }
     cudaGetLastError();
 }
 
@@ -96,7 +101,7 @@ void fail_allocs(uint64_t after, uint64_t count)
     g_fail_count = count;
 }
 
-cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream)
+cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream, bool index)
 {
     if (g_fail_count) {
         if (g_fail_after) {
@@ -109,9 +114,44 @@ cudaError_t pool_malloc(void **p, size_t nbytes, cudaStream_t stream)
     }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(stream, &cs);
-    cudaMemPool_t pool = cs == cudaStreamCaptureStatusNone ? work_pool() : nullptr;
+    cudaMemPool_t pool = cs == cudaStreamCaptureStatusNone ? device_pool(index) : nullptr;
     return pool ? cudaMallocFromPoolAsync(p, nbytes, pool, stream)
                 : cudaMallocAsync(p, nbytes, stream);
+}
+
+// Bytes of the indexes alive on a device, and the most that the pool holds for them. (Counted here:
+// the pool's own count of used memory leaves out what cudaFree gave back.)
+struct IndexBytes {
+    std::mutex mu;
+    uint64_t live = 0, held = 0;
+};
+static IndexBytes g_index_bytes[64];
+
+cudaError_t index_malloc(void **p, size_t nbytes, cudaStream_t stream, int device)
+{
+    const cudaError_t e = pool_malloc(p, nbytes, stream, true);
+    if (e == cudaSuccess && device >= 0 && device < 64) {
+        IndexBytes &b = g_index_bytes[device];
+        std::lock_guard<std::mutex> lk(b.mu);
+        b.live += nbytes;
+        b.held = std::max(b.held, b.live);
+    }
+    return e;
+}
+
+void index_free(void *const *p, size_t n, size_t bytes, size_t keep, int device)
+{
+    for (size_t k = 0; k < n; k++) cudaFree(p[k]);
+    if (device < 0 || device >= 64) return;
+    IndexBytes &b = g_index_bytes[device];
+    std::lock_guard<std::mutex> lk(b.mu);
+    b.live -= bytes;
+    if (b.held <= b.live + keep) return;
+    b.held = b.live + keep;
+    // (given back in whole blocks, and only what a wait has seen freed)
+    cudaMemPool_t pool = device_pool(true);
+    if (pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(pool, b.held);
+    cudaGetLastError();
 }
 
 ts_status DevBuf::alloc(size_t nbytes, cudaStream_t stream)

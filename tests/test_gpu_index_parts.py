@@ -65,3 +65,35 @@ def test_an_index_in_the_pool_is_given_back():
         torch.cuda.synchronize()
         used.append(torch.cuda.mem_get_info()[0])
     assert max(used[1:]) - min(used[1:]) < (1 << 20)
+
+
+def test_freed_indexes_leave_a_bound():
+    """What freed indexes leave in the pool is bounded for all together (512 MB, and a few blocks of
+    memory that the pool gives back whole), for many of less than that and for one of more."""
+    import torch
+    rng = np.random.default_rng(6)
+    db = random_segments(rng, 1000000, box=200.0, max_len=1.0)
+    idx = api.ts_build_index(db, kind="spatiotemporal")
+    size = idx.info()["device_bytes"]
+    idx.free()
+    torch.cuda.synchronize()
+    room = torch.cuda.mem_get_info()[0]
+    many = int(2e9 // size) + 1
+    assert size < (512 << 20)
+    held = [api.ts_build_index(db, kind="spatiotemporal") for _ in range(many)]
+    for idx in held:
+        idx.free()
+    torch.cuda.synchronize()
+    assert room - torch.cuda.mem_get_info()[0] < (640 << 20)
+    big = Segments.from_matrix(np.tile(db.as_matrix(), (6, 1)))
+    idx = api.ts_build_index(big, kind="spatiotemporal")
+    size = idx.info()["device_bytes"]
+    assert size > (700 << 20)
+    alive = torch.cuda.mem_get_info()[0]
+    idx.free()
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] - alive > size - (640 << 20)
+    idx = api.ts_build_index(db, kind="spatiotemporal")
+    q = db.take(np.arange(50))
+    assert api.ts_search(idx, q, 0.5, 0.0, 13.0).count >= 50
+    idx.free()
