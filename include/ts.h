@@ -236,8 +236,9 @@ typedef struct ts_batch_params {
     int32_t use_graph;      /* 1: capture the run in a CUDA graph once, then replay it */
     int32_t pair_blocks;    /* blocks of the persistent pair kernel (0 = all resident) */
     uint64_t scratch_rows;  /* hits the count pass keeps (32 B each) and places after the scan;
-                               a run with more hits sweeps its tiles a second time to write them
-                               (0 = max_rows) */
+                               a run with more hits sweeps the tiles of the others a second time
+                               to write them (0 = max_rows, and slots that warps take in advance:
+                               faster where hits are many) */
 } ts_batch_params;
 
 typedef struct ts_batch ts_batch;
@@ -421,6 +422,9 @@ ts_status ts_debug_inject_stall(uint64_t limit_ns);
  * calling thread's allocations from the library's pool, `count` fail as if out of memory after the
  * next `after` have been made (count = 0: none). No allocation is attempted for those. */
 ts_status ts_debug_fail_allocs(uint64_t after, uint64_t count);
+
+/* Whether the count pass of a plan's last run kept every hit (test of scratch_rows). */
+ts_status ts_debug_batch_swept_once(const ts_batch *b, int32_t *once);
 
 /* Library version string. */
 const char *ts_version(void);

@@ -119,6 +119,7 @@ SIGNATURES = {
     "ts_measure_alu_peaks": (_S, [ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double)]),
     "ts_eval_refined_estimates": (_S, [_P, ctypes.c_uint64, _P, _P, _P, _P]),
     "ts_debug_inject_stall": (_S, [ctypes.c_uint64]),
+    "ts_debug_batch_swept_once": (_S, [_P, ctypes.POINTER(ctypes.c_int32)]),
     "ts_debug_fail_allocs": (_S, [ctypes.c_uint64, ctypes.c_uint64]),
     "ts_search_points": (_S, [_P, _P, _P, _P, ctypes.c_uint64, ctypes.c_int32,
                               ctypes.POINTER(ts_query_params), _P, ctypes.POINTER(_P)]),

@@ -395,6 +395,17 @@ ts_status ts_batch_rows(const ts_batch *h, const uint32_t **q_idx, const uint32_
     return TS_OK;
 }
 
+ts_status ts_debug_batch_swept_once(const ts_batch *h, int32_t *once)
+{
+    const BatchPlan *p = reinterpret_cast<const BatchPlan *>(h);
+    if (!p || p->magic != MAGIC_BATCH || !once) {
+        set_error("ts_debug_batch_swept_once: invalid batch handle or NULL argument");
+        return TS_ERR_INVALID_ARG;
+    }
+    *once = p->h_out->stats[ST_LOST] == 0;
+    return clear_error(TS_OK);
+}
+
 ts_status ts_batch_copy_rows(const ts_batch *h, uint64_t first, uint64_t count, uint32_t *q_idx,
                              uint32_t *e_idx, double *t_in, double *t_out)
 {

@@ -141,7 +141,7 @@ void destroy_plan(BatchPlan *p)
 }
 
 ts_status create_plan(const Index *ix, const ts_batch_params *prm, cudaStream_t s, bool own_rows,
-                      BatchPlan **out)
+                      BatchPlan **out, bool exact_scratch)
 {
     *out = nullptr;
     if (!prm || prm->max_requests == 0 || prm->max_queries == 0 ||
@@ -172,9 +172,14 @@ ts_status create_plan(const Index *ix, const ts_batch_params *prm, cudaStream_t 
     k.rows = own_rows ? prm->max_rows : ~0ull;
     // hits the count pass keeps for placement after the scan; more hits than this make the
     // write pass sweep the tiles again
-    k.scratch = prm->scratch_rows ? prm->scratch_rows
-                : scratch_slots(own_rows ? prm->max_rows
-                                         : std::min<uint64_t>(4 * k.nq + (1ull << 20), SCRATCH_MAX));
+    uint64_t warps = 0;
+    TS_CHECK(pair_warps(k, &warps));
+    k.exact_parts = prm->scratch_rows && exact_scratch;
+    k.scratch = prm->scratch_rows
+                    ? prm->scratch_rows
+                    : scratch_slots(own_rows ? prm->max_rows
+                                             : std::min<uint64_t>(4 * k.nq + (1ull << 20), SCRATCH_MAX),
+                                    warps);
     if (k.scratch > 0xffffffffull) k.scratch = 0xffffffffull;  // (slots are numbered in 32 bits)
     Carver sz;
     layout(p.get(), sz);

@@ -72,8 +72,9 @@ struct RowBlock {
 
 void note_launches(unsigned long long n);
 
+// (exact_scratch: prm's scratch_rows is a caller's, as many hits are kept)
 ts_status create_plan(const Index *ix, const ts_batch_params *prm, cudaStream_t s, bool own_rows,
-                      BatchPlan **out);
+                      BatchPlan **out, bool exact_scratch = true);
 void destroy_plan(BatchPlan *p);
 ts_status plan_run(BatchPlan *p, uint32_t nreq, const ts_segments *qs, const ts_query_params *qps,
                    cudaStream_t s);

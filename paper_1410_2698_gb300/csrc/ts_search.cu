@@ -822,6 +822,7 @@ struct PairParams {
     uint64_t tcap;
     uint64_t rows_cap;  // write pass: rows beyond this capacity are not written (flagged)
     uint64_t scap;      // hits the count pass keeps for placement (0: none)
+    bool exact_parts;   // warps take as many slots as they have hits, none in advance
     uint32_t tile;      // records per tile
     uint32_t tile_inv;  // ceil(2^16 / chunks per tile): c * it >> 16 is chunk c's tile (c < 32)
     // > 0 (tests only): the first warp of block 0 waits this long on a barrier phase that never
@@ -887,7 +888,8 @@ __device__ __forceinline__ void pair_batch(WarpSmem &W, const PairParams &P, uin
             if (nh <= left) {
                 if (lane == 0) W.sc_at = sc_at + nh;
             } else if (room) {
-                const uint32_t had = W.sc_had, want = min(256u, max(32u, had / 2));
+                const uint32_t had = W.sc_had;
+                const uint32_t want = P.exact_parts ? nh - left : min(256u, max(32u, had / 2));
                 unsigned long long base = 0;
                 if (lane == 0) base = atomicAdd(&B.stats[ST_SCRATCH], (unsigned long long)want);
                 base = __shfl_sync(FULL, base, 0);
@@ -1441,6 +1443,7 @@ void fill_pair_params(PairParams &P, const Index *ix, const ReqDesc *reqs, const
     P.tcap = c.tiles;
     P.rows_cap = c.rows;
     P.scap = c.scratch;
+    P.exact_parts = c.exact_parts;
     P.tile = c.tile;
     P.tile_inv = (65536u + c.tile / PK_CH - 1) / (c.tile / PK_CH);
     P.stall_ns = 0;
@@ -1613,6 +1616,15 @@ ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const 
         TS_LAUNCH_PDL(k_hdr, dim3(1), dim3(1), 0, s,
                       c.groups, c.tiles, b);
     }
+    return TS_OK;
+}
+
+ts_status pair_warps(const PipeCaps &c, uint64_t *warps)
+{
+    int blocks = 0;
+    TS_CHECK(pair_grid(&blocks));
+    if (c.pair_blocks > 0 && c.pair_blocks < blocks) blocks = c.pair_blocks;
+    *warps = (uint64_t)blocks * PK_WARPS;
     return TS_OK;
 }
 
@@ -2081,8 +2093,10 @@ ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_par
     c.groups = c.units / GROUP + 2;
     c.tiles = group_tiles(ix) * c.groups + 65536;
     if (c.units > ONE_GO_UNITS || c.tiles > ONE_GO_TILES) return TS_OK;
+    uint64_t warps = 0;
+    TS_CHECK(pair_warps(c, &warps));
     c.scratch = scratch_slots(std::min<uint64_t>(std::max<uint64_t>(4 * nq + (1ull << 20), 512 * nq),
-                                                 SCRATCH_MAX));
+                                                 SCRATCH_MAX), warps);
     c.rows = std::min<uint64_t>(8 * nq + 64, ONE_GO_ROWS);
     PipeBufs b = PipeBufs{};
     ReqDesc *reqs = nullptr;
@@ -2230,8 +2244,10 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     b.tdesc = w.tdesc.as<uint4>();
     b.tile_hits = w.tiles.as<uint32_t>();
     // hits kept by the count pass and placed after the scan (a second sweep when they overflow)
+    uint64_t warps = 0;
+    TS_CHECK(pair_warps(c, &warps));
     c.scratch = scratch_slots(std::min<uint64_t>(std::max<uint64_t>(4 * nq + (1ull << 20), 512 * nq),
-                                                 SCRATCH_MAX));
+                                                 SCRATCH_MAX), warps);
     if (w.scratch.alloc(32 * c.scratch, s) != TS_OK) {  // (short of memory: sweep twice instead)
         c.scratch = std::min<uint64_t>(4 * nq + (1ull << 20), SCRATCH_MAX);
         TS_CHECK(w.scratch.alloc(32 * c.scratch, s));

@@ -96,14 +96,16 @@ struct PipeCaps {
     uint32_t tile = PK_TILE;  // records per tile (multiple of PK_CH)
     int pair_blocks = 0;      // pair kernel grid (0 = all resident blocks)
     uint64_t scratch = 0;     // hits the count pass keeps for placement (0: the write pass sweeps)
+    bool exact_parts = false; // the scratch is taken hit by hit: a caller's size keeps that many
     uint64_t stall_ns = 0;    // plain searches only, tests of the timeout path (inject_stall)
 };
 constexpr uint64_t SCRATCH_MAX = 1ull << 24;  // rows (32 B each)
-// Slots that keep n hits: the count pass's warps take their parts in advance, so some slots of each
-// stay empty (at most 32, or a third of what it has had, or 256).
-inline uint64_t scratch_slots(uint64_t n)
+// Slots that keep n hits of `warps` warps of the count pass, which take their parts in advance: a
+// warp's last part holds one hit at least and is at most 32 slots, or half of what the warp has
+// filled, and never more than 256.
+inline uint64_t scratch_slots(uint64_t n, uint64_t warps)
 {
-    return n + (n / 2 + 100000 < 700000 ? n / 2 + 100000 : 700000);
+    return n + (n / 2 + 31 * warps < 255 * warps ? n / 2 + 31 * warps : 255 * warps);
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -168,6 +170,7 @@ ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const 
                      cudaStream_t s);
 ts_status pipe_count(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, const PipeCaps &c,
                      cudaStream_t s);
+ts_status pair_warps(const PipeCaps &c, uint64_t *warps);  // of the count pass
 ts_status pipe_scan_rows(const PipeBufs &b, const PipeCaps &c, cudaStream_t s);
 // Tests of the timeout path: the count pass of the next plain search stalls one warp for ns
 // nanoseconds on a barrier phase that never completes, then takes the timeout path.

@@ -157,7 +157,7 @@ void count_done(Server *s, Slot &sl)
             grow = true;
         }
         BatchPlan *np = nullptr;
-        if (grow && create_plan(p->ix, &bp, nullptr, false, &np) == TS_OK) {
+        if (grow && create_plan(p->ix, &bp, nullptr, false, &np, s->prm.scratch_rows != 0) == TS_OK) {
             s->plan_bytes += np->dbytes;
             s->plan_bytes -= std::min(s->plan_bytes, (uint64_t)p->dbytes);
             destroy_plan(p);
@@ -463,7 +463,7 @@ ts_status server_create(const Index *ix, const ts_server_params *prm, Server **o
                           : std::max<uint64_t>(1ull << 20, s->budget / 8 / 32);
     for (Slot &sl : s->slots) {
         // the plans run up to the row scan; every batch's rows are allocated at its exact size
-        ts_status st = create_plan(ix, &bp, nullptr, false, &sl.plan);
+        ts_status st = create_plan(ix, &bp, nullptr, false, &sl.plan, prm->scratch_rows != 0);
         if (st == TS_OK) s->plan_bytes += sl.plan->dbytes;
         if (st == TS_OK) {
             cudaError_t e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
