@@ -1894,14 +1894,16 @@ uint64_t grid_runs(const Index *ix, double d)
     return runs;
 }
 
-// About the most tiles of a group: all entries without bins, those of the bins that a window as
-// long as the longest entry meets, twice over, with bins; a few runs of cells on the grid.
-uint64_t group_tiles(const Index *ix)
+// About the most tiles of a group: all entries without bins, with bins those of the bins that a query
+// of this window (negative: as long as the longest entry's) meets and a few more; a few runs of
+// cells on the grid.
+uint64_t group_tiles(const Index *ix, double window)
 {
     if (ix->kind == TS_INDEX_SPATIAL) return 64;
     double n = (double)ix->n;
     if (ix->kind != TS_INDEX_BRUTE && ix->b > 0.0)
-        n = std::min(n, 2.0 * (ceil(ix->max_dur / ix->b) + 4.0) * (n / ix->m));
+        n = std::min(n, (ceil((window < 0.0 ? ix->max_dur : window) / ix->b) +
+                         ceil(ix->max_dur / ix->b) + 8.0) * (n / ix->m));
     return (uint64_t)(n / PK_TILE) + GROUP + 2;
 }
 
@@ -2062,7 +2064,7 @@ ts_status alloc_rows(SearchOut *out, uint64_t n, cudaStream_t s, PipeBufs &b)
 // allocator, 12 pageable copies, four waits, 18 kernels before) 327 -> 207 us, of 10,000
 // against 1M on the grid 395 -> 245 us, with the binding and the copies of the rows.
 ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_params *qp,
-                       cudaStream_t s, SearchOut *out, bool *done)
+                       double window, cudaStream_t s, SearchOut *out, bool *done)
 {
     const uint64_t nq = q->n;
     const bool grid = ix->kind == TS_INDEX_SPATIAL;
@@ -2091,7 +2093,7 @@ ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_par
     c.nreq = 1;
     c.units = grid ? nq * grid_runs(ix, qp->d) + 1024 : nq;
     c.groups = c.units / GROUP + 2;
-    c.tiles = group_tiles(ix) * c.groups + 65536;
+    c.tiles = group_tiles(ix, window) * c.groups + 65536;
     if (c.units > ONE_GO_UNITS || c.tiles > ONE_GO_TILES) return TS_OK;
     uint64_t warps = 0;
     TS_CHECK(pair_warps(c, &warps));
@@ -2187,9 +2189,9 @@ ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_par
 // (memory may also run short after the arena: for the query copy, a sort's or a scan's buffers, the
 // rows. What was enqueued has ended by then, and the arena is back in the pool.)
 ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_params *qp,
-                        cudaStream_t s, SearchOut *out, bool *done)
+                        double window, cudaStream_t s, SearchOut *out, bool *done)
 {
-    const ts_status st = one_go_steps(ix, q, qp, s, out, done);
+    const ts_status st = one_go_steps(ix, q, qp, window, s, out, done);
     if (st != TS_ERR_OOM) return st;
     free_rows(out, s);
     out->count = 0;
@@ -2202,7 +2204,7 @@ ts_status search_one_go(const Index *ix, const ts_segments *q, const ts_query_pa
 }  // namespace
 
 ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_params *qp,
-                       cudaStream_t s, SearchOut *out)
+                       cudaStream_t s, SearchOut *out, double window)
 {
     TS_CHECK(check_query_params(qp));
     if (!q) {
@@ -2220,7 +2222,7 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     if (nq == 0) return TS_OK;
     if (nq <= ONE_GO_QUERIES) {
         bool done = false;
-        const ts_status got = search_one_go(ix, q, qp, s, out, &done);
+        const ts_status got = search_one_go(ix, q, qp, window, s, out, &done);
         if (done) return got;
     }
     DevBuf qcopy;
@@ -2501,7 +2503,9 @@ ts_status search_points(const Index *ix, const double *x, const double *y, const
     q.x1 = c + 4 * n; q.y1 = c + 5 * n; q.z1 = c + 6 * n; q.t1 = c + 7 * n;
     q.n = n;
     q.on_host = 0;
-    return search_plain(ix, &q, qp, s, out);
+    // (every point's window is the interval's part of the database's time)
+    const double window = std::min(qp->t_end, ix->tmax) - std::max(qp->t_start, ix->tmin);
+    return search_plain(ix, &q, qp, s, out, std::max(0.0, window));
 }
 
 ts_status schedule_only(const Index *ix, const ts_segments *q, const ts_query_params *qp,

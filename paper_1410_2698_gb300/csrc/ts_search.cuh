@@ -148,8 +148,9 @@ const char *last_error();
 unsigned long long launch_count();
 
 // Plain search (R = 1) with exact-size allocations; synchronises the stream.
+// (window: of the queries, as far as the caller knows it, for a guess of sizes; negative: unknown)
 ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_params *qp,
-                       cudaStream_t s, SearchOut *out);
+                       cudaStream_t s, SearchOut *out, double window = -1.0);
 ts_status measure_alu_peaks(double *fp32_tflops, double *fp64_tflops);
 ts_status eval_estimates(const double *x, uint64_t n, double *rcp_est, double *sqrt_est,
                          double *rcp_ref, double *sqrt_ref);

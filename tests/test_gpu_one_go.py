@@ -174,3 +174,25 @@ def test_rows_sorted_on_the_device(nq, box, kind):
         _lib.check(lib.ts_result_copy_sorted_to_host(res.handle, None, None, None,
                                                      only.ctypes.data, None))
         assert np.array_equal(only, rows["t_out"][order])
+
+
+@pytest.mark.parametrize("kind", ["temporal", "spatiotemporal"])
+def test_points_over_the_whole_interval(kind):
+    """3,000 fixed points meet all of the 2,000 bins: they take the kernels of 1,000 points and those of
+    a sort of more than one block, not a second search step by step."""
+    rng = np.random.default_rng(12)
+    db = random_segments(rng, 200000, box=300.0, t_range=(0.0, 1000.0), max_dur=0.4)
+    idx = api.ts_build_index(db, kind=kind, t_bins=2000)
+    took = []
+    for n in (1000, 3000):
+        p = rng.uniform(0.0, 300.0, (n, 3))
+        before = api.ts_kernel_launches()
+        res = api.ts_search_points(idx, p[:, 0], p[:, 1], p[:, 2], 1.0, -5.0, 2000.0)
+        took.append(api.ts_kernel_launches() - before)
+        m = np.column_stack([p, np.full(n, -5.0), p, np.full(n, 2000.0)])
+        ref = oracle.search(db, Segments.from_matrix(m), -5.0, 2000.0, 1.0)
+        got = res.to_host(sort=True)
+        assert ref["q_idx"].size > 0
+        for k in ("q_idx", "e_idx"):
+            assert np.array_equal(got[k], ref[k])
+    assert took[1] <= took[0] + 10, took
