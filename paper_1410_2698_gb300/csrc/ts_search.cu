@@ -404,12 +404,20 @@ __global__ void k_qprep(PrepParams P)
 // unit slots (query i owns slots quoff[i] .. quoff[i] + qnu[i] - 1, so the warp's slots are one
 // contiguous range), then run over the warp's slots 32 at a time, each lane finding the query of
 // its slot among the lanes' starts; the unit counts per request are summed in the warp.
+// all_or_none: more runs than the unit buffers hold leave no unit at all, and the kernels that
+// follow nothing to do (a search in one go whose guess was too small starts over with exact sizes;
+// what fits was sorted, swept and placed before: 60,000 queries of 20 cells on 100^3 cells
+// 3,007 -> 2,618 us, 2,000 698 -> 511).
 __global__ void k_grid_units(uint64_t nqcap, uint64_t ucap, KeyFmt kf, uint32_t g,
-                             const uint32_t *g_off, PipeBufs b)
+                             const uint32_t *g_off, bool all_or_none, PipeBufs b)
 {
     pdl_enter();
     const unsigned FULL = 0xffffffffu;
     const uint64_t nq = b.run ? min((uint64_t)b.run[0], nqcap) : nqcap;
+    if (all_or_none && b.quoff[nq] > ucap) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) b.hdr[HDR_NU] = 0;
+        return;
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0)
         b.hdr[HDR_NU] = (uint32_t)min((uint64_t)b.quoff[nq], ucap);  // unit slots of the runs
     const int lane = threadIdx.x & 31;
@@ -1586,12 +1594,12 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
 }
 
 ts_status pipe_grid_units(const Index *ix, uint64_t nq, const PipeBufs &b, const PipeCaps &c,
-                          cudaStream_t s)
+                          cudaStream_t s, bool all_or_none)
 {
     if (!nq) return TS_OK;
     const unsigned ublk = (unsigned)std::min<uint64_t>((nq + TPB - 1) / TPB, 152 * 16);
     TS_LAUNCH_PDL(k_grid_units, dim3(ublk), dim3(TPB), 0, s,
-                  nq, c.units, key_fmt(ix, c), ix->g, ix->g_off, b);
+                  nq, c.units, key_fmt(ix, c), ix->g, ix->g_off, all_or_none, b);
     return TS_OK;
 }
 
@@ -2136,7 +2144,7 @@ ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_par
     TS_CHECK(pipe_prepare(ix, nullptr, nq, reqs, 1, b, c, s));
     if (grid) {
         TS_CHECK(scan_u32(b.qnu, b.quoff, nq, b.status, s));
-        TS_CHECK(pipe_grid_units(ix, nq, b, c, s));
+        TS_CHECK(pipe_grid_units(ix, nq, b, c, s, true));
     }
     TS_CHECK(pipe_group(ix, reqs, 1, b, c, false, s));
     c.stall_ns = g_stall_ns.exchange(0);  // (a stall requested by a test of the timeout path)

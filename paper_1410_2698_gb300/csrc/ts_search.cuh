@@ -165,7 +165,7 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
                        const ReqDesc *reqs, uint32_t nreq, const PipeBufs &b, const PipeCaps &c,
                        cudaStream_t s);
 ts_status pipe_grid_units(const Index *ix, uint64_t nq, const PipeBufs &b, const PipeCaps &c,
-                          cudaStream_t s);
+                          cudaStream_t s, bool all_or_none = false);
 ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const PipeBufs &b,
                      const PipeCaps &c, bool host_tiles,
                      cudaStream_t s);
