@@ -258,9 +258,11 @@ __global__ void __launch_bounds__(TPB) k_axis_hist(const RecF *rec, uint64_t n, 
         if (h[i]) atomicAdd(&hist[i], h[i]);
 }
 
-// The share of the entries before every place (a warp per axis).
-__global__ void k_axis_rank(const uint32_t *hist, float *rank)
+// The share of the entries before every place (a warp per axis), and whether the order is that of x.
+__global__ void k_axis_rank(const uint32_t *hist, uint64_t n, float *rank)
 {
+    if (threadIdx.x == 0)
+        rank[3 * (AXIS_BINS + 1)] = n <= BY_X_ENTRIES * hist[3 * AXIS_BINS] ? 1.0f : 0.0f;
     const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
     constexpr int PER = AXIS_BINS / 32;
     uint32_t sum = 0;
@@ -329,13 +331,16 @@ __global__ void k_bins_init(uint32_t m, double tmin, double b, double *bin_start
     end_key[j] = dkey(part_bound(tmin, b, (int)j + 1));
 }
 
-// off[j] = first sorted entry with bin >= j (bin_of is non-decreasing)
-__global__ void k_bin_bounds(const uint32_t *bin_of, uint64_t n, uint32_t m, uint32_t *off)
+// off[j] = first sorted entry with bin >= j (bin_of is non-decreasing); *occupied: bins with entries
+__global__ void k_bin_bounds(const uint32_t *bin_of, uint64_t n, uint32_t m, uint32_t *off,
+                             uint32_t *occupied)
 {
-    uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t j = s < n ? bin_of[s] : 0u;
+    const uint32_t jp = s && s < n ? bin_of[s - 1] + 1 : 0u;
+    const int heads = __syncthreads_count(s < n && jp <= j);
+    if (threadIdx.x == 0 && heads) atomicAdd(occupied, (uint32_t)heads);
     if (s >= n) return;
-    uint32_t j = bin_of[s];
-    uint32_t jp = s ? bin_of[s - 1] + 1 : 0;
     for (uint32_t k = jp; k <= j; k++) off[k] = (uint32_t)s;
     if (s == n - 1)
         for (uint32_t k = j + 1; k <= m; k++) off[k] = (uint32_t)n;
@@ -732,27 +737,29 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     TS_LAUNCHED();
     keys.release();
     vals.release();
-    k_bin_bounds<<<nblocks(n), TPB, 0, s>>>(bin_of.as<uint32_t>(), n, ix->m, ix->bin_off);
+    DevBuf hist;  // entries by place (k_axis_hist), and the occupied bins
+    TS_CHECK(hist.alloc(sizeof(uint32_t) * (3 * AXIS_BINS + 1), s));
+    TS_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(uint32_t) * (3 * AXIS_BINS + 1), s));
+    k_bin_bounds<<<nblocks(n), TPB, 0, s>>>(bin_of.as<uint32_t>(), n, ix->m, ix->bin_off,
+                                            hist.as<uint32_t>() + 3 * AXIS_BINS);
     TS_LAUNCHED();
     k_bin_ends<<<1, 1024, 0, s>>>(end_key.as<unsigned long long>(), ix->m, ix->bin_end,
                                   ix->bin_pmax);
     TS_LAUNCHED();
 
     if (p->kind != TS_INDEX_SPATIAL) {
-        // bins ordered along the Morton curve inside (ranges over the start-time order cover
-        // whole bins): 4 bits an axis more than it takes to tell the entries of a mean bin apart
+        // bins ordered along the Morton curve inside, or by x (ranges over the start-time order
+        // cover whole bins): 4 bits an axis more than it takes to tell the entries of a mean bin apart
         const int per_bin = bits_for(n / ix->m);
-        DevBuf tkeys, hist;
-        TS_CHECK(hist.alloc(sizeof(uint32_t) * 3 * AXIS_BINS, s));
-        TS_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(uint32_t) * 3 * AXIS_BINS, s));
-        TS_CHECK(ix->alloc(&ix->axis_rank, 3 * (AXIS_BINS + 1)));
+        DevBuf tkeys;
+        TS_CHECK(ix->alloc(&ix->axis_rank, 3 * (AXIS_BINS + 1) + 1));
         TS_CHECK(ix->alloc(&ix->tid, n));
         const MortonMap mm =
             morton_map(ix, std::min(10, std::max(4, (per_bin + 2) / 3 + 4)));
         k_axis_hist<<<64, TPB, 0, s>>>(ix->rec, n, std::max<uint64_t>(1, n >> 17), mm,
                                        hist.as<uint32_t>());
         TS_LAUNCHED();
-        k_axis_rank<<<1, 96, 0, s>>>(hist.as<uint32_t>(), ix->axis_rank);
+        k_axis_rank<<<1, 96, 0, s>>>(hist.as<uint32_t>(), n, ix->axis_rank);
         TS_LAUNCHED();
         TS_CHECK(tkeys.alloc(sizeof(uint64_t) * n, s));
         k_tm_key<<<nblocks(n), TPB, 0, s>>>(ix->rec, bin_of.as<uint32_t>(), n, mm,
