@@ -331,7 +331,8 @@ __global__ void k_bins_init(uint32_t m, double tmin, double b, double *bin_start
     end_key[j] = dkey(part_bound(tmin, b, (int)j + 1));
 }
 
-// off[j] = first sorted entry with bin >= j (bin_of is non-decreasing); *occupied: bins with entries
+// off[j] = first sorted entry with bin >= j (bin_of is non-decreasing); *occupied (where asked for):
+// bins with entries
 __global__ void k_bin_bounds(const uint32_t *bin_of, uint64_t n, uint32_t m, uint32_t *off,
                              uint32_t *occupied)
 {
@@ -339,7 +340,7 @@ __global__ void k_bin_bounds(const uint32_t *bin_of, uint64_t n, uint32_t m, uin
     const uint32_t j = s < n ? bin_of[s] : 0u;
     const uint32_t jp = s && s < n ? bin_of[s - 1] + 1 : 0u;
     const int heads = __syncthreads_count(s < n && jp <= j);
-    if (threadIdx.x == 0 && heads) atomicAdd(occupied, (uint32_t)heads);
+    if (threadIdx.x == 0 && heads && occupied) atomicAdd(occupied, (uint32_t)heads);
     if (s >= n) return;
     for (uint32_t k = jp; k <= j; k++) off[k] = (uint32_t)s;
     if (s == n - 1)
@@ -738,10 +739,12 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     keys.release();
     vals.release();
     DevBuf hist;  // entries by place (k_axis_hist), and the occupied bins
-    TS_CHECK(hist.alloc(sizeof(uint32_t) * (3 * AXIS_BINS + 1), s));
-    TS_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(uint32_t) * (3 * AXIS_BINS + 1), s));
+    if (p->kind != TS_INDEX_SPATIAL) {
+        TS_CHECK(hist.alloc(sizeof(uint32_t) * (3 * AXIS_BINS + 1), s));
+        TS_CUDA(cudaMemsetAsync(hist.p, 0, sizeof(uint32_t) * (3 * AXIS_BINS + 1), s));
+    }
     k_bin_bounds<<<nblocks(n), TPB, 0, s>>>(bin_of.as<uint32_t>(), n, ix->m, ix->bin_off,
-                                            hist.as<uint32_t>() + 3 * AXIS_BINS);
+                                            hist.p ? hist.as<uint32_t>() + 3 * AXIS_BINS : nullptr);
     TS_LAUNCHED();
     k_bin_ends<<<1, 1024, 0, s>>>(end_key.as<unsigned long long>(), ix->m, ix->bin_end,
                                   ix->bin_pmax);
