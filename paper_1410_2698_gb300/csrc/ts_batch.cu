@@ -91,8 +91,6 @@ static void layout(BatchPlan *p, Carver &c)
     b.ustart = c.take<uint32_t>(k.nreq + 1);
     b.req_groups = c.take<uint32_t>(k.nreq);
     b.gstart = c.take<uint32_t>(k.nreq + 1);
-    b.g_first = c.take<uint32_t>(k.groups);
-    b.g_count = c.take<uint32_t>(k.groups);
     b.g_nseg = c.take<uint32_t>(k.groups);
     b.gmem = c.take<MemberRec>(GROUP * k.groups);
     b.ghdr = c.take<float4>(3 * k.groups);
@@ -321,11 +319,9 @@ static ts_status enqueue_run(BatchPlan *p, cudaStream_t s, bool write)
         TS_CHECK(pipe_grid_units(p->ix, k.nq, b, k, s));
     }
     TS_CHECK(pipe_group(p->ix, p->d_reqs, k.nreq, b, k, false, s));
-    TS_CHECK(pipe_count(p->ix, p->d_reqs, b, k, s));
+    TS_CHECK(pipe_count(p->ix, b, k, s));
     TS_CHECK(pipe_scan_rows(b, k, s));
-    if (write) {
-            TS_CHECK(pipe_write(p->ix, p->d_reqs, b, k, s));
-        }
+    if (write) TS_CHECK(pipe_write(p->ix, b, k, s));
     TS_LAUNCH_PDL(k_req_rows, dim3(1), dim3(256), 0, s,
                   p->d_run, k.nreq, k.tiles, b, p->dh_row0, p->dh_out);
     return TS_OK;
@@ -484,7 +480,7 @@ ts_status search_batch(const Index *ix, uint32_t nreq, const ts_segments *qs,
         p->b.out_tin = block->tin;
         p->b.out_tout = block->tout;
         p->caps.rows = total;
-        TS_CHECK(pipe_write(ix, p->d_reqs, p->b, p->caps, st));
+        TS_CHECK(pipe_write(ix, p->b, p->caps, st));
         TS_CUDA(cudaMemcpyAsync(&p->h_out->status, p->b.status, 4, cudaMemcpyDeviceToHost, st));
         TS_CUDA(cudaStreamSynchronize(st));
         status = p->h_out->status;

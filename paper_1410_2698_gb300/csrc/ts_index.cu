@@ -448,6 +448,8 @@ int bits_for(uint64_t maxval)
 struct Ctx {
     cudaStream_t s;
     DevBuf status;
+    DevBuf rec;  // FP32 prefilter records in start-time order
+    DevBuf tid;  // the bins' entries in their sweep order
     ts_status read_status()
     {
         uint32_t st = 0;
@@ -493,7 +495,7 @@ ts_status build_st_dim(Ctx &c, Index *ix, int dim, const uint32_t *part_in, cons
     DevBuf keys;
     TS_CHECK(keys.alloc(sizeof(uint32_t) * len, c.s));
     TS_CHECK(ix->alloc(&ix->st_ids[dim], len));
-    k_part_emit<<<nblocks(n), TPB, 0, c.s>>>(part_in, ix->orig, ix->tid, n, pos,
+    k_part_emit<<<nblocks(n), TPB, 0, c.s>>>(part_in, ix->orig, c.tid.as<uint32_t>(), n, pos,
                                              keys.as<uint32_t>(), ix->st_ids[dim]);
     TS_LAUNCHED();
     TS_CHECK(radix_sort_u32(keys.as<uint32_t>(), ix->st_ids[dim], len, bits_for((uint64_t)v - 1),
@@ -508,7 +510,8 @@ ts_status build_st_dim(Ctx &c, Index *ix, int dim, const uint32_t *part_in, cons
     TS_CHECK(ix->alloc(&ix->st_off[dim], nbins + 1));
     TS_CHECK(scan_u32(h.as<uint32_t>(), ix->st_off[dim], nbins, c.status.as<uint32_t>(), c.s));
     TS_CHECK(ix->alloc(&ix->st_rec[dim], (len + CHUNK - 1) / CHUNK));
-    k_gather_rec<<<nblocks(len), TPB, 0, c.s>>>(ix->st_ids[dim], len, ix->rec, ix->st_rec[dim]);
+    k_gather_rec<<<nblocks(len), TPB, 0, c.s>>>(ix->st_ids[dim], len, c.rec.as<RecF>(),
+                                                ix->st_rec[dim]);
     TS_LAUNCHED();
     TS_CHECK(build_boxes(c, ix, ix->st_rec[dim], len, &ix->st_box[dim]));
     ix->st_len[dim] = len;
@@ -534,7 +537,7 @@ ts_status build_grid(Ctx &c, Index *ix, const uint32_t *cell_in)
     TS_CHECK(ix->alloc(&ix->g_off, ncell + 1));
     TS_CHECK(scan_u32(h.as<uint32_t>(), ix->g_off, ncell, c.status.as<uint32_t>(), c.s));
     TS_CHECK(ix->alloc(&ix->ga_rec, (n + CHUNK - 1) / CHUNK));
-    k_gather_rec<<<nblocks(n), TPB, 0, c.s>>>(ix->ga, n, ix->rec, ix->ga_rec);
+    k_gather_rec<<<nblocks(n), TPB, 0, c.s>>>(ix->ga, n, c.rec.as<RecF>(), ix->ga_rec);
     TS_LAUNCHED();
     // chunk bounding records: the cell sort is stable over the start-time order, so a chunk of
     // a cell spans a short stretch of time and a query's window skips most of a cell's chunks
@@ -730,10 +733,10 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
     TS_CHECK(radix_sort_u64(keys.as<uint64_t>(), vals.as<uint32_t>(), n, 64, s, nullptr, false,
                             hred[R_VARY]));
     TS_CHECK(ix->alloc(&ix->seg, n));
-    TS_CHECK(ix->alloc(&ix->rec, n));
+    TS_CHECK(c.rec.alloc(sizeof(RecF) * n, s));
     TS_CHECK(ix->alloc(&ix->orig, n));
     k_gather<<<nblocks(n), TPB, 0, s>>>(in, n, vals.as<uint32_t>(), bin_in.as<uint32_t>(), ix->seg,
-                                        ix->rec, ix->orig, bin_of.as<uint32_t>(),
+                                        c.rec.as<RecF>(), ix->orig, bin_of.as<uint32_t>(),
                                         end_key.as<unsigned long long>());
     TS_LAUNCHED();
     keys.release();
@@ -756,22 +759,23 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         const int per_bin = bits_for(n / ix->m);
         DevBuf tkeys;
         TS_CHECK(ix->alloc(&ix->axis_rank, 3 * (AXIS_BINS + 1) + 1));
-        TS_CHECK(ix->alloc(&ix->tid, n));
+        TS_CHECK(c.tid.alloc(sizeof(uint32_t) * n, s));
         const MortonMap mm =
             morton_map(ix, std::min(10, std::max(4, (per_bin + 2) / 3 + 4)));
-        k_axis_hist<<<64, TPB, 0, s>>>(ix->rec, n, std::max<uint64_t>(1, n >> 17), mm,
+        k_axis_hist<<<64, TPB, 0, s>>>(c.rec.as<RecF>(), n, std::max<uint64_t>(1, n >> 17), mm,
                                        hist.as<uint32_t>());
         TS_LAUNCHED();
         k_axis_rank<<<1, 96, 0, s>>>(hist.as<uint32_t>(), n, ix->axis_rank);
         TS_LAUNCHED();
         TS_CHECK(tkeys.alloc(sizeof(uint64_t) * n, s));
-        k_tm_key<<<nblocks(n), TPB, 0, s>>>(ix->rec, bin_of.as<uint32_t>(), n, mm,
-                                            tkeys.as<uint64_t>(), ix->tid);
+        k_tm_key<<<nblocks(n), TPB, 0, s>>>(c.rec.as<RecF>(), bin_of.as<uint32_t>(), n, mm,
+                                            tkeys.as<uint64_t>(), c.tid.as<uint32_t>());
         TS_LAUNCHED();
-        TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), ix->tid, n,
+        TS_CHECK(radix_sort_u64(tkeys.as<uint64_t>(), c.tid.as<uint32_t>(), n,
                                 3 * mm.bits + bits_for((uint64_t)ix->m - 1), s, nullptr, false));
         TS_CHECK(ix->alloc(&ix->trec, (n + CHUNK - 1) / CHUNK));
-        k_gather_rec<<<nblocks(n), TPB, 0, s>>>(ix->tid, n, ix->rec, ix->trec);
+        k_gather_rec<<<nblocks(n), TPB, 0, s>>>(c.tid.as<uint32_t>(), n, c.rec.as<RecF>(),
+                                                ix->trec);
         TS_LAUNCHED();
         TS_CHECK(build_boxes(c, ix, ix->trec, n, &ix->tbox));
     }
@@ -781,8 +785,8 @@ ts_status build_index(const ts_segments *db, const ts_index_params *p, cudaStrea
         DevBuf cnt, pos;
         TS_CHECK(cnt.alloc(sizeof(uint32_t) * 3 * n, s));
         TS_CHECK(pos.alloc(sizeof(uint32_t) * 3 * (n + 1), s));
-        k_part_count<<<nblocks(n), TPB, 0, s>>>(part_in.as<uint32_t>(), ix->orig, ix->tid, n,
-                                                cnt.as<uint32_t>());
+        k_part_count<<<nblocks(n), TPB, 0, s>>>(part_in.as<uint32_t>(), ix->orig,
+                                                c.tid.as<uint32_t>(), n, cnt.as<uint32_t>());
         TS_LAUNCHED();
         uint32_t len[3];
         for (int d = 0; d < 3; d++) {

@@ -18,18 +18,17 @@ struct Index {
 
     // entries in start-time order (Sec. 4.2: D sorted by t_start and renumbered)
     SegD *seg = nullptr;     // exact FP64 data
-    RecF *rec = nullptr;     // FP32 prefilter records
     uint32_t *orig = nullptr;  // sorted position -> caller's index
 
     // extents (exact, from the ingest reductions)
     double tmin = 0, tmax = 0, max_dur = 0;
     double emin[3] = {0, 0, 0}, emax[3] = {0, 0, 0}, longest[3] = {0, 0, 0};
 
-    // the entries of every temporal bin once more, in Morton order inside the bin (the bins keep
-    // their ranges [B^first, B^last]): records, their start-time positions, and the bounding
-    // record of every aligned chunk of 64 (built for every kind whose ranges cover bins)
+    // the entries of every temporal bin in the order in which they are swept, near ones together
+    // (MortonMap; the bins keep their ranges [B^first, B^last]): prefilter records with their
+    // start-time positions, and the bounding record of every aligned chunk of 64 (built for every
+    // kind whose ranges cover bins)
     Chunk *trec = nullptr;
-    uint32_t *tid = nullptr;
     RecF *tbox = nullptr;
     float *axis_rank = nullptr;  // share of the entries before each of 256 places of each axis
 
@@ -39,7 +38,7 @@ struct Index {
     double *bin_start = nullptr, *bin_end = nullptr, *bin_pmax = nullptr;  // m each
     uint32_t *bin_off = nullptr;  // m + 1
 
-    // spatiotemporal subbins (Sec. 4.3): per dimension an id array in (subbin, bin, Morton) order
+    // spatiotemporal subbins (Sec. 4.3): per dimension an id array in (subbin, bin, sweep) order
     // (the export gives it in start-time order), a duplicated prefilter record per id, the
     // chunks' bounding records, and offsets off[j*m + i]
     uint32_t v[3] = {0, 0, 0};

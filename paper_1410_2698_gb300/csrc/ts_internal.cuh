@@ -56,15 +56,6 @@ struct __align__(32) QueryD {
 };
 static_assert(sizeof(QueryD) == 96, "QueryD is 96 bytes");
 
-// Query group: up to 32 consecutive (sorted) queries sharing one candidate array and range.
-struct Group {
-    uint32_t first;  // first sorted query
-    uint32_t count;  // 1..32
-    uint32_t sel;    // 0,1,2: X/Y/Z id array; 3: time-sorted entries; 4: grid lookup array
-    uint32_t lo, hi; // union of the members' candidate ranges [lo, hi)
-    uint32_t pad[3];
-};
-
 enum : uint32_t { SEL_X = 0, SEL_Y = 1, SEL_Z = 2, SEL_T = 3, SEL_GRID = 4 };
 
 // Status bits written by kernels (device status word).

@@ -156,7 +156,6 @@ struct PrepParams {
     // index
     uint64_t n;
     uint32_t m;
-    double tmin, tmax;
     const double *bin_start, *bin_pmax;
     const uint32_t *bin_off;
     float bin_iwf;      // ~ 1 / bin width (first guesses only)
@@ -168,7 +167,7 @@ struct PrepParams {
     uint32_t g;
     const double *g_bound[3];    // grid boundary tables (g + 1 each)
     float g_iwf[3];
-    double g_lo[3], g_w[3], longest[3];
+    double longest[3];
     uint32_t smem_bytes;  // > 0: the lookup tables are first copied into shared memory
     PipeBufs b;
 };
@@ -557,8 +556,6 @@ __global__ void k_groups(uint32_t nreq_cap, uint64_t gcap, uint32_t tile, const 
         end = min(first + GROUP, end);
         const uint32_t n = end - first;
         if (lane == 0) {
-            b.g_first[g] = first;
-            b.g_count[g] = n;
             const ReqDesc &R = reqs[r];
             b.ghdr[3 * g] =
                 make_float4(R.d_dn, R.d2u, __uint_as_float(R.q_first), __uint_as_float(n));
@@ -821,15 +818,13 @@ constexpr uint32_t TILE_REDO = 0x80000000u;
 
 struct PairParams {
     PipeBufs b;
-    const ReqDesc *reqs;
     const Chunk *rec[5];
     const RecF *box[5];  // bounding record per chunk
-    uint32_t len[5];     // records of the array
     const SegD *seg;
     const uint32_t *orig;
     uint64_t tcap;
     uint64_t rows_cap;  // write pass: rows beyond this capacity are not written (flagged)
-    uint64_t scap;      // hits the count pass keeps for placement (0: none)
+    uint64_t scap;      // slots for the hits that the count pass keeps for placement
     bool exact_parts;   // warps take as many slots as they have hits, none in advance
     uint32_t tile;      // records per tile
     uint32_t tile_inv;  // ceil(2^16 / chunks per tile): c * it >> 16 is chunk c's tile (c < 32)
@@ -886,53 +881,51 @@ __device__ __forceinline__ void pair_batch(WarpSmem &W, const PairParams &P, uin
     const uint32_t rank = (tile == wt_cur ? wt_cnt : 0u) + __popc(mine & lt_mask);
     if (PASS == PASS_COUNT) {
         if (h && (mine & lt_mask) == 0) atomicAdd(&B.tile_hits[tile], (uint32_t)__popc(mine));
-        if (P.scap) {
-            const uint32_t sc_at = W.sc_at, sc_end = W.sc_end;
-            const uint32_t nh = __popc(hm), left = sc_end - sc_at;
-            const uint32_t k = __popc(hm & lt_mask);  // rank among the batch's hits
-            uint32_t slot = sc_at + k;
-            bool kept = h && k < left;
-            __syncwarp();
-            if (nh <= left) {
-                if (lane == 0) W.sc_at = sc_at + nh;
-            } else if (room) {
-                const uint32_t had = W.sc_had;
-                const uint32_t want = P.exact_parts ? nh - left : min(256u, max(32u, had / 2));
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(&B.stats[ST_SCRATCH], (unsigned long long)want);
-                base = __shfl_sync(FULL, base, 0);
-                if (base + want <= P.scap) {
-                    if (k >= left) slot = (uint32_t)base + (k - left);
-                    kept = h;
-                    if (lane == 0) {
-                        W.sc_at = (uint32_t)base + (nh - left);
-                        W.sc_end = (uint32_t)base + want;
-                        W.sc_had = had + want;
-                    }
-                } else {
-                    // (the part's slots inside the scratch hold no hit)
-                    for (unsigned long long j = base + lane; j < P.scap; j += 32)
-                        B.s_tile[j] = 0xffffffffu;
-                    if (lane == 0) {
-                        B.stats[ST_LOST] = 1;
-                        W.sc_at = sc_end;
-                        W.room = 0;
-                    }
+        const uint32_t sc_at = W.sc_at, sc_end = W.sc_end;
+        const uint32_t nh = __popc(hm), left = sc_end - sc_at;
+        const uint32_t k = __popc(hm & lt_mask);  // rank among the batch's hits
+        uint32_t slot = sc_at + k;
+        bool kept = h && k < left;
+        __syncwarp();
+        if (nh <= left) {
+            if (lane == 0) W.sc_at = sc_at + nh;
+        } else if (room) {
+            const uint32_t had = W.sc_had;
+            const uint32_t want = P.exact_parts ? nh - left : min(256u, max(32u, had / 2));
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(&B.stats[ST_SCRATCH], (unsigned long long)want);
+            base = __shfl_sync(FULL, base, 0);
+            if (base + want <= P.scap) {
+                if (k >= left) slot = (uint32_t)base + (k - left);
+                kept = h;
+                if (lane == 0) {
+                    W.sc_at = (uint32_t)base + (nh - left);
+                    W.sc_end = (uint32_t)base + want;
+                    W.sc_had = had + want;
+                }
+            } else {
+                // (the part's slots inside the scratch hold no hit)
+                for (unsigned long long j = base + lane; j < P.scap; j += 32)
+                    B.s_tile[j] = 0xffffffffu;
+                if (lane == 0) {
+                    B.stats[ST_LOST] = 1;
+                    W.sc_at = sc_end;
+                    W.room = 0;
                 }
             }
-            if (kept) {
-                B.s_tile[slot] = tile;
-                B.s_rank[slot] = rank;
-                B.s_q[slot] = ql;
-                B.s_e[slot] = orig;
-                B.s_tin[slot] = tin;
-                B.s_tout[slot] = tout;
-            }
-            // a tile with a hit the scratch could not keep is swept again by the write pass
-            const unsigned lost = __ballot_sync(FULL, h && !kept);
-            if (h && !kept && (mine & lost & lt_mask) == 0)
-                atomicOr(&B.tile_hits[tile], TILE_REDO);
         }
+        if (kept) {
+            B.s_tile[slot] = tile;
+            B.s_rank[slot] = rank;
+            B.s_q[slot] = ql;
+            B.s_e[slot] = orig;
+            B.s_tin[slot] = tin;
+            B.s_tout[slot] = tout;
+        }
+        // a tile with a hit the scratch could not keep is swept again by the write pass
+        const unsigned lost = __ballot_sync(FULL, h && !kept);
+        if (h && !kept && (mine & lost & lt_mask) == 0)
+            atomicOr(&B.tile_hits[tile], TILE_REDO);
     } else if (h) {
         const uint64_t o = B.tile_off[tile] + rank;
         if (o < B.tile_off[tile + 1]) {
@@ -956,9 +949,9 @@ __device__ __forceinline__ void pair_batch(WarpSmem &W, const PairParams &P, uin
 }
 
 // Exact tests of the queued candidates, oldest first, 32 at a time; with `all` the rest too.
-// Returns how many stay queued (moved to the front). Not inlined, and called at one place, where
-// the sweep has little in registers (what lasts is in shared memory), so that those of the exact
-// test do not limit the warps that sweep.
+// Returns how many stay queued (moved to the front). Not inlined, and called only between two
+// chunks' survivors and at a warp's end, where the sweep has little in registers (what lasts is in
+// shared memory), so that those of the exact test do not limit the warps that sweep.
 template <int PASS>
 __device__ __noinline__ uint32_t pair_flush(uint32_t qn, bool all)
 {
@@ -994,10 +987,10 @@ __device__ __noinline__ uint32_t pair_flush(uint32_t qn, bool all)
 
 // Persistent pair kernel. Warps take listed tiles (a group of up to 32 query units and up to
 // `tile` consecutive entries of one sorted array, or a run of such tiles): the first by their
-// index in the grid, the rest from a device counter. Entry records stream through a ring of PK_STAGES shared-memory buffers
-// filled by 1-D bulk copies. The conservative FP32 filters pick the candidates of the exact test;
-// those wait in a per-warp queue that is carried across tiles and drained 32 at a time, so that
-// the exact tests run on full warps.
+// index in the grid, the rest from a device counter. Entry records stream through a ring of
+// PK_STAGES shared-memory buffers filled by 1-D bulk copies. The conservative FP32 filters pick the
+// candidates of the exact test; those wait in a per-warp queue that is carried across tiles and
+// drained 32 at a time, so that the exact tests run on full warps.
 //
 // Bound: instruction issue (63 % of the slots on 11 M exact tests among 2.3 G candidates; ALU 50 %,
 // shared-memory wavefronts 52 %, FP64 33 %). What it waits for is mostly the fixed latency of its
@@ -1029,7 +1022,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
         W.wt_cur = 0xffffffffu;
         W.wt_cnt = 0;
         W.sc_at = W.sc_end = W.sc_had = 0;
-        W.room = PASS == PASS_COUNT && P.scap != 0;
+        W.room = PASS == PASS_COUNT;
         for (int k = 0; k < PK_STAGES; k++) mbar_init(&W.bar[k], 1);
         mbar_init(&W.mbar, 1);
         mbar_init(&W.xbar, 1);
@@ -1041,15 +1034,13 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
     uint32_t parity = 0u, pending = 0u;
     constexpr uint32_t MEM = 1u << PK_STAGES;
     bool abort = false;
-    if (PASS == PASS_WRITE && !P.scap && blockIdx.x == 0 && threadIdx.x == 0)
-        B.stats[ST_WR0] = globaltimer_ns();
     if (P.stall_ns && blockIdx.x == 0 && wid == 0)
         abort = !mbar_wait_bounded(&W.xbar, 0u, P.stall_ns);  // (never arrived on: times out)
 
     const uint64_t all_tiles = (uint64_t)B.hdr[HDR_T_LO] | ((uint64_t)B.hdr[HDR_T_HI] << 32);
     uint32_t ntiles = B.counters[2];  // listed tiles
     if (all_tiles > P.tcap || all_tiles > PK_MAX_TILES) ntiles = 0;  // overflow already flagged
-    if (PASS == PASS_WRITE && P.scap && B.stats[ST_LOST] == 0)
+    if (PASS == PASS_WRITE && B.stats[ST_LOST] == 0)
         ntiles = 0;  // the count pass kept every hit: k_place writes the rows
     // (otherwise the write pass sweeps only the tiles whose hits were not all kept)
     if (PASS == PASS_WRITE && ntiles && B.tile_off[all_tiles] > P.rows_cap) {
@@ -1075,7 +1066,7 @@ __global__ void __launch_bounds__(PK_THREADS, PK_MIN_BLOCKS) k_pair(const PairPa
             bool redo = false;
             if (c < 32 && (D.y >> c) != 0u) {  // (a tile of the entry, or before its last one)
                 const uint32_t th = B.tile_hits[(D.x & PK_MAX_TILES) + lane];
-                redo = (th & ~TILE_REDO) != 0 && (!P.scap || (th & TILE_REDO));
+                redo = (th & TILE_REDO) != 0;
             }
             const uint32_t bits = tch < 32 ? (1u << tch) - 1u : FULL;
             D.y &= __reduce_or_sync(FULL, redo ? bits << c : 0u);
@@ -1428,24 +1419,19 @@ ts_status pair_grid(int *blocks)
     return TS_OK;
 }
 
-void fill_pair_params(PairParams &P, const Index *ix, const ReqDesc *reqs, const PipeBufs &b,
-                      const PipeCaps &c)
+void fill_pair_params(PairParams &P, const Index *ix, const PipeBufs &b, const PipeCaps &c)
 {
     P.b = b;
-    P.reqs = reqs;
     for (int k = 0; k < 3; k++) {
         P.rec[k] = ix->st_rec[k];
         P.box[k] = ix->st_box[k];
-        P.len[k] = (uint32_t)ix->st_len[k];
     }
     // ranges over the start-time order cover whole bins: they are swept in the copy in Morton
     // order inside every bin, chunk by chunk with the chunks' bounding records
     P.rec[SEL_T] = ix->trec;
     P.box[SEL_T] = ix->tbox;
-    P.len[SEL_T] = (uint32_t)ix->n;
     P.rec[SEL_GRID] = ix->ga_rec;
     P.box[SEL_GRID] = ix->gbox;
-    P.len[SEL_GRID] = (uint32_t)ix->g_len;
     P.seg = ix->seg;
     P.orig = ix->orig;
     P.tcap = c.tiles;
@@ -1553,8 +1539,6 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
     P.mm = morton_map(ix, P.kf.morton);
     P.n = ix->n;
     P.m = ix->m;
-    P.tmin = ix->tmin;
-    P.tmax = ix->tmax;
     P.bin_start = ix->bin_start;
     P.bin_pmax = ix->bin_pmax;
     P.bin_off = ix->bin_off;
@@ -1570,8 +1554,6 @@ ts_status pipe_prepare(const Index *ix, const double *const cols[8], uint64_t nq
         P.st_off[d] = ix->st_off[d];
         P.g_bound[d] = ix->g_bound[d];
         P.g_iwf[d] = ix->g_w[d] > 0.0 ? (float)(1.0 / ix->g_w[d]) : 0.0f;
-        P.g_lo[d] = ix->g_lo[d];
-        P.g_w[d] = ix->g_w[d];
         P.longest[d] = ix->longest[d];
     }
     P.g = ix->g;
@@ -1636,14 +1618,14 @@ ts_status pair_warps(const PipeCaps &c, uint64_t *warps)
     return TS_OK;
 }
 
-ts_status pipe_count(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, const PipeCaps &c,
+ts_status pipe_count(const Index *ix, const PipeBufs &b, const PipeCaps &c,
                      cudaStream_t s)
 {
     int blocks = 0;
     TS_CHECK(pair_grid(&blocks));
     if (c.pair_blocks > 0 && c.pair_blocks < blocks) blocks = c.pair_blocks;
     PairParams P;
-    fill_pair_params(P, ix, reqs, b, c);
+    fill_pair_params(P, ix, b, c);
     P.stall_ns = c.stall_ns;
     if (c.tiles) {
         ArrayPtrs<const RecF> box;
@@ -1665,19 +1647,16 @@ ts_status pipe_scan_rows(const PipeBufs &b, const PipeCaps &c, cudaStream_t s)
     return scan_u32_to_u64(b.tile_hits, b.tile_off, c.tiles, s, b.hdr + HDR_T_LO, ~TILE_REDO);
 }
 
-ts_status pipe_write(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, const PipeCaps &c,
-                     cudaStream_t s)
+ts_status pipe_write(const Index *ix, const PipeBufs &b, const PipeCaps &c, cudaStream_t s)
 {
     int blocks = 0;
     TS_CHECK(pair_grid(&blocks));
     if (c.pair_blocks > 0 && c.pair_blocks < blocks) blocks = c.pair_blocks;
     PairParams P;
-    fill_pair_params(P, ix, reqs, b, c);
+    fill_pair_params(P, ix, b, c);
     if (c.tiles) {
-        if (c.scratch) {
-            TS_LAUNCH_PDL(k_place, dim3(152 * 32), dim3(TPB), 0, s,
-                          b, c.scratch, c.tiles, c.rows);
-        }
+        TS_LAUNCH_PDL(k_place, dim3(152 * 32), dim3(TPB), 0, s,
+                      b, c.scratch, c.tiles, c.rows);
         TS_LAUNCH_PDL(k_pair<PASS_WRITE>, dim3(blocks), dim3(PK_THREADS),
                       PAIR_SMEM, s, P);
     }
@@ -1825,16 +1804,14 @@ ts_status plain_prepare(const Index *ix, const double *const cols[8], uint64_t n
     c.units = units;
     if (!group) return TS_OK;
     c.groups = (units + GROUP - 1) / GROUP + 1;
-    TS_CHECK(w.groups.alloc(sizeof(uint32_t) * 3 * c.groups, s));
+    TS_CHECK(w.groups.alloc(sizeof(uint32_t) * c.groups, s));
     TS_CHECK(w.gmem.alloc((sizeof(MemberRec) * GROUP + 3 * sizeof(float4)) * c.groups, s));
     b.gmem = w.gmem.as<MemberRec>();
     b.ghdr = reinterpret_cast<float4 *>(b.gmem + GROUP * c.groups);
     TS_CHECK(w.segs.alloc(sizeof(uint32_t) * 4 * GROUP * c.groups, s));
     TS_CHECK(w.ntiles.alloc(sizeof(uint32_t) * c.groups, s));
     TS_CHECK(w.tile_base.alloc(sizeof(uint64_t) * (c.groups + 1), s));
-    b.g_first = w.groups.as<uint32_t>();
-    b.g_count = b.g_first + c.groups;
-    b.g_nseg = b.g_count + c.groups;
+    b.g_nseg = w.groups.as<uint32_t>();
     b.seg_lo = w.segs.as<uint32_t>();
     b.seg_hi = b.seg_lo + GROUP * c.groups;
     b.seg_sel = b.seg_hi + GROUP * c.groups;
@@ -1884,7 +1861,7 @@ namespace {
 
 constexpr uint64_t ONE_GO_QUERIES = 1ull << 16;  // above, the kernels dwarf the waits
 constexpr uint64_t ONE_GO_ROWS = 1ull << 16;     // rows a result may have room for unasked
-constexpr uint64_t ONE_GO_UNITS = 1ull << 22;    // (2 KB of work buffers each 32)
+constexpr uint64_t ONE_GO_UNITS = 1ull << 22;    // (3 KB of work buffers each 32)
 constexpr uint64_t ONE_GO_TILES = 1ull << 24;    // (28 B of work buffers each)
 constexpr uint64_t STAGE_QUERIES = 1024;         // host queries read in place from pinned memory
 
@@ -2019,8 +1996,6 @@ void plain_layout(Carver &k, const PipeCaps &c, bool grid, PipeBufs &b, ReqDesc 
     b.u_sel = k.take<uint32_t>(c.units);
     b.keys = k.take<uint64_t>(c.units);
     b.vals = k.take<uint32_t>(c.units);
-    b.g_first = k.take<uint32_t>(c.groups);
-    b.g_count = k.take<uint32_t>(c.groups);
     b.g_nseg = k.take<uint32_t>(c.groups);
     b.gmem = k.take<MemberRec>(GROUP * c.groups);
     b.ghdr = k.take<float4>(3 * c.groups);
@@ -2148,9 +2123,9 @@ ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_par
     }
     TS_CHECK(pipe_group(ix, reqs, 1, b, c, false, s));
     c.stall_ns = g_stall_ns.exchange(0);  // (a stall requested by a test of the timeout path)
-    TS_CHECK(pipe_count(ix, reqs, b, c, s));
+    TS_CHECK(pipe_count(ix, b, c, s));
     TS_CHECK(pipe_scan_rows(b, c, s));
-    TS_CHECK(pipe_write(ix, reqs, b, c, s));
+    TS_CHECK(pipe_write(ix, b, c, s));
     TS_LAUNCH_PDL(k_plain_out, dim3(1), dim3(32), 0, s, nq, c.tiles, b, dout);
     TS_CUDA(cudaStreamSynchronize(s));
     slot.is_busy = false;
@@ -2184,7 +2159,7 @@ ts_status one_go_steps(const Index *ix, const ts_segments *q, const ts_query_par
     c.stall_ns = 0;
     slot.is_busy = true;
     TS_CUDA(cudaMemsetAsync(b.status, 0, sizeof(uint32_t), s));  // (the rows' overflow)
-    TS_CHECK(pipe_write(ix, reqs, b, c, s));
+    TS_CHECK(pipe_write(ix, b, c, s));
     TS_LAUNCH_PDL(k_plain_out, dim3(1), dim3(32), 0, s, nq, c.tiles, b, dout);
     TS_CUDA(cudaStreamSynchronize(s));
     slot.is_busy = false;
@@ -2271,7 +2246,7 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     b.tile_off = w.tile_off.as<uint64_t>();
 
     c.stall_ns = g_stall_ns.exchange(0);  // (a stall requested by a test of the timeout path)
-    TS_CHECK(pipe_count(ix, w.reqdesc.as<ReqDesc>(), b, c, s));
+    TS_CHECK(pipe_count(ix, b, c, s));
     TS_CHECK(pipe_scan_rows(b, c, s));
     uint64_t total = 0;
     TS_CUDA(cudaMemcpyAsync(&total, b.tile_off + c.tiles, 8, cudaMemcpyDeviceToHost, s));
@@ -2299,7 +2274,7 @@ ts_status search_plain(const Index *ix, const ts_segments *q, const ts_query_par
     b.out_tin = out->tin;
     b.out_tout = out->tout;
     c.rows = total;
-    TS_CHECK(pipe_write(ix, w.reqdesc.as<ReqDesc>(), b, c, s));
+    TS_CHECK(pipe_write(ix, b, c, s));
     TS_CHECK(copy_stats(b, s, &out->stats, &st));
     return read_dev_status(st);
 }

@@ -65,7 +65,7 @@ struct PipeBufs {
     // per request
     uint32_t *req_units, *ustart, *req_groups, *gstart;  // R, R+1, R, R+1
     // groups
-    uint32_t *g_first, *g_count, *g_nseg;
+    uint32_t *g_nseg;
     MemberRec *gmem;      // GROUP per group, in the group's (array, start) order
     // per group, three: its request's d_dn, d2u, q_first (bits), members (bits); the lower and
     // the upper bounds of its members' expanded boxes (the windows' in .w)
@@ -95,7 +95,7 @@ struct PipeCaps {
     uint32_t nreq = 1;
     uint32_t tile = PK_TILE;  // records per tile (multiple of PK_CH)
     int pair_blocks = 0;      // pair kernel grid (0 = all resident blocks)
-    uint64_t scratch = 0;     // hits the count pass keeps for placement (0: the write pass sweeps)
+    uint64_t scratch = 0;     // slots for the hits that the count pass keeps for placement (> 0)
     bool exact_parts = false; // the scratch is taken hit by hit: a caller's size keeps that many
     uint64_t stall_ns = 0;    // plain searches only, tests of the timeout path (inject_stall)
 };
@@ -169,14 +169,14 @@ ts_status pipe_grid_units(const Index *ix, uint64_t nq, const PipeBufs &b, const
 ts_status pipe_group(const Index *ix, const ReqDesc *reqs, uint32_t nreq, const PipeBufs &b,
                      const PipeCaps &c, bool host_tiles,
                      cudaStream_t s);
-ts_status pipe_count(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, const PipeCaps &c,
+ts_status pipe_count(const Index *ix, const PipeBufs &b, const PipeCaps &c,
                      cudaStream_t s);
 ts_status pair_warps(const PipeCaps &c, uint64_t *warps);  // of the count pass
 ts_status pipe_scan_rows(const PipeBufs &b, const PipeCaps &c, cudaStream_t s);
 // Tests of the timeout path: the count pass of the next plain search stalls one warp for ns
 // nanoseconds on a barrier phase that never completes, then takes the timeout path.
 void inject_stall(uint64_t ns);
-ts_status pipe_write(const Index *ix, const ReqDesc *reqs, const PipeBufs &b, const PipeCaps &c,
+ts_status pipe_write(const Index *ix, const PipeBufs &b, const PipeCaps &c,
                      cudaStream_t s);
 // Layout of a unit's sort key: request | array (sel_bits) | top lo_bits bits of the range start |
 // Morton code of the query (morton bits per axis).

@@ -244,7 +244,7 @@ void try_admit(Server *s, Slot &sl)
         p->b.out_tin = block->tin;
         p->b.out_tout = block->tout;
         p->caps.rows = sl.rows;
-        st = pipe_write(p->ix, p->d_reqs, p->b, p->caps, p->stream);
+        st = pipe_write(p->ix, p->b, p->caps, p->stream);
     }
     if (st == TS_OK) {
         cudaError_t e = cudaMemcpyAsync(&p->h_out->status, p->b.status, 4,
