@@ -14,6 +14,7 @@ cores, on a bounded sample of the same workload.
 from __future__ import annotations
 
 import argparse
+import gc
 import hashlib
 import json
 import math
@@ -296,9 +297,11 @@ def _timed(args, stream, flush, step, steps=None):
     """Time `steps` calls of step() with CUDA events on the bench stream; the L2 is flushed (a
     256 MB write, finished before the step starts) before every step, outside the events. A step
     that runs on other streams synchronises with the host before it returns, so the events
-    bracket all of its work."""
+    bracket all of its work. The interpreter collects its garbage before or after, not between (a
+    full collection in the middle of a step made 1.5 ms of 0.3)."""
     import torch
     ms = []
+    gc.disable()
     for _ in range(args.steps if steps is None else steps):
         flush.zero_()
         a = torch.cuda.Event(enable_timing=True)
@@ -309,6 +312,7 @@ def _timed(args, stream, flush, step, steps=None):
         b.record(stream)
         b.synchronize()
         ms.append(a.elapsed_time(b))
+    gc.enable()
     return ms
 
 
