@@ -42,16 +42,16 @@ INTERVAL_FLOPS = 10  # FP64 flops per hit for the roots (sqrt, 2 div, clamps; sq
 # dram__bytes_write.sum; the gathered FP64 records and the kept hits). The merger-like workload at
 # a tenth of the particles (merger-like-2m) stands in for the full one, whose launches are too
 # large to capture: the per-unit counts are those of the same kernel at the same hit ratio.
-_MERGER_PROFILE = {"fp64_inst_per_exact": 15.74, "warp_inst_per_test": 0.4728,
-                   "dram_bytes_per_exact": 64.63, "hit_ratio": 0.8697,
+_MERGER_PROFILE = {"fp64_inst_per_exact": 15.74, "warp_inst_per_test": 0.4735,
+                   "dram_bytes_per_exact": 65.75, "hit_ratio": 0.8697,
                    "capture": "profiles/k_pair_merger-like-2m_count-pass.md",
-                   "sources": "e452e00c9567bcdf"}
+                   "sources": "fb7fb544bc31b608"}
 # the Random-walk 1M workload (filter-bound: the issue slots bind); its DRAM bytes are mostly the
 # records the sweep streams, scaled here by the exact tests of the same workload
-_RW1M_PROFILE = {"fp64_inst_per_exact": 5.67, "warp_inst_per_test": 0.6133,
-                 "dram_bytes_per_exact": 478.4, "hit_ratio": 0.348,
+_RW1M_PROFILE = {"fp64_inst_per_exact": 5.67, "warp_inst_per_test": 0.5189,
+                 "dram_bytes_per_exact": 471.7, "hit_ratio": 0.348,
                  "capture": "profiles/k_pair_random-walk-1m_count-pass.md",
-                 "sources": "e452e00c9567bcdf"}
+                 "sources": "fb7fb544bc31b608"}
 PAIR_PROFILE = {"merger-like-20m": _MERGER_PROFILE, "merger-like-2m": _MERGER_PROFILE,
                 "random-walk-1m": _RW1M_PROFILE}
 PAIR_SOURCES = ("ts_search.cuh", "ts_internal.cuh", "ts_device.cuh")
